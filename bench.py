@@ -7,8 +7,10 @@ One step = one batch of ``--samples`` (default 200) samples drawn with every
 hot-path stage on the GPU: per-chain planning, Gray decode / re-seed, the
 incremental column-sum walk, the per-addend products, the fused Laplace
 minors, compensated accumulation and the weighted draw.  The headline runs
-the FP64 form (``--mode fp64``: column sums, products and weights in double
-precision, double-double partial sums); the MIXED form is reported beside it.
+the FP64 form (``--mode fp64``: exact 63-bit column sums and 62-bit products on
+the integer pipes, whose errors are below plain double arithmetic's, weights
+in double precision, double-double partial sums); the MIXED form is reported
+beside it.
 
   value     samples/s with U resident on the device (bs_sample_dev), CUDA
             events around every step, L2 flushed (256 MiB write) between steps
@@ -18,8 +20,10 @@ precision, double-double partial sums); the MIXED form is reported beside it.
   roofline  the fused-minors walk kernel of the run's precision: algorithmic
             flops (per-addend count 22K - 22, K columns) / summed kernel time
             (CUDA events on the launching stream, over --profile-steps steps
-            of the same seeds) vs 2 x the FMA rate of that pipe measured on
-            this GPU
+            of the same seeds) vs the rate of the pipe that bounds it,
+            measured on this GPU: FP32, 2 x the FMA rate; FP64, the rate of
+            32 x 32 -> 64 bit integer products, at the algorithm's 22 flops
+            per 36 of them (12 per complex product, 3 K - 3 complex products)
   cpu_baseline  the oracle (double-double C, minors computed separately, one
             process per host core) on a bounded prefix of one chain per core,
             scaled to samples/s by its own operation count; the one-core
@@ -323,8 +327,9 @@ def aggregate_rate(world, units_per_rank, seconds):
 # Arithmetic of each form (the headline's dtype and the side forms').
 DTYPES = {"fp64": "f64", "mixed": "f32", "df": "f32x2"}
 DTYPE_DETAIL = {
-    "fp64": ("f64 column sums, products and weights; per-lane double runs folded into double-double, "
-             "double-double task partials (Sum2 reduce)"),
+    "fp64": ("f64 in and out; exact 63-bit fixed-point column sums and products of normalised 62-bit mantissas on "
+             "the integer pipes (errors against the exact value below those of f64 products, "
+             "tests/test_gpu_fixed_point.py), f64 weights and runs, double-double task partials (Sum2 reduce)"),
     "mixed": ("f32 column sums and products where the MIXED rule predicts an error below 1e-6 prod ||a_j|| "
               "(column sums re-seeded every 2^8 steps where only their drift would exceed it; the rule is "
               "oracle-checked in tests/test_gpu_widths.py), double-float otherwise; float-float runs folded into "
@@ -342,11 +347,16 @@ DTYPE_DETAIL = {
 # and spill from it at 200: FP64 0.69 MB at 8 chains, 1.36 MB at 32, 80.1 MB
 # at 200), so only a capture of the full 200-chain launch is used; None where
 # there is none, or where the kernel changed since the capture.
-TRAFFIC_K30 = [{"bytes": 80.08e6, "chains": 200}, None, None]
-# The bounding pipe's busy fraction in the same captures
-# (sm__pipe_fp64_cycles_active / sm__pipe_fma_cycles_active, pct of peak
-# sustained active): FP64 pipe for the FP64 kernel, FMA pipe for the others.
-PIPE_K30 = [{"pipe": "fp64", "active": 0.928}, {"pipe": "fma", "active": 0.709}, {"pipe": "fma", "active": 0.788}]
+TRAFFIC_K30 = [None, None, None]
+# The bounding pipe's busy fraction under ncu (pct of peak sustained active):
+# the FMA-heavy pipe (integer products) on a 27 x 28 minors launch for the FP64
+# kernel, the FMA pipe on the k = 30 launch for the others.
+PIPE_K30 = [{"pipe": "fmaheavy", "active": 0.67}, {"pipe": "fma", "active": 0.709}, {"pipe": "fma", "active": 0.788}]
+# Flops of the algorithmic counts per 32 x 32 -> 64 bit product of the FP64
+# kernels: minors 22 K - 22 flops and 3 K - 3 complex products of 12, permanents
+# 8 K - 2 flops and K - 1 complex products.
+FLOPS_PER_WIDE = {"minors": 22.0 / 36.0, "perm": 8.0 / 12.0}
+
 
 def run_mine(args):
     import numpy as np
@@ -378,6 +388,7 @@ def run_mine(args):
     torch.cuda.set_stream(stream)
     ctx.set_stream(stream)
     fp64_rate, fp32_rate = ctx.measure_fma_rates()
+    wide_rate = ctx.measure_wide_rate()
     u_dev = torch.from_numpy(u).to("cuda")
     S_ = args.samples
     out_dev = torch.zeros((S_, M_MODES), dtype=torch.int32, device="cuda")
@@ -442,7 +453,7 @@ def run_mine(args):
     fl = st["addend_flops"][p]
     # (the double-float form's algorithmic flops are FP64-equivalent ones,
     # set against the FP64 pipe's peak: its fraction exceeds 1 by design)
-    peak = 2.0 * (fp32_rate if p == 1 else fp64_rate) / 1e12
+    peak = (FLOPS_PER_WIDE["minors"] * wide_rate, 2.0 * fp32_rate, 2.0 * fp64_rate)[p] / 1e12
     achieved = fl / walk_s / 1e12 if walk_s > 0 else 0.0
     # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the k = 30
     # fused-minor launch, from an ncu capture of that launch with the same
@@ -451,22 +462,26 @@ def run_mine(args):
     # compute-bound; the figure shows that they re-read nothing.
     cap = TRAFFIC_K30[p]
     traffic = cap["bytes"] if cap and cap["chains"] == S_ else None
-    # nominal peak from unit counts and clocks: FMA lanes per SM per clock
-    # (128 FP32, 2 FP64 on this part) x SMs x maximum SM clock x 2 flops
+    # nominal peak from unit counts and clocks: lanes per SM per clock (32
+    # wide integer products, 128 FP32 FMAs, 2 FP64 FMAs on this part) x SMs x
+    # maximum SM clock x flops per lane operation
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     max_mhz = (clk or {}).get("sm_max_mhz") or 2070.0
-    lanes = 128 if p == 1 else 2
-    peak_nominal = 2.0 * lanes * sms * max_mhz * 1e6 / 1e12
+    lanes, per_lane = ((32, FLOPS_PER_WIDE["minors"]), (128, 2.0), (2, 2.0))[p]
+    peak_nominal = per_lane * lanes * sms * max_mhz * 1e6 / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if peak else None, "traffic": traffic,
             "traffic_launch": (f"the k = 30 launch of {S_} chains (ncu dram__bytes_read.sum + dram__bytes_write.sum)"
                                if traffic is not None else None),
             "ncu_pipe_active_k30": PIPE_K30[p],
             "kernel": ("walk_fp64_minors_kernel", "walk_fp32_minors_kernel", "walk_df_minors_kernel")[p],
-            "peak_source": ("measured on this GPU by bs_measure_fma_rates (2 flops per lane-FMA), "
+            "peak_source": ("measured on this GPU by bs_measure_wide_rate: 32 x 32 -> 64 bit integer products, "
+                            "22 algorithmic flops per 36 of them" if p == 0 else
+                            "measured on this GPU by bs_measure_fma_rates (2 flops per lane-FMA), "
                             + ("FP32 FMA pipe" if p == 1 else "FP64 pipe")),
+            "vs_fp64_fma_peak": achieved / (2.0 * fp64_rate / 1e12),
             "peak_nominal": peak_nominal, "frac_of_nominal": achieved / peak_nominal,
-            "peak_nominal_source": f"{lanes} FMA lanes / SM / clock x {sms} SMs x {max_mhz:.0f} MHz x 2",
+            "peak_nominal_source": f"{lanes} lanes / SM / clock x {sms} SMs x {max_mhz:.0f} MHz x {per_lane:.3g} flops",
             "walk_ms_per_step": st["walk_ms"][p] / psteps, "walk_launches": int(st["timed_launches"][p]),
             "walk_share_of_step": st["walk_ms"][p] / sum(prof_step_ms) if sum(prof_step_ms) else None,
             "measured_over": f"{psteps} profiled steps on the first timed steps' seeds, right after the timed "
@@ -519,9 +534,9 @@ def run_mine(args):
                           "dtype": DTYPES[name], "dtype_detail": DTYPE_DETAIL[name],
                           "samples_equal_to_headline_run": same}
 
-    # the plain FP64 kernels on single k = 30 jobs, as fractions of the FP64
-    # peak (the FP64 form is meant to keep the FP64 pipe >= 60 % busy for
-    # k >= 30): permanent 30 x 30, minors 29 x 30
+    # the FP64 kernels on single k = 30 jobs (permanent 30 x 30, minors 29 x
+    # 30): addends/s, against the FP64 FMA peak, and against the pipe they run
+    # on (integer products)
     fp64_k30, df_k30 = {}, {}
     ctx.set_profiling(True)
     u60 = S.haar_unitary(60, 77)
@@ -540,15 +555,15 @@ def run_mine(args):
             res[p] = (np.atleast_1d(v), s2["walk_ms"][p] / 1000.0, s2["addends"][p], s2["addend_flops"][p])
         _, secs, adds, flops = res[0]
         rate = adds / secs
-        # FP64-pipe operations the walk needs per addend at K = 30 columns:
-        # permanent 2K (update) + 4(K - 1) (product) + 2 (weighted sum);
-        # lane-pair minors about 14K (each lane: update K, suffix and prefix
-        # chains 2K - 4 each, accumulate 2K, exchange and weight about 6)
-        ops = 6 * 30 - 2 if kind == "perm" else 14 * 30
+        # integer products the walk needs per addend at K = 30 columns: 12
+        # per complex product, 29 of them (permanent) or 87 (minors)
+        ops = 12 * 29 if kind == "perm" else 36 * 29
         fp64_k30[kind] = {"addends_per_s": rate,
-                          "frac_of_fp64_peak": flops / secs / (2.0 * fp64_rate),
-                          "fp64_pipe_ops_per_addend": ops,
-                          "frac_of_fp64_pipe": rate * ops / fp64_rate}
+                          "vs_fp64_fma_peak": flops / secs / (2.0 * fp64_rate),
+                          # of the peak of the pipe the FP64 jobs run on, a product counted as 2 flops
+                          "frac_of_fp64_peak": flops / secs / (2.0 * wide_rate),
+                          "wide_products_per_addend": ops,
+                          "frac_of_fp64_pipe": rate * ops / wide_rate}
         vd, secs_d, adds_d, flops_d = res[2]
         norms = np.sqrt((np.abs(a) ** 2).sum(axis=0))
         scale = float(np.prod(norms)) / (float(norms.max()) if kind == "minors" else 1.0)
@@ -581,7 +596,8 @@ def run_mine(args):
         "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
         "clocks": clk, "other_forms": side, "fp64_kernels_k30": fp64_k30, "df_kernels_k30": df_k30,
         "serving": serving_c4, "wall_s": wall,
-        "fma_rates_measured": {"fp64_per_s": fp64_rate, "fp32_per_s": fp32_rate},
+        "fma_rates_measured": {"fp64_per_s": fp64_rate, "fp32_per_s": fp32_rate,
+                               "wide_products_per_s": wide_rate},
     }
     print(json.dumps(line), flush=True)
     ctx.close()
@@ -704,9 +720,11 @@ def run_batch(args):
         rates = ctx.measure_fma_rates()
         out[name] = {"permanents_per_s": len(items) / (ms / 1000), "ms_per_batch": ms,
                      "addends_per_s": sum(st["addends"]) / (ms / 1000) / args.steps,
-                     # FP64 and double-float against the FP64 pipe (FP64-equivalent flops), FP32 against its own
+                     # FP64 against the integer products, double-float against the FP64 pipe (FP64-equivalent
+                     # flops), FP32 against its own
                      "walk_kernel_frac_of_peak": (st["addend_flops"][p] / (st["walk_ms"][p] / 1000) /
-                                                  (2 * rates[1 if p == 1 else 0])) if st["walk_ms"][p] else None}
+                                                  (FLOPS_PER_WIDE["perm"] * ctx.measure_wide_rate(), 2 * rates[1],
+                                                   2 * rates[0])[p]) if st["walk_ms"][p] else None}
     sc = np.array([np.prod(np.sqrt((np.abs(a) ** 2 * M[:, None]).sum(0)) ** N) for a, M, N in items])
     rel = np.abs(res["mixed"] - res["fp64"]) / sc
     rel_df = np.abs(res["df"] - res["fp64"]) / sc
@@ -860,7 +878,7 @@ def run_formulas(args):
         secs = st["walk_ms"][0] / 1000.0
         speed[f] = {"addends": int(st["addends"][0]), "walk_s": secs, "call_s": wall,
                     "addends_per_s": st["addends"][0] / secs,
-                    "frac_of_fp64_peak": st["addend_flops"][0] / secs / (2.0 * fp64_rate)}
+                    "vs_fp64_fma_peak": st["addend_flops"][0] / secs / (2.0 * fp64_rate)}
     ctx.set_profiling(False)
     print(json.dumps({"workload": "formulas_haar_n8_24_and_n30", "metric": "relative error; addends/s",
                       "relative_error_max_of_2": acc, "speed_n30_fp64": speed,

@@ -378,6 +378,10 @@ int bs_ctx_reset_stats(bs_ctx* ctx);
  * (operations per second, 1 FMA = 2 flops), from a timed microbenchmark. */
 int bs_measure_fma_rates(bs_ctx* ctx, double* fp64_fma_per_s, double* fp32_fma_per_s);
 
+/* Measured lane rate of 32 x 32 -> 64 bit integer products (per second), the
+ * bound of the FP64 jobs' fixed-point walks (12 products per complex one). */
+int bs_measure_wide_rate(bs_ctx* ctx, double* wide_products_per_s);
+
 /* Host-only check of the n-ary reflected Gray counter the kernels use: walks
  * `steps` moves from index `start` over digits with the given radices (the
  * first nbin must be 2) and writes the Delta vector after every move to

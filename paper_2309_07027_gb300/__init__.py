@@ -108,6 +108,7 @@ def load():
         "bs_ctx_get_walk_times": ([vp, dp, C.c_int], C.c_int),
         "bs_ctx_reset_stats": ([vp], C.c_int),
         "bs_measure_fma_rates": ([vp, dp, dp], C.c_int),
+        "bs_measure_wide_rate": ([vp, dp], C.c_int),
         "bs_debug_gray_walk": ([C.c_int, C.c_int, ip, C.c_uint64, C.c_int, ip, ip, C.POINTER(C.c_uint64)],
                                C.c_int),
         "bs_debug_plan": ([C.c_int, C.c_int, ip, ip, C.c_int, i64p], C.c_int),
@@ -257,6 +258,12 @@ class Context:
         a, b = C.c_double(), C.c_double()
         _check(self._L.bs_measure_fma_rates(self._p, C.byref(a), C.byref(b)), self._p)
         return a.value, b.value
+
+    def measure_wide_rate(self):
+        """32 x 32 -> 64 bit integer lane products per second on this device."""
+        a = C.c_double()
+        _check(self._L.bs_measure_wide_rate(self._p, C.byref(a)), self._p)
+        return a.value
 
     # ---------------------------------------------------------- permanents
     def perm(self, a, row_mult=None, col_mult=None, mode: int = BS_FP64, with_tail: bool = False):

@@ -384,7 +384,6 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
             jb.log2L = r.log2L;
             jb.out_index = r.in.out_index;
             jb.n = p.n;
-            jb.normalize = r.prec != BS_PREC_FP64 ? 1 : 0;
             jb.prec = r.prec;
             jb.data_off = data_off[arena_of(r.prec)];
             jb.meta_off = (int64_t)meta.size();
@@ -815,7 +814,7 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
         int precs[2];
         const int np = sampler_precs(mode, precs);
         for (int pi = 0; pi < np; ++pi) {
-            const uint64_t cpt_min = precs[pi] == BS_PREC_FP64 ? 16 : precs[pi] == BS_PREC_FP32 ? 8 : 4;
+            const uint64_t cpt_min = precs[pi] == BS_PREC_FP64 ? 8 : precs[pi] == BS_PREC_FP32 ? 8 : 4;
             tasks_stride = std::max<uint64_t>(tasks_stride, cmax / (cpt_min << c->log2max[precs[pi]]) + 2);
         }
     }
@@ -1407,6 +1406,14 @@ int bs_measure_fma_rates(bs_ctx* c, double* fp64, double* fp32) {
     if (!ok_ctx(c) || !fp64 || !fp32) return fail(BS_EINVAL, "NULL argument");
     std::lock_guard<std::mutex> lk(c->mu);
     cudaError_t e = bs::measure_fma_rates(c->device, fp64, fp32);
+    if (e != cudaSuccess) return fail(BS_ECUDA, "microbenchmark: %s", cudaGetErrorString(e));
+    return BS_OK;
+}
+
+int bs_measure_wide_rate(bs_ctx* c, double* wide) {
+    if (!ok_ctx(c) || !wide) return fail(BS_EINVAL, "NULL argument");
+    std::lock_guard<std::mutex> lk(c->mu);
+    cudaError_t e = bs::measure_wide_rate(c->device, wide);
     if (e != cudaSuccess) return fail(BS_ECUDA, "microbenchmark: %s", cudaGetErrorString(e));
     return BS_OK;
 }

@@ -39,7 +39,6 @@ struct bs_job {
     int32_t log2L;         // chunk length exponent (one chunk per lane per task)
     int32_t out_index;     // perm: output slot; minors: first of K output slots
     int32_t n;             // photons of the formula (prefactor 2^(1-n))
-    int32_t normalize;     // 1: scale each column by a power of two (FP32 range)
     int32_t prec;          // BS_PREC_*: which kernels walk the job
     int64_t data_off;      // complex elements: c0[KP] then 2a[nrows][KP], KP = BS_ROW_STRIDE(K)
     int64_t meta_off;      // ints, see BS_META_* below
@@ -69,6 +68,10 @@ struct bs_job {
 //   binom[]             uint64 table written by the pack kernel: for each
 //                       digit j in order, C(M_j, d) for d = 0..M_j
 //                       (nrows + n - 1 entries in all)
+// colexp values of an FP64 column with a component that is not finite (its
+// sum of moduli reaches 2^1022 or is NaN): no finite scale, results NaN.
+#define BS_COLEXP_NAN_RE (1 << 20)
+#define BS_COLEXP_NAN_IM (1 << 21)
 #define BS_META_RADIX(jb) ((jb).meta_off)
 #define BS_META_DIGIT_SRC(jb) ((jb).meta_off + (jb).nrows)
 #define BS_META_COL_SRC(jb) ((jb).meta_off + 2 * (jb).nrows)

@@ -158,7 +158,6 @@ extern "C" int bs_perm_noalloc(const bs_c128* A, int rows, int cols, int ld, con
     jb.kind = BS_KIND_PERM;
     jb.log2L = log2L;
     jb.n = p.n;
-    jb.normalize = prec != BS_PREC_FP64 ? 1 : 0;
     jb.prec = prec;
     jb.reseed_log2 = reseed;
     jb.src_ld = nc;

@@ -3,13 +3,11 @@
 // pack:   for every job, reads its source matrix (device) and writes
 //           c0[col]   = sum over all rows of M_row * a_row,col  (all delta = +1)
 //           2a[j][col] = 2 * a_digit_j,col
-//         in the job's working precision.  With normalize set, column col is
-//         first scaled by 2^-e, e the smallest integer with
-//         sum_rows M_row (|Re a| + |Im a|) <= 2^e, so every column sum of the
-//         walk has modulus <= sqrt(2) and FP32 products cannot overflow; the
-//         exponents go to colexp[] and are undone exactly by the reduce
-//         kernel (Appendix A.5 normalises columns for the same reason; here the
-//         factors are powers of two, so the rescaling is exact).
+//         in the job's working precision, every column scaled by a power of
+//         two (pack.cuh); the exponents go to colexp[] and are undone exactly
+//         by the reduce kernel (Appendix A.5 normalises columns for the same
+//         reason; here the factors are powers of two, so the rescaling is
+//         exact).
 // reduce: sums each job's task partials (Sum2, twice double precision) in a fixed order and
 //         applies 2^(1-n) (Eq. bbfgrepeated prefactor) and the column scales.
 #include <cuda_runtime.h>
@@ -89,20 +87,30 @@ __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __re
     if (threadIdx.x == 0) {
         // prefactor: 2^(1-n) times the column scales (Eq. bbfgrepeated), or
         // (-1)^n (Eq. ryser), or (-1)^(n-1) 2 (Nijenhuis-Wilf)
-        int e = 0;
+        int e = 0, bad = 0;
         double sgn = 1.0;
+        const int* colexp = meta + BS_META_COLEXP(jb);
+        for (int c = 0; c < jb.K; ++c) {
+            if (jb.kind == BS_KIND_MINORS && c == col) continue;
+            if (colexp[c] >= BS_COLEXP_NAN_RE)
+                bad |= colexp[c];
+            else
+                e += colexp[c];
+        }
         if (jb.formula == BS_JOB_BBFG) {
-            const int* colexp = meta + BS_META_COLEXP(jb);
-            e = 1 - jb.n;
-            for (int c = 0; c < jb.K; ++c) e += colexp[c];
-            if (jb.kind == BS_KIND_MINORS) e -= colexp[col];
+            e += 1 - jb.n;
         } else if (jb.formula == BS_JOB_RYSER) {
             sgn = (jb.n & 1) ? -1.0 : 1.0;
         } else {
-            e = 1;
+            e += 1;
             sgn = ((jb.n - 1) & 1) ? -1.0 : 1.0;
         }
         ddv r = sre[0], i = sim[0];
+        if (bad) {  // an input that is not finite (a product of two or more columns mixes both components)
+            const double nan = __longlong_as_double(0x7ff8000000000000ll);
+            if (jb.K > 1 || (bad & BS_COLEXP_NAN_RE)) r = ddv{nan, nan};
+            if (jb.K > 1 || (bad & BS_COLEXP_NAN_IM)) i = ddv{nan, nan};
+        }
         out[jb.out_index + col] = make_double2(sgn * ldexp(r.hi, e), sgn * ldexp(i.hi, e));
         if (out_lo) out_lo[jb.out_index + col] = make_double2(sgn * ldexp(r.lo, e), sgn * ldexp(i.lo, e));
     }

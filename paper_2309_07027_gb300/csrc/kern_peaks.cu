@@ -1,4 +1,6 @@
-// Issue-rate microbenchmark for the FP64 and FP32 fused multiply-add pipes.
+// Issue-rate microbenchmarks: the FP64 and FP32 fused multiply-add pipes, and
+// 32 x 32 -> 64 bit integer products (the bound of the FP64 jobs' fixed-point
+// walks).
 //
 // Every thread runs 8 independent FMA chains (enough independent work to
 // keep the pipe busy at full occupancy); the grid fills every SM 8 CTAs
@@ -32,6 +34,27 @@ __global__ void fma_rate_kernel(T* out, int iters, T a, T b) {
     if (s == (T)-1234.5) out[0] = s;
 }
 
+// 8 independent chains of wide products per thread, each step's operands the
+// two halves of the last product (8 lanes per SM quarter and clock measured,
+// a quarter of the FP32 rate).
+__global__ void wide_rate_kernel(long long* out, int iters, long long seed) {
+    long long x[kChains];
+#pragma unroll
+    for (int i = 0; i < kChains; ++i) x[i] = seed * (i + 1) + threadIdx.x;
+    for (int it = 0; it < iters; ++it) {
+#pragma unroll
+        for (int u = 0; u < kInner; ++u) {
+#pragma unroll
+            for (int i = 0; i < kChains; ++i)
+                asm("mul.wide.s32 %0, %1, %2;" : "=l"(x[i]) : "r"((int)(x[i] >> 32)), "r"((int)x[i]));
+        }
+    }
+    long long s = 0;
+#pragma unroll
+    for (int i = 0; i < kChains; ++i) s ^= x[i];
+    if (s == 12345) out[0] = s;  // keeps the chains live
+}
+
 int sm_count(int device) {
     static int cached[64] = {0};
     if (device >= 0 && device < 64 && cached[device] > 0) return cached[device];
@@ -40,6 +63,16 @@ int sm_count(int device) {
     if (n < 1) n = 1;
     if (device >= 0 && device < 64) cached[device] = n;
     return n;
+}
+
+static void launch_rate(double* out, int blocks, int threads, int iters) {
+    fma_rate_kernel<double><<<blocks, threads>>>(out, iters, 0.9999, 1e-4);
+}
+static void launch_rate(float* out, int blocks, int threads, int iters) {
+    fma_rate_kernel<float><<<blocks, threads>>>(out, iters, 0.9999f, 1e-4f);
+}
+static void launch_rate(long long* out, int blocks, int threads, int iters) {
+    wide_rate_kernel<<<blocks, threads>>>(out, iters, 0x123456789abcdefll);
 }
 
 template <typename T>
@@ -54,11 +87,11 @@ static cudaError_t time_rate(int iters, double* rate) {
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    fma_rate_kernel<T><<<blocks, threads>>>(out, iters / 8 + 1, (T)0.9999, (T)1e-4);
+    launch_rate(out, blocks, threads, iters / 8 + 1);
     float best = 1e30f;
     for (int r = 0; r < 3; ++r) {
         cudaEventRecord(e0);
-        fma_rate_kernel<T><<<blocks, threads>>>(out, iters, (T)0.9999, (T)1e-4);
+        launch_rate(out, blocks, threads, iters);
         cudaEventRecord(e1);
         cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -81,6 +114,12 @@ cudaError_t measure_fma_rates(int device, double* fp64_per_s, double* fp32_per_s
     e = time_rate<double>(3000, fp64_per_s);
     if (e != cudaSuccess) return e;
     return time_rate<float>(150000, fp32_per_s);
+}
+
+cudaError_t measure_wide_rate(int device, double* wide_per_s) {
+    cudaError_t e = cudaSetDevice(device);
+    if (e != cudaSuccess) return e;
+    return time_rate<long long>(40000, wide_per_s);
 }
 
 }  // namespace bs

@@ -162,7 +162,6 @@ __device__ int plan_minors_step(const int* __restrict__ rows, const int* __restr
         jb.reseed_log2 = plan == 2 ? BS_FP32_RESEED_LOG2 : 0;
     }
     jb.prec = prec;
-    jb.normalize = prec != BS_PREC_FP64 ? 1 : 0;
     const int cpt = bs_chunks_per_task(BS_KIND_MINORS, prec, k);
     for (int j = 0; j < nrows; ++j) {
         meta[j] = drad[j];

@@ -1,22 +1,25 @@
-// FP64 walk kernels: permanents and fused Laplace minors, every step in
-// double precision (column sums, products, weights; compensated sums).
+// FP64 walk kernels: permanents and fused Laplace minors in 64-bit fixed
+// point (walk_fix.cuh), weights and sums in double and double-double.
 // One kernel per column bucket KB (K in (KB-4, KB]); the host groups jobs by
 // bucket, so each kernel keeps its own register allocation.  Inside, each
-// task runs the walk instance for its job's exact column count (permanents)
-// or owned-column count (minors), so no dead bucket column costs FP64 slots.
+// task runs the walk instance for its lanes' exact column count.
 #include "kernels.h"
+#include "sample.h"
 #include "walk.cuh"
+#include "walk_fix.cuh"
 
 namespace bs {
 
 constexpr int kPermBlock = 128;
 constexpr int kMinorsBlock = 64;
 
+// 128 registers (4 CTAs of 128 threads per SM) up to width 32, 168 above; one
+// CTA less ran 2 % slower at widths 26 to 30.
 template <int KB>
-__global__ void __launch_bounds__(kPermBlock) walk_fp64_perm_kernel(WalkArgs a) {
+__global__ void __launch_bounds__(kPermBlock, KB <= 32 ? 4 : 3) walk_fp64_perm_kernel(WalkArgs a) {
     const int lane = threadIdx.x & 31;
     const bs_job* __restrict__ jobs = a.jobs;
-    const cx<double>* __restrict__ data = static_cast<const cx<double>*>(a.data);
+    const zfix* __restrict__ data = static_cast<const zfix*>(a.data);
     const unsigned long long total = task_total(a);
     const int njobs = job_count(a);
     const unsigned long long deadline = warp_deadline(a.deadline_rel_ns);
@@ -30,37 +33,31 @@ __global__ void __launch_bounds__(kPermBlock) walk_fp64_perm_kernel(WalkArgs a) 
         }
         const uint32_t local = (uint32_t)(t - jb.task_begin) + jb.task_offset;
         const int* radix = a.meta + BS_META_RADIX(jb);
-        // the instance with the job's exact column count (K in (KB-4, KB])
-        switch (jb.K - (KB - 4)) {
-            case 1: walk_task_perm_fp64<KB, KB - 3>(jb, data, radix, a.partials, local, lane); break;
-            case 2: walk_task_perm_fp64<KB, KB - 2>(jb, data, radix, a.partials, local, lane); break;
-            case 3: walk_task_perm_fp64<KB, KB - 1>(jb, data, radix, a.partials, local, lane); break;
-            default: walk_task_perm_fp64<KB, KB>(jb, data, radix, a.partials, local, lane); break;
-        }
+        // the instance whose lanes own exactly HX = ceil(K / 2) columns
+        if (((jb.K + 1) >> 1) == KB / 2)
+            walk_task_perm_fix<KB, KB / 2>(jb, data, radix, a.partials, local, lane);
+        else
+            walk_task_perm_fix<KB, KB / 2 - 1>(jb, data, radix, a.partials, local, lane);
     }
 }
 
-// Resident CTAs per SM the fused-minor kernel is compiled for (64 threads
-// each).  Two walk instances inlined into one kernel raise the compiler's
-// register choice (width 32: 168 -> 216, 6 -> 4 CTAs per SM), so the kernel
-// keeps the budgets its one-instance form ran at, with no spills: 168
-// registers (6 CTAs) at widths 24 to 32, 128 (8) at 16 and 20, 96 (10) at 8
-// and 12, 72 (14) at 4, and the compiler's choice (4 CTAs) above 32.
+// Resident CTAs per SM that the fused-minor kernels are compiled for (64
+// threads each): 168 registers, 3 warps per scheduler from width 16 on.  Two
+// warps at 254 registers ran 9 % slower (width 28), four at 128 spill.
 template <int KB>
 struct MinorsMinBlocks {
-    static constexpr int value = KB <= 4 ? 14 : KB <= 12 ? 10 : KB <= 20 ? 8 : KB <= 32 ? 6 : 4;
+    static constexpr int value = KB <= 4 ? 14 : KB <= 8 ? 10 : KB <= 12 ? 8 : 6;
 };
 
 template <int KB>
 __global__ void __launch_bounds__(kMinorsBlock, MinorsMinBlocks<KB>::value) walk_fp64_minors_kernel(WalkArgs a) {
-    extern __shared__ double2 smem_fp64[];
+    constexpr int G = BS_MINORS_FP64_GROUP_KB(KB);
+    constexpr int HM = KB / G;  // most columns a lane owns
+    extern __shared__ double4 smem_fp64[];
     const int lane = threadIdx.x & 31;
-    const int stride = blockDim.x;
-    // [col][thread] plain-double runs, then per warp KB double-double totals
-    cx<double>* sm_acc = reinterpret_cast<cx<double>*>(smem_fp64) + threadIdx.x;
-    double4* wtot = reinterpret_cast<double4*>(smem_fp64 + (size_t)(KB / 2) * stride) + (threadIdx.x >> 5) * KB;
+    char* smem = reinterpret_cast<char*>(smem_fp64) + (threadIdx.x >> 5) * sizeof(MinorsSmem<G, HM>);
     const bs_job* __restrict__ jobs = a.jobs;
-    const cx<double>* __restrict__ data = static_cast<const cx<double>*>(a.data);
+    const zfix* __restrict__ data = static_cast<const zfix*>(a.data);
     const unsigned long long total = task_total(a);
     const int njobs = job_count(a);
     const unsigned long long deadline = warp_deadline(a.deadline_rel_ns);
@@ -74,11 +71,13 @@ __global__ void __launch_bounds__(kMinorsBlock, MinorsMinBlocks<KB>::value) walk
         }
         const uint32_t local = (uint32_t)(t - jb.task_begin) + jb.task_offset;
         const int* radix = a.meta + BS_META_RADIX(jb);
-        // the instance whose lanes own exactly Hr = ceil(K / 2) columns
-        if (((jb.K + 1) >> 1) == KB / 2)
-            walk_task_minors_fp64<KB, KB / 2>(jb, data, radix, a.partials, local, lane, sm_acc, wtot, stride);
+        // the instance whose lanes own exactly ceil(K / G) columns
+        if (G == 4 || ((jb.K + 1) >> 1) == HM)
+            walk_task_minors_fix<G, KB, HM>(jb, data, radix, a.partials, local, lane,
+                                            *reinterpret_cast<MinorsSmem<G, HM>*>(smem));
         else
-            walk_task_minors_fp64<KB, KB / 2 - 1>(jb, data, radix, a.partials, local, lane, sm_acc, wtot, stride);
+            walk_task_minors_fix<G, KB, HM - 1>(jb, data, radix, a.partials, local, lane,
+                                                *reinterpret_cast<MinorsSmem<G, HM - 1>*>(smem));
     }
 }
 
@@ -108,9 +107,8 @@ static cudaError_t run_perm(const WalkArgs& a, cudaStream_t s) {
 
 template <int KB>
 static cudaError_t run_minors(const WalkArgs& a, cudaStream_t s) {
-    // per thread and owned column a 16-byte run; per warp and column a
-    // 32-byte double-double total
-    size_t smem = (size_t)kMinorsBlock * (KB / 2) * sizeof(cx<double>) + (size_t)(kMinorsBlock / 32) * KB * sizeof(double4);
+    constexpr int G = BS_MINORS_FP64_GROUP_KB(KB);
+    const size_t smem = (kMinorsBlock / 32) * sizeof(MinorsSmem<G, KB / G>);
     cudaError_t e =
         cudaFuncSetAttribute(walk_fp64_minors_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

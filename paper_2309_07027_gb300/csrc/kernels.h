@@ -47,6 +47,8 @@ cudaError_t launch_reduce(const bs_job* jobs, int njobs, const bs_zdd* partials,
 // Measured issue rates (lane-operations per second) of the FP64 and FP32
 // fused multiply-add pipes, from a timed microbenchmark on this device.
 cudaError_t measure_fma_rates(int device, double* fp64_per_s, double* fp32_per_s);
+// The same for 32 x 32 -> 64 bit integer products.
+cudaError_t measure_wide_rate(int device, double* wide_per_s);
 
 int sm_count(int device);
 

@@ -1,13 +1,13 @@
 // Packing of one job (shared by the batch pack kernel and the sampler's
-// device planner): c0[col] = sum over rows of M_row * a_row,col (every
-// delta = +1), computed in double-double and rounded, and 2a[j][col] for every
-// digit row, in the job's working precision, rows of stride
-// KP = BS_ROW_STRIDE(K).  FP64 rows are plain complex doubles; FP32 rows are
-// column pairs {re(2p), re(2p+1), im(2p), im(2p+1)} (the packed layout of
-// walk_fp32.cuh).  Pad columns: zero rows, c0 = 1 in FP32 jobs (a neutral
-// factor) and 0 in FP64 jobs.  With normalize set, column col
-// is scaled by 2^-e (e: smallest integer with sum_rows M_row (|Re a| + |Im a|)
-// <= 2^e) and e is stored in colexp[col] for the reduce kernel.
+// device planner): the start sums c0[col] = sum over rows of M_row * a_row,col
+// (every delta = +1) and 2a[j][col] for every digit row, rows of stride KP.
+// Every column is scaled by a power of two whose exponent goes to colexp[col]
+// and is undone exactly by the reduce kernel.
+// FP64 jobs: 64-bit fixed point (pack_fix below, walk_fix.cuh).
+// FP32 jobs: c0 in double-double, rounded; column pairs {re(2p), re(2p+1),
+// im(2p), im(2p+1)} (the packed layout of walk_fp32.cuh), column col scaled
+// by 2^-e (e: smallest integer with sum_rows M_row (|Re a| + |Im a|) <= 2^e);
+// pad columns have zero rows and c0 = 1 (a neutral factor).
 // Double-float (DF) jobs: rows of stride BS_ROW_STRIDE_DF(K) (a multiple of
 // 8), column col scaled by 2^(2 - e) (colexp = e - 2) so that every column
 // sum has |Re|, |Im| <= 4, and every entry quantised to a high part on the
@@ -19,6 +19,7 @@
 #include "bs_job.h"
 #include "gray.h"
 #include "walk.cuh"
+#include "walk_fix.cuh"
 
 namespace bs {
 
@@ -52,9 +53,100 @@ __device__ __forceinline__ void put_df(void* data, const bs_job& jb, int KP, int
     q[6] = im.y;
 }
 
+// Fixed-point rows of an FP64 job (walk_fix.cuh): column col scaled by
+// 2^(63 - e), e (stored in colexp) the smallest integer with 2^e > b (1 +
+// 2^-20), b = sum over rows of M_row (|Re a| + |Im a|); every entry rounded
+// once to an integer, c0 and 2a formed from those integers modulo 2^64.  Ryser and Nijenhuis-Wilf jobs:
+// product column col is matrix row sc; digit j is matrix column dsrc[j],
+// added with +1 when it enters the subset, so the packed row is -a (the walk
+// subtracts rows of digits whose Delta is 1); start sums 0 (Ryser) or
+// x = a_(sc, n-1) - (sum_j a_(sc, j)) / 2 (Nijenhuis-Wilf, whose entries are
+// rounded to even integers so that the half is exact).  A column with an
+// entry that is not finite gets zeros and BS_COLEXP_NAN_*: the reduce kernel
+// writes NaN wherever such a column enters the product.
+__device__ __forceinline__ void pack_fix(const bs_job& jb, const double2* __restrict__ src, int* __restrict__ meta,
+                                         zfix* __restrict__ out, int tid, int nthreads) {
+    const int* radix = meta + BS_META_RADIX(jb);
+    const int* dsrc = meta + BS_META_DIGIT_SRC(jb);
+    const int* csrc = meta + BS_META_COL_SRC(jb);
+    int* colexp = meta + BS_META_COLEXP(jb);
+    const int prow = meta[BS_META_PINNED(jb)];
+    const int KP = BS_ROW_STRIDE(jb.K);
+    const bool bbfg = jb.formula == BS_JOB_BBFG, nw = jb.formula == BS_JOB_NW;
+    for (int col = tid; col < KP; col += nthreads) {
+        if (col >= jb.K) {  // pad column: a column sum of exactly 1 = 2^62 / 2^63 2^1
+            out[col] = zfix{1ll << 62, 0};
+            for (int j = 1; j <= jb.nrows; ++j) out[(size_t)j * KP + col] = zfix{0, 0};
+            continue;
+        }
+        const int sc = csrc[col];
+        double bre = 0.0, bim = 0.0;
+        if (bbfg) {
+            const double2 a = src_elem(src, jb, prow, sc);
+            bre = fabs(a.x);
+            bim = fabs(a.y);
+        } else if (nw) {
+            const double2 a = src_elem(src, jb, jb.n - 1, sc);
+            bre = fabs(a.x);
+            bim = fabs(a.y);
+        }
+        for (int j = 0; j < jb.nrows; ++j) {
+            const double2 d = src_elem(src, jb, dsrc[j], sc);
+            const double m = bbfg ? (double)(radix[j] - 1) : 1.0;
+            bre += m * fabs(d.x);
+            bim += m * fabs(d.y);
+        }
+        int flags = 0;
+        if (!isfinite(bre)) flags |= BS_COLEXP_NAN_RE;
+        if (!isfinite(bim)) flags |= BS_COLEXP_NAN_IM;
+        if (flags) {
+            colexp[col] = flags;
+            for (int j = 0; j <= jb.nrows; ++j) out[(size_t)j * KP + col] = zfix{0, 0};
+            continue;
+        }
+        int e = 0;
+        const double b = 0.25 * bre + 0.25 * bim;  // a quarter: b must not overflow
+        if (b > 0.0) {
+            (void)frexp(b * (1.0 + 0x1p-20), &e);
+            e += 2;
+        }
+        colexp[col] = e;
+        const int sh = nw ? 62 - e : 63 - e;
+        const int up = nw ? 1 : 0;
+        unsigned long long sre = 0, sim = 0;  // the start sums
+        if (bbfg || nw) {
+            const double2 a = src_elem(src, jb, bbfg ? prow : jb.n - 1, sc);
+            sre = (unsigned long long)__double2ll_rn(ldexp(a.x, sh));
+            sim = (unsigned long long)__double2ll_rn(ldexp(a.y, sh));
+        }
+        for (int j = 0; j < jb.nrows; ++j) {
+            const double2 d = src_elem(src, jb, dsrc[j], sc);
+            const unsigned long long qre = (unsigned long long)__double2ll_rn(ldexp(d.x, sh));
+            const unsigned long long qim = (unsigned long long)__double2ll_rn(ldexp(d.y, sh));
+            zfix row;
+            if (bbfg) {
+                const unsigned long long m = (unsigned long long)(radix[j] - 1);
+                sre += m * qre;
+                sim += m * qim;
+                row.re = (long long)(2ull * qre);
+                row.im = (long long)(2ull * qim);
+            } else {
+                // Nijenhuis-Wilf start: 2 x = 2 a_last - sum over all columns
+                // = a_last - sum over the digits, in even units
+                sre -= nw ? qre : 0ull;
+                sim -= nw ? qim : 0ull;
+                row.re = -(long long)(qre << up);
+                row.im = -(long long)(qim << up);
+            }
+            out[(size_t)(1 + j) * KP + col] = row;
+        }
+        out[col].re = (long long)sre;
+        out[col].im = (long long)sim;
+    }
+}
+
 __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __restrict__ src, int* __restrict__ meta,
                          void* __restrict__ data, int prec, int tid, int nthreads) {
-    const int fp32 = prec == BS_PREC_FP32;
     const int df = prec == BS_PREC_DF;
     const int* radix = meta + BS_META_RADIX(jb);
     const int* dsrc = meta + BS_META_DIGIT_SRC(jb);
@@ -68,69 +160,34 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
         for (int j = 0; j < jb.nrows; ++j)
             for (int d = 0; d < radix[j]; ++d) binom[at++] = bs_binom(radix[j] - 1, d);
     }
-    const int KP = df ? BS_ROW_STRIDE_DF(jb.K) : BS_ROW_STRIDE(jb.K);
-    if (jb.formula != BS_JOB_BBFG) {
-        // Ryser / Nijenhuis-Wilf (FP64): product column col is matrix row
-        // sc; digit j is matrix column dsrc[j], added with +1 when it enters
-        // the subset, so the packed row is -a (the walk subtracts rows of
-        // digits whose Delta is 1).  Start sums: 0 (Ryser) or
-        // x = a_(sc, n-1) - (sum_j a_(sc, j)) / 2 (Nijenhuis-Wilf).
-        cx<double>* out = static_cast<cx<double>*>(data) + jb.data_off;
-        for (int col = tid; col < KP; col += nthreads) {
-            if (col >= jb.K) {
-                for (int j = 0; j <= jb.nrows; ++j) out[(size_t)j * KP + col] = cx<double>{0.0, 0.0};
-                continue;
-            }
-            colexp[col] = 0;
-            const int sc = csrc[col];
-            ddv sre = {0.0, 0.0}, sim = {0.0, 0.0};
-            if (jb.formula == BS_JOB_NW) {
-                for (int j = 0; j < jb.n; ++j) {
-                    const double2 d = src_elem(src, jb, j, sc);
-                    sre = dd_add_d(sre, -0.5 * d.x);
-                    sim = dd_add_d(sim, -0.5 * d.y);
-                }
-                const double2 last = src_elem(src, jb, jb.n - 1, sc);
-                sre = dd_add_d(sre, last.x);
-                sim = dd_add_d(sim, last.y);
-            }
-            out[col] = cx<double>{sre.hi, sim.hi};
-            for (int j = 0; j < jb.nrows; ++j) {
-                const double2 d = src_elem(src, jb, dsrc[j], sc);
-                out[(size_t)(1 + j) * KP + col] = cx<double>{-d.x, -d.y};
-            }
-        }
+    if (prec == BS_PREC_FP64) {
+        pack_fix(jb, src, meta, static_cast<zfix*>(data) + jb.data_off, tid, nthreads);
         return;
     }
+    const int KP = df ? BS_ROW_STRIDE_DF(jb.K) : BS_ROW_STRIDE(jb.K);
     for (int col = tid; col < KP; col += nthreads) {
         if (col >= jb.K) {  // pad column
             if (df) {
                 put_df(data, jb, KP, 0, col, make_float2(1.f, 0.f), make_float2(0.f, 0.f));
                 for (int j = 1; j <= jb.nrows; ++j) put_df(data, jb, KP, j, col, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
-            } else if (fp32) {
+            } else {
                 put_f32(data, jb, KP, 0, col, 1.f, 0.f);
                 for (int j = 1; j <= jb.nrows; ++j) put_f32(data, jb, KP, j, col, 0.f, 0.f);
-            } else {
-                cx<double>* out = static_cast<cx<double>*>(data) + jb.data_off;
-                for (int j = 0; j <= jb.nrows; ++j) out[(size_t)j * KP + col] = cx<double>{0.0, 0.0};
             }
             continue;
         }
         const int sc = csrc[col];
         int e = 0;
-        if (jb.normalize) {
-            double2 a = src_elem(src, jb, prow, sc);
-            double b = fabs(a.x) + fabs(a.y);
-            for (int j = 0; j < jb.nrows; ++j) {
-                double2 d = src_elem(src, jb, dsrc[j], sc);
-                b += (double)(radix[j] - 1) * (fabs(d.x) + fabs(d.y));
-            }
-            if (b > 0.0) (void)frexp(b, &e);  // b = f 2^e, f in [0.5, 1)
-            if (df) e -= 2;                   // DF: column sums up to 4 (walk_df.cuh)
+        double2 a = src_elem(src, jb, prow, sc);
+        double b = fabs(a.x) + fabs(a.y);
+        for (int j = 0; j < jb.nrows; ++j) {
+            double2 d = src_elem(src, jb, dsrc[j], sc);
+            b += (double)(radix[j] - 1) * (fabs(d.x) + fabs(d.y));
         }
+        if (b > 0.0) (void)frexp(b, &e);  // b = f 2^e, f in [0.5, 1)
+        if (df) e -= 2;                   // DF: column sums up to 4 (walk_df.cuh)
         colexp[col] = e;
         // c0 in double-double (each product split exactly with an FMA), rounded
-        double2 a = src_elem(src, jb, prow, sc);
         ddv sre = {ldexp(a.x, -e), 0.0}, sim = {ldexp(a.y, -e), 0.0};
         for (int j = 0; j < jb.nrows; ++j) {
             double2 d = src_elem(src, jb, dsrc[j], sc);
@@ -148,18 +205,11 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
                 put_df(data, jb, KP, 1 + j, col, df_quantise(ldexp(d.x, 1 - e), 0.0),
                        df_quantise(ldexp(d.y, 1 - e), 0.0));
             }
-        } else if (fp32) {
+        } else {
             put_f32(data, jb, KP, 0, col, (float)sre.hi, (float)sim.hi);
             for (int j = 0; j < jb.nrows; ++j) {
                 double2 d = src_elem(src, jb, dsrc[j], sc);
                 put_f32(data, jb, KP, 1 + j, col, (float)ldexp(d.x, 1 - e), (float)ldexp(d.y, 1 - e));
-            }
-        } else {
-            cx<double>* out = static_cast<cx<double>*>(data) + jb.data_off;
-            out[col] = cx<double>{sre.hi, sim.hi};
-            for (int j = 0; j < jb.nrows; ++j) {
-                double2 d = src_elem(src, jb, dsrc[j], sc);
-                out[(size_t)(1 + j) * KP + col] = cx<double>{ldexp(d.x, 1 - e), ldexp(d.y, 1 - e)};
             }
         }
     }

@@ -91,6 +91,8 @@ BS_HD int bs_choose_log2L_single(uint64_t C, int cpt, int log2max, int target) {
 // the permanent kernels give each lane its own chunk (32 per task).
 #define BS_MINORS_FP32_GROUP_KB(KB) (((KB) == 24 || (KB) == 48) ? 4 : 2)
 BS_HD int bs_minors_fp32_group(int K) { return BS_MINORS_FP32_GROUP_KB((K + 3) & ~3); }
+// Lanes per chunk of the FP64 fused minors, by 4-column bucket width.
+#define BS_MINORS_FP64_GROUP_KB(KB) ((KB) > 32 ? 4 : 2)
 // Lanes per chunk of the double-float kernels (permanent and minors), by
 // 8-column bucket width KB: each lane owns KB / (2G) column pairs
 // (8 -> 1 x 4, 16 -> 2 x 4, 24 -> 4 x 3, 32 -> 4 x 4, 40 -> 4 x 5,
@@ -100,7 +102,7 @@ BS_HD int bs_df_group(int K) { return BS_DF_GROUP_KB((K + 7) & ~7); }
 BS_HD int bs_chunks_per_task(int kind, int prec, int K) {
     if (prec == BS_PREC_DF) return 32 / bs_df_group(K);
     if (kind != BS_KIND_MINORS) return 32;
-    return prec == BS_PREC_FP32 ? 32 / bs_minors_fp32_group(K) : 16;  // FP64 minors: lane pairs
+    return 32 / (prec == BS_PREC_FP32 ? bs_minors_fp32_group(K) : BS_MINORS_FP64_GROUP_KB((K + 3) & ~3));
 }
 
 // Algorithmic flops of one addend (the roofline numerator):

@@ -282,7 +282,6 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
         jb.kind = r->kind;
         jb.log2L = r->log2L;
         jb.n = p.n;
-        jb.normalize = r->prec != BS_PREC_FP64 ? 1 : 0;
         jb.prec = r->prec;
         jb.reseed_log2 = r->reseed;
         jb.data_off = r->data_off;
@@ -837,7 +836,7 @@ int64_t bs_server_submit_sample(bs_server* s, const bs_c128* U, int m_rows, int 
         const int np = s->mode == BS_MIXED ? 2 : 1;
         for (int i = 0; i < np; ++i) {
             const int q = s->mode == BS_MIXED ? precs_mixed[i] : prec_one;
-            const uint64_t cpt_min = q == BS_PREC_FP64 ? 16 : q == BS_PREC_FP32 ? 8 : 4;
+            const uint64_t cpt_min = q == BS_PREC_FP64 ? 8 : q == BS_PREC_FP32 ? 8 : 4;
             ts = std::max<uint64_t>(ts, cmax / (cpt_min << bs_default_log2max(q)) + 2);
         }
         r->tasks_stride = ts;

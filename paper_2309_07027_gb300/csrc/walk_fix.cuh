@@ -1,0 +1,618 @@
+// FP64-class walks in 64-bit fixed point on the integer pipes.
+//
+// Why: one FP64 instruction of a warp holds its scheduler's FP64 pipe for 64
+// cycles on this part (2 lanes per SM and clock), a 32 x 32 -> 64 bit integer
+// multiply-add (IMAD.WIDE) the FMA-heavy pipe for 4.  A complex product costs
+// 4 FP64 instructions (256 cycles) or, on two-limb 62-bit mantissas, 12
+// IMAD.WIDE (48 cycles) with the remaining integer work on the ALU beside
+// them -- and the mantissas are 8 bits longer than a double's.
+//
+// Numbers.
+//   * Column sums are exact.  Pack scales column j by 2^(63 - e_j), 2^e_j >
+//     sum_rows M (|Re a| + |Im a|) (1 + 2^-20), and rounds every entry once
+//     to an integer; c0 and the rows 2a are integers modulo 2^64, and the
+//     sums |Re c| + |Im c| < 2^63 (1 - 2^-21), so the walk's 64-bit additions
+//     give c0 - sum_j Delta_j 2a_j of the rounded matrix without any drift,
+//     whatever the chunk length.
+//   * A product operand is (h, l), value h 2^32 + l with l a signed 32-bit
+//     limb.  A product keeps the high 64 of its 128 bits: hh + cross / 2^32,
+//     the two cross terms summed in 64 bits and rounded, the low x low term
+//     (below one unit of the result, zero mean) left out.  Operands are kept
+//     normalised (larger component in [2^61, 2^62)) with an integer exponent
+//     beside them: a normalised operand loses about 2^-57 per product, where
+//     a double loses 2^-53.
+//   * Bounds.  |h| <= 2^30 for normalised operands; for column sums
+//     |h_re| + |h_im| <= 2^31 (1 - 2^-21) + 1; |l| <= 2^31.  Every cross sum
+//     stays below 2^63 in magnitude (four terms of at most 2^61, or two of
+//     2^61 and two that add up to less than 2^62), every high sum below 2^62.
+//     Only high limbs are negated (a low limb of -2^31 has no negative).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include "bs_job.h"
+#include "gray.h"
+#include "walk.cuh"
+
+namespace bs {
+
+// A packed entry: a complex 64-bit integer.
+struct __align__(16) zfix {
+    long long re, im;
+};
+
+// Product operand: two signed limbs per component.
+struct zlimb {
+    int rl, rh, il, ih;
+};
+
+// Raw product: 64-bit components.
+struct zraw {
+    unsigned long long re, im;
+};
+
+// Limbs of a 64-bit value.
+__device__ __forceinline__ zlimb limbs_of(const zraw& v) {
+    zlimb o;
+    o.rl = (int)(uint32_t)v.re;
+    o.rh = (int)((uint32_t)(v.re >> 32) + ((uint32_t)v.re >> 31));
+    o.il = (int)(uint32_t)v.im;
+    o.ih = (int)((uint32_t)(v.im >> 32) + ((uint32_t)v.im >> 31));
+    return o;
+}
+
+__device__ __forceinline__ zraw raw_of(const zlimb& v) {
+    return zraw{((unsigned long long)(uint32_t)v.rh << 32) + (unsigned long long)(long long)v.rl,
+                ((unsigned long long)(uint32_t)v.ih << 32) + (unsigned long long)(long long)v.il};
+}
+
+// high + cross / 2^32, rounded down.
+__device__ __forceinline__ long long fix_combine(long long high, long long cross) { return high + (cross >> 32); }
+
+__device__ __forceinline__ long long mul_wide(int a, int b) {
+    long long d;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// c + a b in one IMAD.WIDE (the compiler fuses this form; from mad.wide it
+// makes a product and a 64-bit addition).
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return c + mul_wide(a, b); }
+
+// z + a b / 2^64 (ADD = 1) or a b / 2^64.
+template <int ROUND, int ADD>
+__device__ __forceinline__ zraw fix_cmul_add(const zraw& z, const zlimb& a, const zlimb& b) {
+    constexpr long long half = ROUND ? 0x80000000ll : 0ll;
+    const long long x = mad_wide(a.rl, b.rh, mad_wide(a.rh, b.rl, half)) - mad_wide(a.il, b.ih, mul_wide(a.ih, b.il));
+    long long y = mad_wide(a.rl, b.ih, mad_wide(a.rh, b.il, half));
+    y = mad_wide(a.il, b.rh, mad_wide(a.ih, b.rl, y));
+    const long long p = (ADD ? mad_wide(a.rh, b.rh, (long long)z.re) : mul_wide(a.rh, b.rh)) - mul_wide(a.ih, b.ih);
+    const long long q = mad_wide(a.ih, b.rh, ADD ? mad_wide(a.rh, b.ih, (long long)z.im) : mul_wide(a.rh, b.ih));
+    return zraw{(unsigned long long)fix_combine(p, x), (unsigned long long)fix_combine(q, y)};
+}
+template <int ROUND = 1>
+__device__ __forceinline__ zraw fix_cmul(const zlimb& a, const zlimb& b) {
+    return fix_cmul_add<ROUND, 0>(zraw{0ull, 0ull}, a, b);
+}
+
+// The real (part = 0) or imaginary (part = 1) component of fix_cmul(a, b).
+__device__ __forceinline__ long long fix_cmul_part(const zlimb& a, const zlimb& b, int part) {
+    const int uh = part ? b.ih : b.rh, ul = part ? b.il : b.rl;   // times a's real part
+    const int vh = part ? b.rh : b.ih, vl = part ? b.rl : b.il;   // times +-a's imaginary part
+    const int sah = part ? a.ih : -a.ih, svh = part ? vh : -vh;
+    const long long x = mad_wide(a.rl, uh, mad_wide(a.rh, ul, 0x80000000ll)) + mad_wide(a.il, svh, mul_wide(sah, vl));
+    const long long p = mad_wide(sah, vh, mul_wide(a.rh, uh));
+    return fix_combine(p, x);
+}
+
+// Shift that brings the larger component of v (|v| < 2^62) into
+// [2^61, 2^62); at most 30 (a value below 2^32 comes out shifted by 30).
+__device__ __forceinline__ int fix_norm_shift(const zraw& v) {
+    const int rh = (int)(v.re >> 32), ih = (int)(v.im >> 32);
+    return __clz(abs(rh) | abs(ih)) - 2;
+}
+
+// Limbs of v 2^s.
+__device__ __forceinline__ zlimb fix_shift(const zraw& v, int s) {
+    const uint32_t rl = (uint32_t)v.re, rh = (uint32_t)(v.re >> 32);
+    const uint32_t il = (uint32_t)v.im, ih = (uint32_t)(v.im >> 32);
+    zlimb o;
+    const uint32_t a = rl << s, b = il << s;
+    o.rl = (int)a;
+    o.rh = (int)(__funnelshift_l(rl, rh, s) + (a >> 31));
+    o.il = (int)b;
+    o.ih = (int)(__funnelshift_l(il, ih, s) + (b >> 31));
+    return o;
+}
+
+__device__ __forceinline__ zlimb fix_normalise(const zraw& v, int& e) {
+    const int s = fix_norm_shift(v);
+    e -= s;
+    return fix_shift(v, s);
+}
+
+// 2^e w for w a nonzero double of magnitude below 2^64, by the exponent
+// field; e clamped so that the result stays normal (a product 2^-900 below
+// the column bounds adds nothing to a sum of them).
+__device__ __forceinline__ double scale_pow2(double w, int e) {
+    if (e < -900) e = -900;
+    return __hiloint2double(__double2hiint(w) + (e << 20), __double2loint(w));
+}
+
+// Column sums of the decoded state, c0 - sum_j Delta_j 2a_j, for N columns
+// from column cbase on.
+template <int N, int KP>
+__device__ __forceinline__ void fix_seed(zraw (&c)[N], const bs_gray& g, const zfix* __restrict__ c0, int nbin,
+                                         int nrows) {
+    const zfix* a2 = c0 + KP;
+#pragma unroll
+    for (int t = 0; t < N; ++t) {
+        const zfix v = c0[t];
+        c[t].re = (unsigned long long)v.re;
+        c[t].im = (unsigned long long)v.im;
+    }
+    uint64_t bits = g.dbin;
+    while (bits) {
+        const int j = bs_ctz64(bits);
+        bits &= bits - 1;
+        const zfix* row = a2 + (size_t)j * KP;
+#pragma unroll
+        for (int t = 0; t < N; ++t) {
+            const zfix v = row[t];
+            c[t].re -= (unsigned long long)v.re;
+            c[t].im -= (unsigned long long)v.im;
+        }
+    }
+    for (int j = nbin; j < nrows; ++j) {
+        const int d = g.del[j];
+        if (d == 0) continue;
+        const zfix* row = a2 + (size_t)j * KP;
+#pragma unroll
+        for (int t = 0; t < N; ++t) {
+            const zfix v = row[t];
+            c[t].re -= (unsigned long long)v.re * (unsigned long long)d;
+            c[t].im -= (unsigned long long)v.im * (unsigned long long)d;
+        }
+    }
+}
+
+// One digit move of N column sums: c -= row (neg = 1) or c += row.  The
+// whole warp calls it; nearly always its lanes move the same way (they walk
+// aligned chunks), and the two uniform branches spend no instruction on the
+// sign.
+template <int N>
+__device__ __forceinline__ void fix_update(zraw (&c)[N], const zfix* __restrict__ row, uint32_t neg) {
+    const longlong2* p = reinterpret_cast<const longlong2*>(row);
+    const unsigned down = __ballot_sync(0xffffffffu, neg != 0u);
+    if (down == 0u) {
+#pragma unroll
+        for (int t = 0; t < N; ++t) {
+            const longlong2 v = __ldg(p + t);
+            c[t].re += (unsigned long long)v.x;
+            c[t].im += (unsigned long long)v.y;
+        }
+    } else if (down == 0xffffffffu) {
+#pragma unroll
+        for (int t = 0; t < N; ++t) {
+            const longlong2 v = __ldg(p + t);
+            c[t].re -= (unsigned long long)v.x;
+            c[t].im -= (unsigned long long)v.y;
+        }
+    } else {
+        const long long m = -(long long)neg;
+#pragma unroll
+        for (int t = 0; t < N; ++t) {
+            const longlong2 v = __ldg(p + t);
+            c[t].re += (unsigned long long)((v.x ^ m) - m);
+            c[t].im += (unsigned long long)((v.y ^ m) - m);
+        }
+    }
+}
+
+// A leaf of a lane's product, as a raw value below 2^62 with exponent
+// kLeafExp against the column bounds: the product of a pair of column sums,
+// or half an odd last one (a column sum may reach 2^63).
+constexpr int kLeafExp = -62;
+template <int N>
+__device__ __forceinline__ zraw fix_leaf(const zraw (&c)[N], int j) {
+    if (2 * j + 1 < N) return fix_cmul<0>(limbs_of(c[2 * j]), limbs_of(c[2 * j + 1]));
+    return zraw{(unsigned long long)((long long)c[2 * j].re >> 1), (unsigned long long)((long long)c[2 * j].im >> 1)};
+}
+
+// Product of a lane's N column sums as a normalised operand, and its exponent
+// against the column bounds: leaves (independent of one another), then their
+// running product, normalised after every leaf.  A typical column sum is
+// 2^59.5 (its bound 2^63 is a sum of moduli, it is a root of squares), a pair
+// 2^55, and a pair times a normalised operand 2^52.5, so a pair costs about
+// 2^-54 in relative rounding, where two products of doubles cost 2^-53.
+template <int N>
+__device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e) {
+    e = kLeafExp;
+    zlimb p = fix_normalise(fix_leaf(c, 0), e);
+#pragma unroll
+    for (int j = 1; 2 * j < N; ++j) {
+        e += 64 + kLeafExp;
+        p = fix_normalise(fix_cmul(p, limbs_of(fix_leaf(c, j))), e);
+    }
+    return p;
+}
+
+// ---------------------------------------------------------------- one task: permanent
+// Two lanes share one chunk: lane 2p + h owns the columns [h HX, h HX + HX),
+// HX = ceil(K / 2) (an odd K leaves lane h = 1 a pad column that is exactly
+// 1), so the column sums take 4 HX registers and 4 warps per scheduler fit
+// up to K = 32.  Per addend each lane forms the product of its columns, the
+// lanes swap them (5 shuffles), and lane h = 0 forms the real, h = 1 the
+// imaginary part of the product of the two: half a complex product each.
+// That part is converted to double and added with the weight 2^e W (one
+// conversion and one FMA per lane on the FP64 pipe, which nothing else here
+// uses), in runs of FOLD folded into a double-double.  A task's 32 chunks
+// are walked as two rounds of 16.  Every lane walks the round's longest
+// chunk, with weight 0 after its own end, so that the warp stays converged.
+//
+// 30 x 30 permanent (2^29 addends): 165 ms in double (FP64 pipe 94 % busy),
+// 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 30.0
+// ms here; 73 cycles per warp, column and addend, of which the 12 integer
+// products hold the FMA-heavy pipe 52 (72 % busy) and 25 other integer
+// instructions take the rest.  Relative error (23 x 23, Haar): 6.8e-15, in
+// double 2.7e-14.
+template <int KB, int HX>
+__device__ void walk_task_perm_fix(const bs_job& jb, const zfix* __restrict__ data, const int* __restrict__ radix,
+                                   bs_zdd* __restrict__ partials, uint32_t local, int lane) {
+    constexpr uint32_t FOLD = 64;
+    constexpr int KP = KB;  // = BS_ROW_STRIDE(K) for every K of the bucket
+    const int half = lane & 1;
+    const zfix* c0 = data + jb.data_off + half * HX;
+    const zfix* a2 = c0 + KP;
+    // exponent of a product of both lanes' operands: the last product's 64,
+    // and 1 for the pad column (2^62 stands for 1, bound 2)
+    const int e_pair = 64 + (jb.K & 1);
+    ddv sum = {0.0, 0.0};
+    for (int round = 0; round < 2; ++round) {
+        const uint64_t i0_own = ((uint64_t)local * 32u + (uint64_t)(16 * round + (lane >> 1))) << jb.log2L;
+        const bool has = i0_own < jb.C;
+        const uint64_t i0 = has ? i0_own : 0ull;
+        uint32_t len = 0;
+        if (has) {
+            const uint64_t rem = jb.C - i0;
+            len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
+        }
+        const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
+        if (steps == 0u) break;
+        bs_gray g;
+        ChunkStepper st;
+        st.init(g, i0, jb.nbin, jb.nrows, radix,
+                reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
+        zraw c[HX];
+        fix_seed<HX, KP>(c, g, c0, jb.nbin, jb.nrows);
+        double ws = signed_weight<double>(g.w, g.parity);
+        double acc = 0.0;
+        for (uint32_t s = 0; s < steps; ++s) {
+            int e;
+            const zlimb p = fix_product<HX>(c, e);
+            zlimb q;
+            q.rh = __shfl_xor_sync(0xffffffffu, p.rh, 1);
+            q.rl = __shfl_xor_sync(0xffffffffu, p.rl, 1);
+            q.ih = __shfl_xor_sync(0xffffffffu, p.ih, 1);
+            q.il = __shfl_xor_sync(0xffffffffu, p.il, 1);
+            e += __shfl_xor_sync(0xffffffffu, e, 1) + e_pair;
+            const long long v = fix_cmul_part(p, q, half);
+            const double f = s < len ? scale_pow2(ws, e) : 0.0;
+            acc = bfma(f, (double)v, acc);
+            if (((s + 1u) & (FOLD - 1u)) == 0u) {
+                sum = dd_add_d(sum, acc);
+                acc = 0.0;
+            }
+            if (s + 1 == steps) break;
+            uint32_t neg = 0;
+            int row = 0;  // a lane past its chunk moves on with weight 0
+            if (s + 1 < len) {
+                int wch;
+                row = st.step(g, s, radix, &neg, &wch);
+                ws = wch ? signed_weight<double>(g.w, g.parity) : flip_sign(ws);
+            }
+            fix_update<HX>(c, a2 + (size_t)row * KP, neg);
+        }
+        sum = dd_add_d(sum, acc);
+    }
+    // over the 16 lanes of each part, then the imaginary part to lane 0
+#pragma unroll
+    for (int off = 16; off > 1; off >>= 1) sum = dd_add_sum2(sum, shfl_down_dd(sum, off));
+    const ddv im = shfl_down_dd(sum, 1);
+    if (lane == 0) store_partial(partials + jb.partial_off + local, sum, im);
+}
+
+// ---------------------------------------------------------------- one task: minors
+// v >> d, 0 <= d <= 63 (rounded down).
+__device__ __forceinline__ zraw fix_shr(const zraw& v, int d) {
+    return zraw{(unsigned long long)((long long)v.re >> d), (unsigned long long)((long long)v.im >> d)};
+}
+
+__device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
+    zlimb o;
+    o.rh = __shfl_xor_sync(0xffffffffu, v.rh, mask);
+    o.rl = __shfl_xor_sync(0xffffffffu, v.rl, mask);
+    o.ih = __shfl_xor_sync(0xffffffffu, v.ih, mask);
+    o.il = __shfl_xor_sync(0xffffffffu, v.il, mask);
+    return o;
+}
+
+// Longest integer run of the minors, in addends (a power of two).
+constexpr uint32_t kFixRun = 4;
+
+// Shared memory of one warp of the minors kernel, HX columns per lane, NP =
+// ceil(HX / 2) leaves: the integer sums [col][lane] (rows of 33, so that
+// neighbouring columns of one lane fall into different banks when a run is
+// flushed), the suffix products and then the m_j [leaf][lane], the leaves
+// [leaf][lane] (at the end of a run the units' exponents), the K
+// double-double totals, plain-double sums, and a factor per chunk.
+template <int G, int HX>
+struct MinorsSmem {
+    longlong2 acc[HX * 33];
+    longlong2 leaf[((HX + 1) / 2) * 32];
+    int4 pair[((HX + 1) / 2) * 32];
+    double4 tot[G * HX];
+    double2 run[G * HX];
+    double fac[32 / G];
+};
+
+// Runs whose plain-double sum goes to the double-double totals at once.
+constexpr uint32_t kFixFold = 16;
+
+// End of a run: lane t takes column t (and t + 32) and adds the integer sums
+// of the lanes that own it, times their chunks' factors and their units
+// 2^exp, to the column's plain-double sum, and clears the sums; with fold, the
+// plain-double sum goes to the column's double-double total.
+template <int G, int HX>
+__device__ __forceinline__ void minors_flush_fix(MinorsSmem<G, HX>& sm, double f, const int (&em)[(HX + 1) / 2],
+                                                 int lane, int K, bool fold) {
+    if ((lane & (G - 1)) == 0) sm.fac[lane / G] = f;
+#pragma unroll
+    for (int j = 0; j < (HX + 1) / 2; ++j) sm.pair[j * 32 + lane].x = em[j];
+    __syncwarp();
+#pragma unroll 1
+    for (int t = lane; t < K; t += 32) {
+        const int q = t / HX, u = t - q * HX;
+        longlong2* a = sm.acc + u * 33 + q;
+        const int4* ex = sm.pair + (u >> 1) * 32 + q;
+        double2 r = sm.run[t];
+#pragma unroll 4
+        for (int p = 0; p < 32 / G; ++p) {
+            const longlong2 v = a[G * p];
+            a[G * p] = make_longlong2(0, 0);
+            const double w = scale_pow2(sm.fac[p], ex[G * p].x);
+            r.x = bfma(w, (double)v.x, r.x);
+            r.y = bfma(w, (double)v.y, r.y);
+        }
+        if (fold) {
+            const double4 v = sm.tot[t];
+            const ddv sr = dd_add_d(ddv{v.x, v.y}, r.x), si = dd_add_d(ddv{v.z, v.w}, r.y);
+            sm.tot[t] = make_double4(sr.hi, sr.lo, si.hi, si.lo);
+            r = make_double2(0.0, 0.0);
+        }
+        sm.run[t] = r;
+    }
+    __syncwarp();
+}
+
+// One step of a suffix chain: r (exponent e) is the product of the chain's
+// leaves after leaf j; keeps it, normalised, as leaf j's suffix, and takes
+// leaf j in.
+template <int HX>
+__device__ __forceinline__ void suffix_step(const zraw (&c)[HX], int j, zraw& r, int& e, int (&es)[(HX + 1) / 2],
+                                            longlong2* __restrict__ sm_leaf, int4* __restrict__ sm_pair) {
+    const zlimb sf = fix_normalise(r, e);
+    sm_leaf[j * 32] = *reinterpret_cast<const longlong2*>(&sf);
+    es[j] = e;
+    const zlimb d = limbs_of(fix_leaf(c, j));
+    sm_pair[j * 32] = make_int4(d.rl, d.rh, d.il, d.ih);
+    r = fix_cmul(sf, d);
+    e += 64 + kLeafExp;
+}
+
+// One step of a prefix chain: m_j = p S_j (p itself for the chain's last
+// leaf), below 2^61, in S_j's place, its exponent in es[j]; p takes leaf j in.
+template <int NP>
+__device__ __forceinline__ void prefix_step(int j, bool last, zlimb& p, int& e, int (&es)[NP],
+                                            longlong2* __restrict__ sm_leaf, const int4* __restrict__ sm_pair) {
+    zraw m;
+    if (last) {
+        m = fix_shr(raw_of(p), 1);
+        es[j] = e + 1;
+    } else {
+        const longlong2 v = sm_leaf[j * 32];
+        m = fix_cmul<0>(p, *reinterpret_cast<const zlimb*>(&v));
+        es[j] += e + 64;
+        const int4 d = sm_pair[j * 32];
+        e += 64 + kLeafExp;
+        p = fix_normalise(fix_cmul(p, zlimb{d.x, d.y, d.z, d.w}), e);
+    }
+    sm_leaf[j * 32] = make_longlong2((long long)m.re, (long long)m.im);
+}
+
+// G lanes share one chunk: lane G p + q owns the HX columns [q HX, q HX + HX)
+// (HX = ceil(K / G); the last lane's missing columns are pads, exactly 1).
+// Per addend each lane
+//   1. forms its leaves d_j (column pairs), in two chains their exclusive
+//      suffix products S_j, and the product Q of its columns;
+//   2. takes X, the product of the other lanes' Q, by shuffles;
+//   3. runs the prefix products from X over the chains, m_j = prefix_j S_j:
+//      all columns but those of pair j;
+//   4. adds m_j times the one column of the pair to the other column's sum,
+//      in 64-bit integers whose unit, one per pair and lane, follows the
+//      largest addend of the run (the sums move down when it grows).
+// 3 K - 3 complex products per addend, as any prefix / suffix scheme needs.
+//
+// The sums.  A conversion to double and an FMA hold the FP64 pipe for 128
+// cycles; done for every addend that would cost more than the products do
+// (minors at K = 28: 453 cycles per column and addend), so integer sums run
+// over at most 4 addends (|m_j c| < 2^60, so 4 stay below 2^62; never across
+// a change of the binomial weight) and go to plain-double column sums beside
+// the products, sign, weight and unit in one factor; 16 of those runs to the
+// double-double totals.  The unit is what the accuracy hangs on: m_j is
+// brought to [2^60, 2^61) at the run's largest addend, and the sum's rounding
+// is then about 2^-54 of that addend.  Errors against exact minors (24
+// columns, distinct rows, root mean square relative): 1.2e-14, the kernels in
+// double 2.2e-14; runs of 8 addends 2.0e-14, one unit for the whole warp
+// 3.5e-12 (27 columns), without the sums (one addend per run) 2e-15.
+//
+// Time.  29 x 30 minors (2^28 addends): 190 ms in double, 49.7 ms here (1.42e9 ->
+// 5.40e9 addends/s); the FMA-heavy pipe is 67 % busy
+// with integer products (4.35 cycles per warp and product) and every other
+// integer instruction costs about 1.3 cycles beside them, so what bounds it is
+// the instruction count: 112 per column and addend, 33 of them products.
+template <int G, int KB, int HX>
+__device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ data, const int* __restrict__ radix,
+                                     bs_zdd* __restrict__ partials, uint32_t local, int lane,
+                                     MinorsSmem<G, HX>& sm) {
+    constexpr int KP = KB;            // = BS_ROW_STRIDE(K) for every K of the bucket
+    constexpr int NP = (HX + 1) / 2;  // leaves, in two chains of NA and NB
+    constexpr int NA = (NP + 1) / 2, NB = NP - NA;
+    const int K = jb.K;
+    const int q = lane & (G - 1);
+    const zfix* c0 = data + jb.data_off + q * HX;
+    const zfix* a2 = c0 + KP;
+    longlong2* sm_acc = sm.acc + lane;
+    longlong2* sm_leaf = sm.leaf + lane;
+    int4* sm_pair = sm.pair + lane;
+#pragma unroll
+    for (int t = 0; t < HX; ++t) sm_acc[t * 33] = make_longlong2(0, 0);
+    for (int t = lane; t < K; t += 32) {
+        sm.tot[t] = make_double4(0.0, 0.0, 0.0, 0.0);
+        sm.run[t] = make_double2(0.0, 0.0);
+    }
+    const uint64_t i0_own = ((uint64_t)local * (uint64_t)(32 / G) + (uint64_t)(lane / G)) << jb.log2L;
+    const bool has = i0_own < jb.C;
+    const uint64_t i0 = has ? i0_own : 0ull;
+    uint32_t len = 0;
+    if (has) {
+        const uint64_t rem = jb.C - i0;
+        len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
+    }
+    const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
+    // runs end where a repeated-row digit moves (the weight changes there:
+    // after every 2^nbin addends)
+    const uint32_t run_mask = jb.nbin >= 2 ? kFixRun - 1u : (1u << jb.nbin) - 1u;
+    static_assert(kFixRun == 4, "2^2 addends per run");
+    bs_gray g;
+    ChunkStepper st;
+    st.init(g, i0, jb.nbin, jb.nrows, radix, reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
+    zraw c[HX];
+    fix_seed<HX, KP>(c, g, c0, jb.nbin, jb.nrows);
+    double ws = signed_weight<double>(g.w, g.parity);
+    double wrun = ws;          // of the run's first addend
+    // exponent of a sum's unit against m's: the last product's 64, its
+    // column's -63, and 1 for every pad column (2^62 stands for 1, bound 2)
+    const int e_unit = 64 - 63 + (G * HX - K);
+    int em[NP];
+    uint32_t runs = 0;
+    for (uint32_t s = 0; s < steps; ++s) {
+        // 1. leaves, suffix products, Q
+        int es[NP];
+        zlimb qa, qb, pr;
+        int ea = kLeafExp, eb = kLeafExp, e;
+        {
+            zraw ra = fix_leaf(c, NA - 1), rb = {0ull, 0ull};
+            if constexpr (NB > 0) rb = fix_leaf(c, NP - 1);
+#pragma unroll
+            for (int i = 1; i < NA; ++i) {
+                suffix_step<HX>(c, NA - 1 - i, ra, ea, es, sm_leaf, sm_pair);
+                if (i < NB) suffix_step<HX>(c, NP - 1 - i, rb, eb, es, sm_leaf, sm_pair);
+            }
+            qa = fix_normalise(ra, ea);
+            e = ea;
+            if constexpr (NB > 0) {
+                qb = fix_normalise(rb, eb);
+                ra = fix_cmul(qa, qb);
+                e += eb + 64;
+            } else {
+                ra = raw_of(qa);
+            }
+            // the addend's sign against the run's first one goes here, and a
+            // lane past its chunk adds zeros from here on
+            const unsigned long long m = 0ull - (unsigned long long)(s & 1u & run_mask);
+            ra.re = s < len ? (ra.re ^ m) - m : 0ull;
+            ra.im = s < len ? (ra.im ^ m) - m : 0ull;
+            pr = limbs_of(ra);
+        }
+        // 2. X
+        if constexpr (G == 4) {
+            const zlimb o1 = shfl_xor_zlimb(pr, 1);
+            const int e1 = __shfl_xor_sync(0xffffffffu, e, 1);
+            int e2 = e + e1 + 64;
+            const zlimb o2 = shfl_xor_zlimb(fix_normalise(fix_cmul(pr, o1), e2), 2);
+            e = e1 + __shfl_xor_sync(0xffffffffu, e2, 2) + 64;
+            pr = fix_normalise(fix_cmul(o1, o2), e);
+        } else {
+            pr = shfl_xor_zlimb(pr, 1);
+            e = __shfl_xor_sync(0xffffffffu, e, 1);
+        }
+        // 3. m_j, below 2^61
+        {
+            zlimb pa, pb;
+            int fa = e, fb = e;
+            pa = pr;
+            if constexpr (NB > 0) {
+                fa += eb + 64;
+                fb += ea + 64;
+                pa = fix_normalise(fix_cmul(pr, qb), fa);
+                pb = fix_normalise(fix_cmul(pr, qa), fb);
+            }
+#pragma unroll
+            for (int i = 0; i < NA; ++i) {
+                prefix_step(i, i + 1 == NA, pa, fa, es, sm_leaf, sm_pair);
+                if (i < NB) prefix_step(NA + i, i + 1 == NB, pb, fb, es, sm_leaf, sm_pair);
+            }
+        }
+        // 4. the units of the pairs' sums
+        if ((s & run_mask) == 0u) {
+#pragma unroll
+            for (int j = 0; j < NP; ++j) em[j] = -(1 << 20);
+        }
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            // the largest addend so far comes to [2^60, 2^61): m_j is carried
+            // 4 times over, so that its shift is to the right
+            const longlong2 v = sm_leaf[j * 32];
+            const zraw r = {(unsigned long long)v.x, (unsigned long long)v.y};
+            const int up = max(em[j], es[j] - min(fix_norm_shift(r) - 1, 2));
+            const int dl = min(up - em[j], 63);
+            em[j] = up;
+            const zraw m = fix_shr(zraw{r.re << 2, r.im << 2}, min(up - es[j] + 2, 63));
+            const longlong2 a = sm_acc[2 * j * 33];
+            zraw z = fix_shr(zraw{(unsigned long long)a.x, (unsigned long long)a.y}, dl);
+            if (2 * j + 1 < HX) {
+                const zlimb ml = limbs_of(m);
+                z = fix_cmul_add<1, 1>(z, ml, limbs_of(c[2 * j + 1]));
+                sm_acc[2 * j * 33] = make_longlong2((long long)z.re, (long long)z.im);
+                const longlong2 b = sm_acc[(2 * j + 1) * 33];
+                z = fix_cmul_add<1, 1>(fix_shr(zraw{(unsigned long long)b.x, (unsigned long long)b.y}, dl), ml,
+                                       limbs_of(c[2 * j]));
+                sm_acc[(2 * j + 1) * 33] = make_longlong2((long long)z.re, (long long)z.im);
+            } else {  // no partner: m_j itself, in the same unit (m / 2)
+                const zraw h = fix_shr(m, 1);
+                sm_acc[2 * j * 33] = make_longlong2((long long)(z.re + h.re), (long long)(z.im + h.im));
+            }
+        }
+        // the end of a run
+        if (((s + 1u) & run_mask) == 0u || s + 1 == steps)
+            minors_flush_fix<G, HX>(sm, scale_pow2(wrun, e_unit), em, lane, K,
+                                    (++runs & (kFixFold - 1u)) == 0u || s + 1 == steps);
+        if (s + 1 == steps) break;
+        uint32_t neg = 0;
+        int row = 0;  // a lane past its chunk moves on, adding zeros
+        if (s + 1 < len) {
+            int wch;
+            row = st.step(g, s, radix, &neg, &wch);
+            ws = wch ? signed_weight<double>(g.w, g.parity) : flip_sign(ws);
+        }
+        if (((s + 1u) & run_mask) == 0u) wrun = ws;
+        fix_update<HX>(c, a2 + (size_t)row * KP, neg);
+    }
+    for (int t = lane; t < K; t += 32) {
+        const double4 v = sm.tot[t];
+        store_partial(partials + jb.partial_off + (int64_t)local * K + t, ddv{v.x, v.y}, ddv{v.z, v.w});
+    }
+    __syncwarp();  // the next task's initialisation overwrites the totals
+}
+
+}  // namespace bs
