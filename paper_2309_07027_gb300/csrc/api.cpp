@@ -808,27 +808,35 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
     // the kernels a chain may be given (bs_choose_log2L gives at most
     // 2 x target tasks unless the chunk length is capped, and then at most
     // C / (cpt 2^log2max) + 1; cpt >= 16 for FP64 minors, 8 for FP32, 4 for DF)
-    uint64_t cmax = n >= 2 ? (1ull << (n - 2)) : 1ull;
-    uint64_t tasks_stride = 2 * BS_TARGET_TASKS_MANY + 1;
-    {
-        int precs[2];
-        const int np = sampler_precs(mode, precs);
-        for (int pi = 0; pi < np; ++pi) {
-            const uint64_t cpt_min = precs[pi] == BS_PREC_FP64 ? 8 : precs[pi] == BS_PREC_FP32 ? 8 : 4;
-            tasks_stride = std::max<uint64_t>(tasks_stride, cmax / (cpt_min << c->log2max[precs[pi]]) + 2);
-        }
-    }
     // a step-k job has <= k - 1 digit rows, K = k <= n columns, n' = k - 1;
     // a chain's data slot fits the widest row stride (DF: multiples of 8)
+    const uint64_t cmax = n >= 2 ? (1ull << (n - 2)) : 1ull;
     const int64_t meta_stride = BS_META_SIZE(n, n, n), data_stride = (int64_t)n * BS_ROW_STRIDE_DF(n);
+    int precs[2];
+    const int np = sampler_precs(mode, precs);
+    auto stride_for = [&](int target) {
+        uint64_t t = 2 * (uint64_t)target + 1;
+        for (int pi = 0; pi < np; ++pi) {
+            const uint64_t cpt_min = precs[pi] == BS_PREC_FP64 ? 16 : precs[pi] == BS_PREC_FP32 ? 8 : 4;
+            t = std::max<uint64_t>(t, cmax / (cpt_min << c->log2max[precs[pi]]) + 2);
+        }
+        return t;
+    };
+    auto chain_bytes = [&](uint64_t stride) {
+        return (size_t)stride * n * sizeof(bs_zdd) + (size_t)data_stride * 16 + meta_stride * 4 + sizeof(bs_job) +
+               (size_t)n * (8 + 16) + 8 + 64;
+    };
     // chains per pass: bounded by the budget (or 2 GiB of partials per pass)
-    const size_t per_chain = (size_t)tasks_stride * n * sizeof(bs_zdd) + (size_t)data_stride * 16 +
-                             meta_stride * 4 + sizeof(bs_job) + (size_t)n * (8 + 16) + 8 + 64;
     size_t cap_bytes = (size_t)2 << 30;
     if (c->budget) {
         size_t free_b = c->budget > c->used ? c->budget - c->used : 0;
         cap_bytes = std::min(cap_bytes, free_b / 2 + c->cc_partials.n);
     }
+    // few chains: more tasks per job, where their partials fit in one pass
+    int target = bs_target_chains(n_samples);
+    if (chain_bytes(stride_for(target)) * (size_t)n_samples > cap_bytes) target = BS_TARGET_TASKS_MANY;
+    const uint64_t tasks_stride = stride_for(target);
+    const size_t per_chain = chain_bytes(tasks_stride);
     int S_max = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_samples, cap_bytes / per_chain));
     int rc;
     const int S0 = std::min(S_max, n_samples);
@@ -887,6 +895,7 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
         a.log2max64 = c->log2max[BS_PREC_FP64];
         a.log2max32 = c->log2max[BS_PREC_FP32];
         a.log2maxdf = c->log2max[BS_PREC_DF];
+        a.target = target;
         a.mixed_log2_tol = c->mixed_log2_tol;
         a.mixed_fallback = kMixedFallback;
         // the kernels read the arguments from device memory (pageable copy:

@@ -24,6 +24,16 @@
 // about half the rows (4096-item batch: 3.6 % faster than with 32768).
 #define BS_TARGET_TASKS_SINGLE_FP32 8192
 #define BS_TARGET_TASKS_MANY 64
+// FP64 and double-float jobs of a sampler call with few chains aim at more
+// tasks, so that the call fills the GPU (about 8192 tasks in all, several per
+// resident warp): 40 chains at 64 tasks each are 1.4 tasks per resident warp,
+// and a call of one chain leaves 9 of 10 schedulers idle.  Served jobs, which
+// know nothing of their company, aim at 512.  Neither form drifts inside a
+// chunk (exact column sums), so shorter chunks cost only their seeding.  FP32
+// jobs keep 64: their chunk length is part of the MIXED rule.
+#define BS_TARGET_TASKS_ALL 8192
+#define BS_TARGET_TASKS_MAX 1024
+#define BS_TARGET_TASKS_SERVED 512
 #define BS_LOG2L_MIN_SINGLE 6
 #define BS_LOG2L_MIN_MANY 3
 // Floor for the tiniest jobs planned alone (at most BS_FILL_TINY_C
@@ -60,6 +70,12 @@ BS_HD int bs_choose_log2L(uint64_t C, int cpt, int log2min, int log2max, int tar
     if (l > log2max) l = log2max;
     return l;
 }
+// Task target of an FP64 or double-float job in a sampler call of S chains.
+BS_HD int bs_target_chains(int64_t S) {
+    int t = BS_TARGET_TASKS_MANY;
+    while (t < BS_TARGET_TASKS_MAX && (int64_t)t * S < BS_TARGET_TASKS_ALL) t *= 2;
+    return t;
+}
 // The rule for jobs planned one call at a time: bs_choose_log2L with the
 // single-call target and floor 2^6, except that a job too small to give
 // BS_TARGET_TASKS_FILL tasks at that floor gets shorter chunks (down to 2^3,
@@ -91,7 +107,9 @@ BS_HD int bs_choose_log2L_single(uint64_t C, int cpt, int log2max, int target) {
 // the permanent kernels give each lane its own chunk (32 per task).
 #define BS_MINORS_FP32_GROUP_KB(KB) (((KB) == 24 || (KB) == 48) ? 4 : 2)
 BS_HD int bs_minors_fp32_group(int K) { return BS_MINORS_FP32_GROUP_KB((K + 3) & ~3); }
-// Lanes per chunk of the FP64 fused minors, by 4-column bucket width.
+// Lanes per chunk of the FP64 fused minors, by 4-column bucket width (above
+// 32 columns two lanes need 255 registers and run 7-24 % slower than four).
+// A warp task covers 16 chunks either way, in one or two rounds.
 #define BS_MINORS_FP64_GROUP_KB(KB) ((KB) > 32 ? 4 : 2)
 // Lanes per chunk of the double-float kernels (permanent and minors), by
 // 8-column bucket width KB: each lane owns KB / (2G) column pairs
@@ -102,7 +120,7 @@ BS_HD int bs_df_group(int K) { return BS_DF_GROUP_KB((K + 7) & ~7); }
 BS_HD int bs_chunks_per_task(int kind, int prec, int K) {
     if (prec == BS_PREC_DF) return 32 / bs_df_group(K);
     if (kind != BS_KIND_MINORS) return 32;
-    return 32 / (prec == BS_PREC_FP32 ? bs_minors_fp32_group(K) : BS_MINORS_FP64_GROUP_KB((K + 3) & ~3));
+    return prec == BS_PREC_FP32 ? 32 / bs_minors_fp32_group(K) : 16;  // FP64 minors
 }
 
 // Algorithmic flops of one addend (the roofline numerator):
@@ -247,6 +265,7 @@ struct StepRule {
     float mixed_log2_tol;
     int mixed_fallback;
     int log2max[BS_NPREC];
+    int target;  // task target of FP64 and double-float jobs
 };
 
 struct CcArgs {
@@ -276,6 +295,7 @@ struct CcArgs {
     float mixed_log2_tol;         // the rule's threshold, log2 of the MIXED tolerance
     int mixed_fallback;           // MIXED: precision of the jobs that fail the rule
     int log2max64, log2max32, log2maxdf;
+    int target;                   // task target of FP64 and double-float jobs
 };
 
 // One served Clifford & Clifford chain (one sample) resident in a server's

@@ -126,6 +126,7 @@ struct Request {
     std::vector<int> counts;           // result: m_det occupation counts
     bs_job job_host{};                 // the pending step's job, as planned on the device
     uint64_t tasks_stride = 0;         // task partial slots per step
+    int target = BS_TARGET_TASKS_MANY; // task target of its FP64 and double-float steps
     // byte offsets of the chain's regions inside its arena block
     size_t c_u = 0, c_in = 0, c_cols = 0, c_rows = 0, c_cnt = 0, c_job = 0, c_meta = 0, c_data = 0, c_part = 0;
 };
@@ -215,6 +216,11 @@ size_t request_bytes(const Request& r) {
     b += up((size_t)r.ntasks * r.ncols * sizeof(bs_zdd));            // task partials
     return b;
 }
+
+// Whether requests of this size could fill every slot at once: only then does
+// a request take the larger task target, so that no budget holds fewer
+// requests than it would with the smaller one.
+bool fits_slot(const bs_server* s, size_t bytes) { return bytes <= s->budget / (size_t)s->max_active; }
 
 void finish(bs_server* s, Request* r, int status) {
     r->status = status;
@@ -405,6 +411,7 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
         d.rule.mixed_log2_tol = BS_MIXED_LOG2_TOL_DEFAULT;
         d.rule.mixed_fallback = BS_MIXED_FALLBACK_PREC;
         for (int q = 0; q < BS_NPREC; ++q) d.rule.log2max[q] = bs_default_log2max(q);
+        d.rule.target = r->target;
         descs.push_back(d);
         max_m_rows = std::max(max_m_rows, r->m_rows);
         back_bytes += r->k < r->n ? sizeof(bs_job) : (size_t)r->m_det * 4;
@@ -733,11 +740,14 @@ int64_t bs_server_submit(bs_server* s, int kind, const bs_c128* A, int rows, int
         r->reseed = plan == 2 ? BS_FP32_RESEED_LOG2 : 0;
     }
     r->cpt = bs_chunks_per_task(r->kind, r->prec, r->plan.K);
-    r->log2L = bs_choose_log2L(r->plan.C, r->cpt, BS_LOG2L_MIN_MANY, bs_default_log2max(r->prec), BS_TARGET_TASKS_MANY);
-    const uint64_t per = (uint64_t)r->cpt << r->log2L;
-    r->ntasks = (uint32_t)((r->plan.C + per - 1) / per);
     r->ncols = r->kind == BS_KIND_PERM ? 1 : r->plan.K;
-    r->bytes = request_bytes(*r);
+    for (int target : {r->prec == BS_PREC_FP32 ? BS_TARGET_TASKS_MANY : BS_TARGET_TASKS_SERVED, BS_TARGET_TASKS_MANY}) {
+        r->log2L = bs_choose_log2L(r->plan.C, r->cpt, BS_LOG2L_MIN_MANY, bs_default_log2max(r->prec), target);
+        const uint64_t per = (uint64_t)r->cpt << r->log2L;
+        r->ntasks = (uint32_t)((r->plan.C + per - 1) / per);
+        r->bytes = request_bytes(*r);
+        if (fits_slot(s, r->bytes)) break;
+    }
     s->waiting.push_back(r);
     s->cv_work.notify_one();
     return r->id;
@@ -830,17 +840,21 @@ int64_t bs_server_submit_sample(bs_server* s, const bs_c128* U, int m_rows, int 
         // task partial slots of the largest step (C <= 2^(n-2)) over the
         // kernels the mode may use (chunks per task >= 16 FP64, 8 FP32, 4 DF)
         const uint64_t cmax = r->n >= 2 ? (1ull << (r->n - 2)) : 1ull;
-        uint64_t ts = 2 * BS_TARGET_TASKS_MANY + 1;
         const int precs_mixed[2] = {BS_PREC_FP32, BS_MIXED_FALLBACK_PREC};
         const int prec_one = s->mode == BS_DF64 ? BS_PREC_DF : BS_PREC_FP64;
         const int np = s->mode == BS_MIXED ? 2 : 1;
-        for (int i = 0; i < np; ++i) {
-            const int q = s->mode == BS_MIXED ? precs_mixed[i] : prec_one;
-            const uint64_t cpt_min = q == BS_PREC_FP64 ? 8 : q == BS_PREC_FP32 ? 8 : 4;
-            ts = std::max<uint64_t>(ts, cmax / (cpt_min << bs_default_log2max(q)) + 2);
+        for (int target : {BS_TARGET_TASKS_SERVED, BS_TARGET_TASKS_MANY}) {
+            uint64_t ts = 2 * (uint64_t)target + 1;
+            for (int i = 0; i < np; ++i) {
+                const int q = s->mode == BS_MIXED ? precs_mixed[i] : prec_one;
+                const uint64_t cpt_min = q == BS_PREC_FP64 ? 16 : q == BS_PREC_FP32 ? 8 : 4;
+                ts = std::max<uint64_t>(ts, cmax / (cpt_min << bs_default_log2max(q)) + 2);
+            }
+            r->target = target;
+            r->tasks_stride = ts;
+            r->bytes = chain_layout(*r);
+            if (fits_slot(s, r->bytes)) break;
         }
-        r->tasks_stride = ts;
-        r->bytes = chain_layout(*r);
     }
     std::lock_guard<std::mutex> lk(s->mu);
     r->id = s->next_id++;

@@ -441,6 +441,7 @@ __device__ __forceinline__ void prefix_step(int j, bool last, zlimb& p, int& e, 
 //      in 64-bit integers whose unit, one per pair and lane, follows the
 //      largest addend of the run (the sums move down when it grows).
 // 3 K - 3 complex products per addend, as any prefix / suffix scheme needs.
+// A task covers 16 chunks, with four lanes per chunk in two rounds.
 //
 // The sums.  A conversion to double and an FMA hold the FP64 pipe for 128
 // cycles; done for every addend that would cost more than the products do
@@ -480,133 +481,136 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
         sm.tot[t] = make_double4(0.0, 0.0, 0.0, 0.0);
         sm.run[t] = make_double2(0.0, 0.0);
     }
-    const uint64_t i0_own = ((uint64_t)local * (uint64_t)(32 / G) + (uint64_t)(lane / G)) << jb.log2L;
-    const bool has = i0_own < jb.C;
-    const uint64_t i0 = has ? i0_own : 0ull;
-    uint32_t len = 0;
-    if (has) {
-        const uint64_t rem = jb.C - i0;
-        len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
-    }
-    const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
-    // runs end where a repeated-row digit moves (the weight changes there:
-    // after every 2^nbin addends)
-    const uint32_t run_mask = jb.nbin >= 2 ? kFixRun - 1u : (1u << jb.nbin) - 1u;
-    static_assert(kFixRun == 4, "2^2 addends per run");
-    bs_gray g;
-    ChunkStepper st;
-    st.init(g, i0, jb.nbin, jb.nrows, radix, reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
-    zraw c[HX];
-    fix_seed<HX, KP>(c, g, c0, jb.nbin, jb.nrows);
-    double ws = signed_weight<double>(g.w, g.parity);
-    double wrun = ws;          // of the run's first addend
-    // exponent of a sum's unit against m's: the last product's 64, its
-    // column's -63, and 1 for every pad column (2^62 stands for 1, bound 2)
-    const int e_unit = 64 - 63 + (G * HX - K);
-    int em[NP];
-    uint32_t runs = 0;
-    for (uint32_t s = 0; s < steps; ++s) {
-        // 1. leaves, suffix products, Q
-        int es[NP];
-        zlimb qa, qb, pr;
-        int ea = kLeafExp, eb = kLeafExp, e;
-        {
-            zraw ra = fix_leaf(c, NA - 1), rb = {0ull, 0ull};
-            if constexpr (NB > 0) rb = fix_leaf(c, NP - 1);
+    for (int round = 0; round < G / 2; ++round) {
+        const uint64_t i0_own = ((uint64_t)local * 16u + (uint64_t)(round * (32 / G) + lane / G)) << jb.log2L;
+        const bool has = i0_own < jb.C;
+        const uint64_t i0 = has ? i0_own : 0ull;
+        uint32_t len = 0;
+        if (has) {
+            const uint64_t rem = jb.C - i0;
+            len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
+        }
+        const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
+        if (steps == 0u) break;
+        // runs end where a repeated-row digit moves (the weight changes there:
+        // after every 2^nbin addends)
+        const uint32_t run_mask = jb.nbin >= 2 ? kFixRun - 1u : (1u << jb.nbin) - 1u;
+        static_assert(kFixRun == 4, "2^2 addends per run");
+        bs_gray g;
+        ChunkStepper st;
+        st.init(g, i0, jb.nbin, jb.nrows, radix, reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
+        zraw c[HX];
+        fix_seed<HX, KP>(c, g, c0, jb.nbin, jb.nrows);
+        double ws = signed_weight<double>(g.w, g.parity);
+        double wrun = ws;          // of the run's first addend
+        // exponent of a sum's unit against m's: the last product's 64, its
+        // column's -63, and 1 for every pad column (2^62 stands for 1, bound 2)
+        const int e_unit = 64 - 63 + (G * HX - K);
+        int em[NP];
+        uint32_t runs = 0;
+        for (uint32_t s = 0; s < steps; ++s) {
+            // 1. leaves, suffix products, Q
+            int es[NP];
+            zlimb qa, qb, pr;
+            int ea = kLeafExp, eb = kLeafExp, e;
+            {
+                zraw ra = fix_leaf(c, NA - 1), rb = {0ull, 0ull};
+                if constexpr (NB > 0) rb = fix_leaf(c, NP - 1);
 #pragma unroll
-            for (int i = 1; i < NA; ++i) {
-                suffix_step<HX>(c, NA - 1 - i, ra, ea, es, sm_leaf, sm_pair);
-                if (i < NB) suffix_step<HX>(c, NP - 1 - i, rb, eb, es, sm_leaf, sm_pair);
+                for (int i = 1; i < NA; ++i) {
+                    suffix_step<HX>(c, NA - 1 - i, ra, ea, es, sm_leaf, sm_pair);
+                    if (i < NB) suffix_step<HX>(c, NP - 1 - i, rb, eb, es, sm_leaf, sm_pair);
+                }
+                qa = fix_normalise(ra, ea);
+                e = ea;
+                if constexpr (NB > 0) {
+                    qb = fix_normalise(rb, eb);
+                    ra = fix_cmul(qa, qb);
+                    e += eb + 64;
+                } else {
+                    ra = raw_of(qa);
+                }
+                // the addend's sign against the run's first one goes here, and a
+                // lane past its chunk adds zeros from here on
+                const unsigned long long m = 0ull - (unsigned long long)(s & 1u & run_mask);
+                ra.re = s < len ? (ra.re ^ m) - m : 0ull;
+                ra.im = s < len ? (ra.im ^ m) - m : 0ull;
+                pr = limbs_of(ra);
             }
-            qa = fix_normalise(ra, ea);
-            e = ea;
-            if constexpr (NB > 0) {
-                qb = fix_normalise(rb, eb);
-                ra = fix_cmul(qa, qb);
-                e += eb + 64;
+            // 2. X
+            if constexpr (G == 4) {
+                const zlimb o1 = shfl_xor_zlimb(pr, 1);
+                const int e1 = __shfl_xor_sync(0xffffffffu, e, 1);
+                int e2 = e + e1 + 64;
+                const zlimb o2 = shfl_xor_zlimb(fix_normalise(fix_cmul(pr, o1), e2), 2);
+                e = e1 + __shfl_xor_sync(0xffffffffu, e2, 2) + 64;
+                pr = fix_normalise(fix_cmul(o1, o2), e);
             } else {
-                ra = raw_of(qa);
+                pr = shfl_xor_zlimb(pr, 1);
+                e = __shfl_xor_sync(0xffffffffu, e, 1);
             }
-            // the addend's sign against the run's first one goes here, and a
-            // lane past its chunk adds zeros from here on
-            const unsigned long long m = 0ull - (unsigned long long)(s & 1u & run_mask);
-            ra.re = s < len ? (ra.re ^ m) - m : 0ull;
-            ra.im = s < len ? (ra.im ^ m) - m : 0ull;
-            pr = limbs_of(ra);
-        }
-        // 2. X
-        if constexpr (G == 4) {
-            const zlimb o1 = shfl_xor_zlimb(pr, 1);
-            const int e1 = __shfl_xor_sync(0xffffffffu, e, 1);
-            int e2 = e + e1 + 64;
-            const zlimb o2 = shfl_xor_zlimb(fix_normalise(fix_cmul(pr, o1), e2), 2);
-            e = e1 + __shfl_xor_sync(0xffffffffu, e2, 2) + 64;
-            pr = fix_normalise(fix_cmul(o1, o2), e);
-        } else {
-            pr = shfl_xor_zlimb(pr, 1);
-            e = __shfl_xor_sync(0xffffffffu, e, 1);
-        }
-        // 3. m_j, below 2^61
-        {
-            zlimb pa, pb;
-            int fa = e, fb = e;
-            pa = pr;
-            if constexpr (NB > 0) {
-                fa += eb + 64;
-                fb += ea + 64;
-                pa = fix_normalise(fix_cmul(pr, qb), fa);
-                pb = fix_normalise(fix_cmul(pr, qa), fb);
+            // 3. m_j, below 2^61
+            {
+                zlimb pa, pb;
+                int fa = e, fb = e;
+                pa = pr;
+                if constexpr (NB > 0) {
+                    fa += eb + 64;
+                    fb += ea + 64;
+                    pa = fix_normalise(fix_cmul(pr, qb), fa);
+                    pb = fix_normalise(fix_cmul(pr, qa), fb);
+                }
+#pragma unroll
+                for (int i = 0; i < NA; ++i) {
+                    prefix_step(i, i + 1 == NA, pa, fa, es, sm_leaf, sm_pair);
+                    if (i < NB) prefix_step(NA + i, i + 1 == NB, pb, fb, es, sm_leaf, sm_pair);
+                }
+            }
+            // 4. the units of the pairs' sums
+            if ((s & run_mask) == 0u) {
+#pragma unroll
+                for (int j = 0; j < NP; ++j) em[j] = -(1 << 20);
             }
 #pragma unroll
-            for (int i = 0; i < NA; ++i) {
-                prefix_step(i, i + 1 == NA, pa, fa, es, sm_leaf, sm_pair);
-                if (i < NB) prefix_step(NA + i, i + 1 == NB, pb, fb, es, sm_leaf, sm_pair);
+            for (int j = 0; j < NP; ++j) {
+                // the largest addend so far comes to [2^60, 2^61): m_j is carried
+                // 4 times over, so that its shift is to the right
+                const longlong2 v = sm_leaf[j * 32];
+                const zraw r = {(unsigned long long)v.x, (unsigned long long)v.y};
+                const int up = max(em[j], es[j] - min(fix_norm_shift(r) - 1, 2));
+                const int dl = min(up - em[j], 63);
+                em[j] = up;
+                const zraw m = fix_shr(zraw{r.re << 2, r.im << 2}, min(up - es[j] + 2, 63));
+                const longlong2 a = sm_acc[2 * j * 33];
+                zraw z = fix_shr(zraw{(unsigned long long)a.x, (unsigned long long)a.y}, dl);
+                if (2 * j + 1 < HX) {
+                    const zlimb ml = limbs_of(m);
+                    z = fix_cmul_add<1, 1>(z, ml, limbs_of(c[2 * j + 1]));
+                    sm_acc[2 * j * 33] = make_longlong2((long long)z.re, (long long)z.im);
+                    const longlong2 b = sm_acc[(2 * j + 1) * 33];
+                    z = fix_cmul_add<1, 1>(fix_shr(zraw{(unsigned long long)b.x, (unsigned long long)b.y}, dl), ml,
+                                           limbs_of(c[2 * j]));
+                    sm_acc[(2 * j + 1) * 33] = make_longlong2((long long)z.re, (long long)z.im);
+                } else {  // no partner: m_j itself, in the same unit (m / 2)
+                    const zraw h = fix_shr(m, 1);
+                    sm_acc[2 * j * 33] = make_longlong2((long long)(z.re + h.re), (long long)(z.im + h.im));
+                }
             }
-        }
-        // 4. the units of the pairs' sums
-        if ((s & run_mask) == 0u) {
-#pragma unroll
-            for (int j = 0; j < NP; ++j) em[j] = -(1 << 20);
-        }
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            // the largest addend so far comes to [2^60, 2^61): m_j is carried
-            // 4 times over, so that its shift is to the right
-            const longlong2 v = sm_leaf[j * 32];
-            const zraw r = {(unsigned long long)v.x, (unsigned long long)v.y};
-            const int up = max(em[j], es[j] - min(fix_norm_shift(r) - 1, 2));
-            const int dl = min(up - em[j], 63);
-            em[j] = up;
-            const zraw m = fix_shr(zraw{r.re << 2, r.im << 2}, min(up - es[j] + 2, 63));
-            const longlong2 a = sm_acc[2 * j * 33];
-            zraw z = fix_shr(zraw{(unsigned long long)a.x, (unsigned long long)a.y}, dl);
-            if (2 * j + 1 < HX) {
-                const zlimb ml = limbs_of(m);
-                z = fix_cmul_add<1, 1>(z, ml, limbs_of(c[2 * j + 1]));
-                sm_acc[2 * j * 33] = make_longlong2((long long)z.re, (long long)z.im);
-                const longlong2 b = sm_acc[(2 * j + 1) * 33];
-                z = fix_cmul_add<1, 1>(fix_shr(zraw{(unsigned long long)b.x, (unsigned long long)b.y}, dl), ml,
-                                       limbs_of(c[2 * j]));
-                sm_acc[(2 * j + 1) * 33] = make_longlong2((long long)z.re, (long long)z.im);
-            } else {  // no partner: m_j itself, in the same unit (m / 2)
-                const zraw h = fix_shr(m, 1);
-                sm_acc[2 * j * 33] = make_longlong2((long long)(z.re + h.re), (long long)(z.im + h.im));
+            // the end of a run
+            if (((s + 1u) & run_mask) == 0u || s + 1 == steps)
+                minors_flush_fix<G, HX>(sm, scale_pow2(wrun, e_unit), em, lane, K,
+                                        (++runs & (kFixFold - 1u)) == 0u || s + 1 == steps);
+            if (s + 1 == steps) break;
+            uint32_t neg = 0;
+            int row = 0;  // a lane past its chunk moves on, adding zeros
+            if (s + 1 < len) {
+                int wch;
+                row = st.step(g, s, radix, &neg, &wch);
+                ws = wch ? signed_weight<double>(g.w, g.parity) : flip_sign(ws);
             }
+            if (((s + 1u) & run_mask) == 0u) wrun = ws;
+            fix_update<HX>(c, a2 + (size_t)row * KP, neg);
         }
-        // the end of a run
-        if (((s + 1u) & run_mask) == 0u || s + 1 == steps)
-            minors_flush_fix<G, HX>(sm, scale_pow2(wrun, e_unit), em, lane, K,
-                                    (++runs & (kFixFold - 1u)) == 0u || s + 1 == steps);
-        if (s + 1 == steps) break;
-        uint32_t neg = 0;
-        int row = 0;  // a lane past its chunk moves on, adding zeros
-        if (s + 1 < len) {
-            int wch;
-            row = st.step(g, s, radix, &neg, &wch);
-            ws = wch ? signed_weight<double>(g.w, g.parity) : flip_sign(ws);
-        }
-        if (((s + 1u) & run_mask) == 0u) wrun = ws;
-        fix_update<HX>(c, a2 + (size_t)row * KP, neg);
     }
     for (int t = lane; t < K; t += 32) {
         const double4 v = sm.tot[t];
