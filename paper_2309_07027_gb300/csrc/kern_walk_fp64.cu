@@ -10,34 +10,50 @@
 
 namespace bs {
 
-constexpr int kPermBlock = 128;
+constexpr int kPermBlock = 64;  // one task per CTA: two warps, half of its chunks each
 constexpr int kMinorsBlock = 64;
 
-// 128 registers (4 CTAs of 128 threads per SM) up to width 32, 168 above; one
-// CTA less ran 2 % slower at widths 26 to 30.
+// 128 registers (16 warps per SM) up to width 32, 168 above; 12 warps ran 2 %
+// slower at widths 26 to 30.  Two warps per task instead of one with twice
+// the chunks: a task's latency halves, which is the time of a job with fewer
+// tasks than resident warps (20 x 20: 109 -> 58 us).
 template <int KB>
-__global__ void __launch_bounds__(kPermBlock, KB <= 32 ? 4 : 3) walk_fp64_perm_kernel(WalkArgs a) {
-    const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kPermBlock, KB <= 32 ? 8 : 6) walk_fp64_perm_kernel(WalkArgs a) {
+    __shared__ unsigned long long s_task;
+    __shared__ ddv s_half[2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bs_job* __restrict__ jobs = a.jobs;
     const zfix* __restrict__ data = static_cast<const zfix*>(a.data);
     const unsigned long long total = task_total(a);
     const int njobs = job_count(a);
     const unsigned long long deadline = warp_deadline(a.deadline_rel_ns);
     for (;;) {
-        unsigned long long t = next_task(a.counter, total, a.status, deadline, lane);
+        if (warp == 0) {
+            const unsigned long long next = next_task(a.counter, total, a.status, deadline, lane);
+            if (lane == 0) s_task = next;
+        }
+        __syncthreads();
+        const unsigned long long t = s_task;
         if (t >= total) break;
         const bs_job jb = jobs[find_job(jobs, a.job_list, njobs, t)];
-        if (((jb.K + 3) >> 2) != KB / 4 || jb.kind != BS_KIND_PERM) {
-            if (lane == 0) atomicExch(a.status, BS_STATUS_BADJOB);
-            continue;
-        }
+        const bool ok = ((jb.K + 3) >> 2) == KB / 4 && jb.kind == BS_KIND_PERM;
         const uint32_t local = (uint32_t)(t - jb.task_begin) + jb.task_offset;
         const int* radix = a.meta + BS_META_RADIX(jb);
-        // the instance whose lanes own exactly HX = ceil(K / 2) columns
-        if (((jb.K + 1) >> 1) == KB / 2)
-            walk_task_perm_fix<KB, KB / 2>(jb, data, radix, a.partials, local, lane);
-        else
-            walk_task_perm_fix<KB, KB / 2 - 1>(jb, data, radix, a.partials, local, lane);
+        ddv re = {0.0, 0.0}, im = {0.0, 0.0};
+        if (!ok) {
+            if (threadIdx.x == 0) atomicExch(a.status, BS_STATUS_BADJOB);
+        } else if (((jb.K + 1) >> 1) == KB / 2) {  // the instance whose lanes own exactly ceil(K / 2) columns
+            walk_task_perm_fix<KB, KB / 2>(jb, data, radix, local, warp, lane, re, im);
+        } else {
+            walk_task_perm_fix<KB, KB / 2 - 1>(jb, data, radix, local, warp, lane, re, im);
+        }
+        if (threadIdx.x == 32) {
+            s_half[0] = re;
+            s_half[1] = im;
+        }
+        __syncthreads();
+        if (ok && threadIdx.x == 0)
+            store_partial(a.partials + jb.partial_off + local, dd_add_sum2(re, s_half[0]), dd_add_sum2(im, s_half[1]));
     }
 }
 
@@ -82,7 +98,7 @@ __global__ void __launch_bounds__(kMinorsBlock, MinorsMinBlocks<KB>::value) walk
 }
 
 template <typename Kern>
-static int persistent_grid(Kern k, int block, size_t smem, const WalkArgs& a) {
+static int persistent_grid(Kern k, int block, size_t smem, int threads_per_task, const WalkArgs& a) {
     int dev = 0;
     cudaGetDevice(&dev);
     int per_sm = 0;
@@ -90,7 +106,7 @@ static int persistent_grid(Kern k, int block, size_t smem, const WalkArgs& a) {
     if (per_sm < 1) per_sm = 1;
     long long grid = (long long)per_sm * sm_count(dev);
     if (!a.total_dev) {
-        long long need = ((long long)a.total_tasks * 32 + block - 1) / block;
+        long long need = ((long long)a.total_tasks * threads_per_task + block - 1) / block;
         if (need < grid) grid = need;
     }
     if (a.grid_cap > 0 && grid > a.grid_cap) grid = a.grid_cap;
@@ -100,7 +116,7 @@ static int persistent_grid(Kern k, int block, size_t smem, const WalkArgs& a) {
 
 template <int KB>
 static cudaError_t run_perm(const WalkArgs& a, cudaStream_t s) {
-    int grid = persistent_grid(walk_fp64_perm_kernel<KB>, kPermBlock, 0, a);
+    int grid = persistent_grid(walk_fp64_perm_kernel<KB>, kPermBlock, 0, kPermBlock, a);
     walk_fp64_perm_kernel<KB><<<grid, kPermBlock, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -112,7 +128,7 @@ static cudaError_t run_minors(const WalkArgs& a, cudaStream_t s) {
     cudaError_t e =
         cudaFuncSetAttribute(walk_fp64_minors_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int grid = persistent_grid(walk_fp64_minors_kernel<KB>, kMinorsBlock, smem, a);
+    int grid = persistent_grid(walk_fp64_minors_kernel<KB>, kMinorsBlock, smem, 32, a);
     walk_fp64_minors_kernel<KB><<<grid, kMinorsBlock, smem, s>>>(a);
     return cudaGetLastError();
 }

@@ -236,6 +236,15 @@ __device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e) {
     return p;
 }
 
+__device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
+    zlimb o;
+    o.rh = __shfl_xor_sync(0xffffffffu, v.rh, mask);
+    o.rl = __shfl_xor_sync(0xffffffffu, v.rl, mask);
+    o.ih = __shfl_xor_sync(0xffffffffu, v.ih, mask);
+    o.il = __shfl_xor_sync(0xffffffffu, v.il, mask);
+    return o;
+}
+
 // ---------------------------------------------------------------- one task: permanent
 // Two lanes share one chunk: lane 2p + h owns the columns [h HX, h HX + HX),
 // HX = ceil(K / 2) (an odd K leaves lane h = 1 a pad column that is exactly
@@ -246,8 +255,9 @@ __device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e) {
 // That part is converted to double and added with the weight 2^e W (one
 // conversion and one FMA per lane on the FP64 pipe, which nothing else here
 // uses), in runs of FOLD folded into a double-double.  A task's 32 chunks
-// are walked as two rounds of 16.  Every lane walks the round's longest
-// chunk, with weight 0 after its own end, so that the warp stays converged.
+// are walked by two warps, 16 each (`half_task`); a warp's sum ends in its
+// lane 0.  Every lane walks the warp's longest chunk, with weight 0 after its
+// own end, so that the warp stays converged.
 //
 // 30 x 30 permanent (2^29 addends): 165 ms in double (FP64 pipe 94 % busy),
 // 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 30.0
@@ -257,7 +267,7 @@ __device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e) {
 // double 2.7e-14.
 template <int KB, int HX>
 __device__ void walk_task_perm_fix(const bs_job& jb, const zfix* __restrict__ data, const int* __restrict__ radix,
-                                   bs_zdd* __restrict__ partials, uint32_t local, int lane) {
+                                   uint32_t local, int half_task, int lane, ddv& sum, ddv& im) {
     constexpr uint32_t FOLD = 64;
     constexpr int KP = KB;  // = BS_ROW_STRIDE(K) for every K of the bucket
     const int half = lane & 1;
@@ -266,74 +276,57 @@ __device__ void walk_task_perm_fix(const bs_job& jb, const zfix* __restrict__ da
     // exponent of a product of both lanes' operands: the last product's 64,
     // and 1 for the pad column (2^62 stands for 1, bound 2)
     const int e_pair = 64 + (jb.K & 1);
-    ddv sum = {0.0, 0.0};
-    for (int round = 0; round < 2; ++round) {
-        const uint64_t i0_own = ((uint64_t)local * 32u + (uint64_t)(16 * round + (lane >> 1))) << jb.log2L;
-        const bool has = i0_own < jb.C;
-        const uint64_t i0 = has ? i0_own : 0ull;
-        uint32_t len = 0;
-        if (has) {
-            const uint64_t rem = jb.C - i0;
-            len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
-        }
-        const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
-        if (steps == 0u) break;
-        bs_gray g;
-        ChunkStepper st;
-        st.init(g, i0, jb.nbin, jb.nrows, radix,
-                reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
-        zraw c[HX];
-        fix_seed<HX, KP>(c, g, c0, jb.nbin, jb.nrows);
-        double ws = signed_weight<double>(g.w, g.parity);
-        double acc = 0.0;
-        for (uint32_t s = 0; s < steps; ++s) {
-            int e;
-            const zlimb p = fix_product<HX>(c, e);
-            zlimb q;
-            q.rh = __shfl_xor_sync(0xffffffffu, p.rh, 1);
-            q.rl = __shfl_xor_sync(0xffffffffu, p.rl, 1);
-            q.ih = __shfl_xor_sync(0xffffffffu, p.ih, 1);
-            q.il = __shfl_xor_sync(0xffffffffu, p.il, 1);
-            e += __shfl_xor_sync(0xffffffffu, e, 1) + e_pair;
-            const long long v = fix_cmul_part(p, q, half);
-            const double f = s < len ? scale_pow2(ws, e) : 0.0;
-            acc = bfma(f, (double)v, acc);
-            if (((s + 1u) & (FOLD - 1u)) == 0u) {
-                sum = dd_add_d(sum, acc);
-                acc = 0.0;
-            }
-            if (s + 1 == steps) break;
-            uint32_t neg = 0;
-            int row = 0;  // a lane past its chunk moves on with weight 0
-            if (s + 1 < len) {
-                int wch;
-                row = st.step(g, s, radix, &neg, &wch);
-                ws = wch ? signed_weight<double>(g.w, g.parity) : flip_sign(ws);
-            }
-            fix_update<HX>(c, a2 + (size_t)row * KP, neg);
-        }
-        sum = dd_add_d(sum, acc);
+    sum = im = ddv{0.0, 0.0};
+    const uint64_t i0_own = ((uint64_t)local * 32u + (uint64_t)(16 * half_task + (lane >> 1))) << jb.log2L;
+    const bool has = i0_own < jb.C;
+    const uint64_t i0 = has ? i0_own : 0ull;
+    uint32_t len = 0;
+    if (has) {
+        const uint64_t rem = jb.C - i0;
+        len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
     }
+    const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
+    if (steps == 0u) return;
+    bs_gray g;
+    ChunkStepper st;
+    st.init(g, i0, jb.nbin, jb.nrows, radix, reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
+    zraw c[HX];
+    fix_seed<HX, KP>(c, g, c0, jb.nbin, jb.nrows);
+    double ws = signed_weight<double>(g.w, g.parity);
+    double acc = 0.0;
+    for (uint32_t s = 0; s < steps; ++s) {
+        int e;
+        const zlimb p = fix_product<HX>(c, e);
+        const zlimb q = shfl_xor_zlimb(p, 1);
+        e += __shfl_xor_sync(0xffffffffu, e, 1) + e_pair;
+        const long long v = fix_cmul_part(p, q, half);
+        const double f = s < len ? scale_pow2(ws, e) : 0.0;
+        acc = bfma(f, (double)v, acc);
+        if (((s + 1u) & (FOLD - 1u)) == 0u) {
+            sum = dd_add_d(sum, acc);
+            acc = 0.0;
+        }
+        if (s + 1 == steps) break;
+        uint32_t neg = 0;
+        int row = 0;  // a lane past its chunk moves on with weight 0
+        if (s + 1 < len) {
+            int wch;
+            row = st.step(g, s, radix, &neg, &wch);
+            ws = wch ? signed_weight<double>(g.w, g.parity) : flip_sign(ws);
+        }
+        fix_update<HX>(c, a2 + (size_t)row * KP, neg);
+    }
+    sum = dd_add_d(sum, acc);
     // over the 16 lanes of each part, then the imaginary part to lane 0
 #pragma unroll
     for (int off = 16; off > 1; off >>= 1) sum = dd_add_sum2(sum, shfl_down_dd(sum, off));
-    const ddv im = shfl_down_dd(sum, 1);
-    if (lane == 0) store_partial(partials + jb.partial_off + local, sum, im);
+    im = shfl_down_dd(sum, 1);
 }
 
 // ---------------------------------------------------------------- one task: minors
 // v >> d, 0 <= d <= 63 (rounded down).
 __device__ __forceinline__ zraw fix_shr(const zraw& v, int d) {
     return zraw{(unsigned long long)((long long)v.re >> d), (unsigned long long)((long long)v.im >> d)};
-}
-
-__device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
-    zlimb o;
-    o.rh = __shfl_xor_sync(0xffffffffu, v.rh, mask);
-    o.rl = __shfl_xor_sync(0xffffffffu, v.rl, mask);
-    o.ih = __shfl_xor_sync(0xffffffffu, v.ih, mask);
-    o.il = __shfl_xor_sync(0xffffffffu, v.il, mask);
-    return o;
 }
 
 // Longest integer run of the minors, in addends (a power of two).
