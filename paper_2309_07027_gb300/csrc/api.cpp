@@ -55,9 +55,10 @@ constexpr int kMaxGroups = 64;
 constexpr int kCtlStatus = kMaxGroups;                          // int status word (in a 64-bit slot)
 constexpr int kCtlTotal = kMaxGroups + 1;                       // sampler task totals, one per precision
 constexpr int kCtlCounter = kCtlTotal + BS_NPREC;                // sampler work counters, one per precision
-constexpr int kCtlStats = kCtlCounter + BS_NPREC;                // [addends, flops] per precision
-constexpr int kCtlListLen = kCtlStats + 2 * BS_NPREC;            // ints: sampler list lengths
-constexpr int kCtlSlots = kCtlListLen + 8;
+constexpr int kCtlListLen = kCtlCounter + BS_NPREC;              // ints: sampler list lengths
+constexpr int kCtlCleared = kCtlListLen + 8;                     // the slots before this one are zeroed for every run
+constexpr int kCtlStats = kCtlCleared;                           // [addends, flops] per precision
+constexpr int kCtlSlots = kCtlStats + 2 * BS_NPREC;
 
 struct Timed {
     cudaEvent_t e0, e1;
@@ -71,7 +72,7 @@ struct bs_ctx {
     cudaStream_t own = nullptr;
     cudaStream_t stream = nullptr;
     size_t budget = 0, used = 0;
-    DevBuf src, jobs, meta, data64, data32, partials, out, out_lo, ctl;
+    DevBuf src, jobs, meta, data64, data32, partials, out, ctl;
     DevBuf cc_inputs, cc_cols, cc_rows, cc_jobs, cc_meta, cc_data, cc_partials, cc_minors, cc_out, cc_U, cc_lists,
         cc_args;
     // captured sampler step loop (one batch), replayed while its key matches
@@ -335,11 +336,18 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
         r.kind = in.p->kind;
         r.bucket = r.prec == BS_PREC_DF ? (in.p->K + 7) >> 3 : (in.p->K + 3) >> 2;
         r.cpt = bs_chunks_per_task(r.kind, r.prec, in.p->K);
-        r.log2L = bs_choose_log2L_single(in.p->C, r.cpt, c->log2max[r.prec],
-                                         r.prec == BS_PREC_FP32 ? BS_TARGET_TASKS_SINGLE_FP32 : BS_TARGET_TASKS_SINGLE);
-        uint64_t per = (uint64_t)r.cpt << r.log2L;
-        r.ntasks = (uint32_t)((in.p->C + per - 1) / per);
         r.ncols = r.kind == BS_KIND_PERM ? 1 : in.p->K;
+        const bool lone = r.kind == BS_KIND_MINORS && r.prec != BS_PREC_FP32;  // (minors never come in batches)
+        for (int fill : {lone ? BS_TARGET_TASKS_FILL_ONE : BS_TARGET_TASKS_FILL, BS_TARGET_TASKS_FILL}) {
+            r.log2L = bs_choose_log2L_single(in.p->C, r.cpt, c->log2max[r.prec],
+                                             r.prec == BS_PREC_FP32 ? BS_TARGET_TASKS_SINGLE_FP32 : BS_TARGET_TASKS_SINGLE,
+                                             fill);
+            const uint64_t per = (uint64_t)r.cpt << r.log2L;
+            r.ntasks = (uint32_t)((in.p->C + per - 1) / per);
+            // (the longer chunks again where a budget would not hold the partials)
+            if (!c->budget || c->used - c->partials.n + (size_t)r.ntasks * r.ncols * sizeof(bs_zdd) + (1u << 20) <= c->budget)
+                break;
+        }
         rows.push_back(r);
     }
     P = Prepared();
@@ -450,12 +458,12 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
 
 // Device half: counters, pack, one walk launch per group, reduce; nothing
 // that synchronises, so it can be captured into a graph.
-int enqueue_device(bs_ctx* c, const Prepared& P, const double2* d_src, double2* d_out, double2* d_out_lo) {
+int enqueue_device(bs_ctx* c, const Prepared& P, const double2* d_src, double2* d_out, double2* d_out_lo,
+                   int* d_status_out) {
     int rc;
     // counters, totals and status; the statistics slots are cleared only by
     // bs_ctx_reset_stats
-    BS_CUDA(cudaMemsetAsync(c->ctl.p, 0, kCtlStats * 8, c->stream));
-    BS_CUDA(cudaMemsetAsync(static_cast<unsigned long long*>(c->ctl.p) + kCtlListLen, 0, (kCtlSlots - kCtlListLen) * 8, c->stream));
+    BS_CUDA(cudaMemsetAsync(c->ctl.p, 0, kCtlCleared * 8, c->stream));
     const bs_job* djobs = static_cast<const bs_job*>(c->jobs.p);
     for (int prec = 0; prec < BS_NPREC; ++prec) {
         const size_t lo = P.pbeg[prec], hi = P.pbeg[prec + 1];
@@ -484,23 +492,17 @@ int enqueue_device(bs_ctx* c, const Prepared& P, const double2* d_src, double2* 
     }
     {
         cudaError_t e = bs::launch_reduce(djobs, (int)P.njobs, static_cast<const bs_zdd*>(c->partials.p),
-                                          static_cast<const int*>(c->meta.p), d_out, d_out_lo, P.max_cols, c->stream);
+                                          static_cast<const int*>(c->meta.p), d_out, d_out_lo, P.max_cols, c->stream,
+                                          reinterpret_cast<const int*>(ctl + kCtlStatus), d_status_out);
         if (e != cudaSuccess) return fail(BS_ECUDA, "reduce launch failed: %s", cudaGetErrorString(e));
         c->stats.kernel_launches++;
     }
     return BS_OK;
 }
 
-int run_jobs(bs_ctx* c, std::vector<JobIn>& ins, const double2* d_src, bs_mode mode, double2* d_out,
-             double2* d_out_lo) {
-    Prepared P;
-    int rc = plan_upload(c, ins, mode, P);
-    if (rc || P.njobs == 0) return rc;
-    if ((rc = enqueue_device(c, P, d_src, d_out, d_out_lo))) return rc;
-    for (int p = 0; p < BS_NPREC; ++p) {
-        c->stats.addends[p] += P.adds[p];
-        c->stats.addend_flops[p] += P.flops[p];
-    }
+int status_code(int st) {
+    if (st == BS_STATUS_TIMEOUT) return fail(BS_ETIMEOUT, "a walk kernel passed its deadline");
+    if (st == BS_STATUS_BADJOB) return fail(BS_ECUDA, "a walk kernel received a job of the wrong bucket");
     return BS_OK;
 }
 
@@ -509,16 +511,16 @@ int check_status(bs_ctx* c) {
     int st = 0;
     BS_CUDA(cudaMemcpy(&st, static_cast<unsigned long long*>(c->ctl.p) + kCtlStatus, sizeof(int),
                        cudaMemcpyDeviceToHost));
-    if (st == BS_STATUS_TIMEOUT) return fail(BS_ETIMEOUT, "a walk kernel passed its deadline");
-    if (st == BS_STATUS_BADJOB) return fail(BS_ECUDA, "a walk kernel received a job of the wrong bucket");
-    return BS_OK;
+    return status_code(st);
 }
 
-// Reads nout results (hi, lo) and the walk status word back through one
-// pinned buffer and one stream synchronisation.
-int read_back_and_check(bs_ctx* c, double2* hi, double2* lo, int nout) {
-    const size_t out_b = (size_t)nout * sizeof(double2);
-    const size_t need = 2 * out_b + sizeof(unsigned long long);
+// c->out holds `n` results and behind them a copy of the walk status word,
+// which the reduce kernel writes: one copy, through a pinned buffer, and one
+// synchronisation bring both back (h: the pinned copy of the results).
+size_t out_bytes(int n) { return (size_t)n * sizeof(double2) + 16; }
+int* out_status(bs_ctx* c, int n) { return reinterpret_cast<int*>(static_cast<double2*>(c->out.p) + n); }
+int read_back_and_check(bs_ctx* c, int n, const double2** h) {
+    const size_t need = out_bytes(n);
     if (c->h_back_n < need) {
         if (c->h_back) cudaFreeHost(c->h_back);
         c->h_back = nullptr;
@@ -527,20 +529,13 @@ int read_back_and_check(bs_ctx* c, double2* hi, double2* lo, int nout) {
         BS_CUDA(cudaHostAlloc(&c->h_back, want, cudaHostAllocDefault));
         c->h_back_n = want;
     }
-    char* h = static_cast<char*>(c->h_back);
-    BS_CUDA(cudaMemcpyAsync(h, c->out.p, out_b, cudaMemcpyDeviceToHost, c->stream));
-    BS_CUDA(cudaMemcpyAsync(h + out_b, c->out_lo.p, out_b, cudaMemcpyDeviceToHost, c->stream));
-    BS_CUDA(cudaMemcpyAsync(h + 2 * out_b, static_cast<unsigned long long*>(c->ctl.p) + kCtlStatus,
-                            sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+    BS_CUDA(cudaMemcpyAsync(c->h_back, c->out.p, need, cudaMemcpyDeviceToHost, c->stream));
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return fail(BS_ECUDA, "stream synchronize: %s", cudaGetErrorString(e));
-    std::memcpy(hi, h, out_b);
-    std::memcpy(lo, h + out_b, out_b);
+    *h = static_cast<const double2*>(c->h_back);
     int st = 0;
-    std::memcpy(&st, h + 2 * out_b, sizeof(int));
-    if (st == BS_STATUS_TIMEOUT) return fail(BS_ETIMEOUT, "a walk kernel passed its deadline");
-    if (st == BS_STATUS_BADJOB) return fail(BS_ECUDA, "a walk kernel received a job of the wrong bucket");
-    return BS_OK;
+    std::memcpy(&st, *h + n, sizeof(int));
+    return status_code(st);
 }
 
 int sync_and_check(bs_ctx* c) {
@@ -571,7 +566,7 @@ void copy_matrix(bs_c128* dst, const bs_c128* A, int rows, int cols, int ld) {
 // the legacy default stream and while the caller captures the stream.
 int batch_walk(bs_ctx* c, std::vector<IntPlan>& plans, const std::vector<int64_t>& key,
                       const int64_t* a_offset, const int* cols, const double2* d_src, double2* d_out, bs_mode mode,
-                      double2* d_out_lo, bool capture_on_repeat = false) {
+                      double2* d_out_lo, int* d_status_out, bool capture_on_repeat = false) {
     int rc;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (c->stream != nullptr) BS_CUDA(cudaStreamIsCapturing(c->stream, &cap));
@@ -602,11 +597,11 @@ int batch_walk(bs_ctx* c, std::vector<IntPlan>& plans, const std::vector<int64_t
     if ((rc = plan_upload(c, ins, mode, P))) return rc;
     if (P.njobs == 0) return BS_OK;
     if (!graphs) {
-        if ((rc = enqueue_device(c, P, d_src, d_out, d_out_lo))) return rc;
+        if ((rc = enqueue_device(c, P, d_src, d_out, d_out_lo, d_status_out))) return rc;
     } else {
         const uint64_t w0 = c->stats.walk_launches, k0 = c->stats.kernel_launches;
         BS_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-        rc = enqueue_device(c, P, d_src, d_out, d_out_lo);
+        rc = enqueue_device(c, P, d_src, d_out, d_out_lo, d_status_out);
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(c->stream, &g);
         if (rc || e != cudaSuccess) {
@@ -685,8 +680,7 @@ int run_single(bs_ctx* c, const bs_c128* A, int rows, int cols, int ld, int kind
     BS_CUDA(cudaSetDevice(c->device));
     const size_t mat_b = (size_t)rows * cols * sizeof(bs_c128);
     if ((rc = ensure(c, c->src, mat_b))) return rc;
-    if ((rc = ensure(c, c->out, nout * sizeof(double2)))) return rc;
-    if ((rc = ensure(c, c->out_lo, nout * sizeof(double2)))) return rc;
+    if ((rc = ensure(c, c->out, out_bytes(2 * nout)))) return rc;
     bs_c128* h = static_cast<bs_c128*>(stage(c, mat_b));
     if (!h) return fail(BS_ENOMEM, "pinned host staging allocation failed");
     copy_matrix(h, A, rows, cols, ld);
@@ -695,9 +689,13 @@ int run_single(bs_ctx* c, const bs_c128* A, int rows, int cols, int ld, int kind
     std::vector<IntPlan> plans = {p};
     const int64_t off0 = 0;
     rc = batch_walk(c, plans, plan_key(c, p, rows, cols, mode), &off0, &cols, static_cast<const double2*>(c->src.p),
-                    static_cast<double2*>(c->out.p), mode, static_cast<double2*>(c->out_lo.p), true);
-    if (rc) return rc;
-    return read_back_and_check(c, hi.data(), lo.data(), nout);
+                    static_cast<double2*>(c->out.p), mode, static_cast<double2*>(c->out.p) + nout,
+                    out_status(c, 2 * nout), true);
+    const double2* h2 = nullptr;
+    if (rc || (rc = read_back_and_check(c, 2 * nout, &h2))) return rc;
+    std::copy(h2, h2 + nout, hi.begin());
+    std::copy(h2 + nout, h2 + 2 * nout, lo.begin());
+    return BS_OK;
 }
 
 int single_job(bs_ctx* c, const bs_c128* A, int rows, int cols, int ld, const int* M, const int* N, int kind,
@@ -857,8 +855,7 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
     BS_CUDA(cudaEventRecord(c->stage_ev[c->stage_cur], c->stream));
     // counters, totals and status; the statistics slots are cleared only by
     // bs_ctx_reset_stats
-    BS_CUDA(cudaMemsetAsync(c->ctl.p, 0, kCtlStats * 8, c->stream));
-    BS_CUDA(cudaMemsetAsync(static_cast<unsigned long long*>(c->ctl.p) + kCtlListLen, 0, (kCtlSlots - kCtlListLen) * 8, c->stream));
+    BS_CUDA(cudaMemsetAsync(c->ctl.p, 0, kCtlCleared * 8, c->stream));
     unsigned long long* ctl = static_cast<unsigned long long*>(c->ctl.p);
     if ((rc = ensure(c, c->cc_args, sizeof(bs::CcArgs)))) return rc;
     bs::CcArgs* da = static_cast<bs::CcArgs*>(c->cc_args.p);
@@ -1025,7 +1022,7 @@ void bs_ctx_destroy(bs_ctx* c) {
         cudaEventDestroy(t.e1);
     }
     DevBuf* bufs[] = {&c->src,       &c->jobs,     &c->meta,     &c->data64,  &c->data32,      &c->partials,
-                      &c->out,       &c->out_lo,   &c->ctl,      &c->cc_inputs, &c->cc_cols,   &c->cc_rows,
+                      &c->out,       &c->ctl,      &c->cc_inputs, &c->cc_cols,   &c->cc_rows,
                       &c->cc_jobs,   &c->cc_meta,  &c->cc_data,  &c->cc_partials, &c->cc_minors, &c->cc_out,
                       &c->cc_U, &c->cc_lists, &c->cc_args};
     if (c->cc_exec) cudaGraphExecDestroy(c->cc_exec);
@@ -1211,7 +1208,7 @@ int bs_perm_batch(bs_ctx* c, int count, const bs_c128* A_packed, const int64_t* 
         if (!plans[b].trivial) total += (size_t)rows[b] * cols[b];
     }
     if ((rc = ensure(c, c->src, total * sizeof(bs_c128)))) return rc;
-    if ((rc = ensure(c, c->out, count * sizeof(double2)))) return rc;
+    if ((rc = ensure(c, c->out, out_bytes(count)))) return rc;
     bs_c128* h = static_cast<bs_c128*>(stage(c, total * sizeof(bs_c128)));
     if (!h) return fail(BS_ENOMEM, "pinned host staging allocation failed");
     for (int b = 0; b < count; ++b)
@@ -1222,11 +1219,12 @@ int bs_perm_batch(bs_ctx* c, int count, const bs_c128* A_packed, const int64_t* 
     const std::vector<int64_t> key =
         batch_key(c, count, off.data(), rows, cols, mult_packed, row_mult_off, col_mult_off, mode);
     rc = batch_walk(c, plans, key, off.data(), cols, static_cast<const double2*>(c->src.p),
-                    static_cast<double2*>(c->out.p), mode, nullptr);
+                    static_cast<double2*>(c->out.p), mode, nullptr, out_status(c, count));
     if (rc) return rc;
-    std::vector<double2> res(count);
-    BS_CUDA(cudaMemcpyAsync(res.data(), c->out.p, count * sizeof(double2), cudaMemcpyDeviceToHost, c->stream));
-    if ((rc = sync_and_check(c))) return rc;
+    bool walked = false;
+    for (int b = 0; b < count; ++b) walked |= !plans[b].trivial;
+    const double2* res = nullptr;
+    if (walked && (rc = read_back_and_check(c, count, &res))) return rc;
     for (int b = 0; b < count; ++b) {
         if (plans[b].trivial) {
             out[b].re = 1.0;
@@ -1256,7 +1254,7 @@ int bs_perm_batch_dev(bs_ctx* c, int count, const bs_c128* A_packed_dev, const i
     const std::vector<int64_t> key =
         batch_key(c, count, a_offset, rows, cols, mult_packed, row_mult_off, col_mult_off, mode);
     rc = batch_walk(c, plans, key, a_offset, cols, reinterpret_cast<const double2*>(A_packed_dev),
-                    reinterpret_cast<double2*>(out_dev), mode, nullptr);
+                    reinterpret_cast<double2*>(out_dev), mode, nullptr, nullptr);
     if (rc) return rc;
     if (!trivial.empty()) {
         static const double2 one = {1.0, 0.0};
@@ -1563,7 +1561,8 @@ int bs_debug_plan(int rows, int cols, const int* row_mult, const int* col_mult, 
     // chunking of this job planned alone in FP64 mode (default maximum 2^12)
     const int kd = kind == 1 ? BS_KIND_MINORS : BS_KIND_PERM;
     const int cpt = bs_chunks_per_task(kd, 0, p.K);
-    const int l = p.trivial ? 0 : bs_choose_log2L_single(p.C, cpt, bs_default_log2max(BS_PREC_FP64), BS_TARGET_TASKS_SINGLE);
+    const int l = p.trivial ? 0 : bs_choose_log2L_single(p.C, cpt, bs_default_log2max(BS_PREC_FP64), BS_TARGET_TASKS_SINGLE,
+                                                         kd == BS_KIND_MINORS ? BS_TARGET_TASKS_FILL_ONE : BS_TARGET_TASKS_FILL);
     const uint64_t per = (uint64_t)cpt << l;
     info[6] = l;
     info[7] = p.trivial ? 0 : (int64_t)((p.C + per - 1) / per);

@@ -49,78 +49,113 @@ __device__ __forceinline__ ddv sum2_final(ddv a) {
     return ddv{h, __dadd_rn(__dsub_rn(a.hi, __dsub_rn(h, bb)), __dsub_rn(a.lo, bb))};
 }
 
+// x 2^e: one multiplication where 2^e is a normal double (the same rounding
+// as ldexp, whose general form takes several times as long).
+__device__ __forceinline__ double scale2(double x, int e) {
+    return abs(e) <= 1000 ? x * __hiloint2double((1023 + e) << 20, 0) : ldexp(x, e);
+}
+
+// One CTA per (job, output column).  A CTA's time is its chain of dependent
+// FP64 operations and loads, so the tree starts at the level the task count
+// needs (in one warp, by shuffles, up to 32 tasks: no barrier), the column
+// exponents are read by a warp at once, and the four results are scaled by
+// four lanes.  9 tasks, 12 columns: 10.5 -> 7.6 us.
 __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __restrict__ jobs,
                                                               const bs_zdd* __restrict__ partials,
                                                               const int* __restrict__ meta, double2* __restrict__ out,
-                                                              double2* __restrict__ out_lo) {
+                                                              double2* __restrict__ out_lo,
+                                                              const int* __restrict__ status,
+                                                              int* __restrict__ status_out) {
     // Sum2 (Ogita, Rump and Oishi 2005): the high parts are added with TwoSum,
     // the TwoSum errors and the low parts go to one plain double c; result
     // (s, c) as accurate as a sum in twice the working precision, at 8 FP64
     // operations per addition instead of about 20 for a double-double add.
     __shared__ ddv sre[kReduceBlock];
     __shared__ ddv sim[kReduceBlock];
-    const bs_job jb = jobs[blockIdx.x];
-    const int ncols = jb.kind == BS_KIND_PERM ? 1 : jb.K;
+    if (status_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status_out = *status;
+    const bs_job& jb = jobs[blockIdx.x];
+    const int K = jb.K;
+    const bool minors = jb.kind != BS_KIND_PERM;
+    const int ncols = minors ? K : 1;
     const int col = blockIdx.y;
     if (col >= ncols) return;
+    const uint32_t ntasks = jb.ntasks;
+    const int lane = threadIdx.x & 31;
+    if (ntasks <= 32u && threadIdx.x >= 32) return;
+    const bs_zdd* p = partials + jb.partial_off + col;
     ddv re = {0.0, 0.0}, im = {0.0, 0.0};  // (s, c)
-    for (uint32_t t = threadIdx.x; t < jb.ntasks; t += kReduceBlock) {
-        bs_zdd p = partials[jb.partial_off + (int64_t)t * ncols + col];
-        re = sum2_add(re, p.re_hi, p.re_lo);
-        im = sum2_add(im, p.im_hi, p.im_lo);
+    for (uint32_t t = threadIdx.x; t < ntasks; t += kReduceBlock) {
+        const bs_zdd v = p[(int64_t)t * ncols];
+        re = sum2_add(re, v.re_hi, v.re_lo);
+        im = sum2_add(im, v.im_hi, v.im_lo);
     }
-    sre[threadIdx.x] = re;
-    sim[threadIdx.x] = im;
-    __syncthreads();
-    for (int w = kReduceBlock / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            const ddv r2 = sre[threadIdx.x + w], i2 = sim[threadIdx.x + w];
-            sre[threadIdx.x] = sum2_add(sre[threadIdx.x], r2.hi, r2.lo);
-            sim[threadIdx.x] = sum2_add(sim[threadIdx.x], i2.hi, i2.lo);
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        sre[0] = sum2_final(sre[0]);
-        sim[0] = sum2_final(sim[0]);
-    }
-    if (threadIdx.x == 0) {
-        // prefactor: 2^(1-n) times the column scales (Eq. bbfgrepeated), or
-        // (-1)^n (Eq. ryser), or (-1)^(n-1) 2 (Nijenhuis-Wilf)
-        int e = 0, bad = 0;
-        double sgn = 1.0;
+    int e = 0, bad = 0;
+    if (threadIdx.x < 32) {  // the exponents of the columns that enter the product
         const int* colexp = meta + BS_META_COLEXP(jb);
-        for (int c = 0; c < jb.K; ++c) {
-            if (jb.kind == BS_KIND_MINORS && c == col) continue;
-            if (colexp[c] >= BS_COLEXP_NAN_RE)
-                bad |= colexp[c];
+        for (int c = lane; c < K; c += 32) {
+            if (minors && c == col) continue;
+            const int x = colexp[c];
+            if (x >= BS_COLEXP_NAN_RE)
+                bad |= x;
             else
-                e += colexp[c];
+                e += x;
         }
-        if (jb.formula == BS_JOB_BBFG) {
-            e += 1 - jb.n;
-        } else if (jb.formula == BS_JOB_RYSER) {
-            sgn = (jb.n & 1) ? -1.0 : 1.0;
-        } else {
-            e += 1;
-            sgn = ((jb.n - 1) & 1) ? -1.0 : 1.0;
-        }
-        ddv r = sre[0], i = sim[0];
-        if (bad) {  // an input that is not finite (a product of two or more columns mixes both components)
-            const double nan = __longlong_as_double(0x7ff8000000000000ll);
-            if (jb.K > 1 || (bad & BS_COLEXP_NAN_RE)) r = ddv{nan, nan};
-            if (jb.K > 1 || (bad & BS_COLEXP_NAN_IM)) i = ddv{nan, nan};
-        }
-        out[jb.out_index + col] = make_double2(sgn * ldexp(r.hi, e), sgn * ldexp(i.hi, e));
-        if (out_lo) out_lo[jb.out_index + col] = make_double2(sgn * ldexp(r.lo, e), sgn * ldexp(i.lo, e));
+        e = __reduce_add_sync(0xffffffffu, e);
+        bad = (int)__reduce_or_sync(0xffffffffu, (unsigned)bad);
     }
+    if (ntasks > 32u) {
+        sre[threadIdx.x] = re;
+        sim[threadIdx.x] = im;
+        __syncthreads();
+        int w = kReduceBlock / 2;
+        while (w >= (int)ntasks) w >>= 1;  // the upper half holds zeros
+        for (; w >= 32; w >>= 1) {
+            if ((int)threadIdx.x < w) {
+                const ddv r2 = sre[threadIdx.x + w], i2 = sim[threadIdx.x + w];
+                sre[threadIdx.x] = re = sum2_add(re, r2.hi, r2.lo);
+                sim[threadIdx.x] = im = sum2_add(im, i2.hi, i2.lo);
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x >= 32) return;
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        if (off >= (int)ntasks) continue;
+        const ddv r2 = shfl_down_dd(re, off), i2 = shfl_down_dd(im, off);
+        re = sum2_add(re, r2.hi, r2.lo);
+        im = sum2_add(im, i2.hi, i2.lo);
+    }
+    // prefactor: 2^(1-n) times the column scales (Eq. bbfgrepeated), or
+    // (-1)^n (Eq. ryser), or (-1)^(n-1) 2 (Nijenhuis-Wilf)
+    double sgn = 1.0;
+    if (jb.formula == BS_JOB_BBFG) {
+        e += 1 - jb.n;
+    } else if (jb.formula == BS_JOB_RYSER) {
+        sgn = (jb.n & 1) ? -1.0 : 1.0;
+    } else {
+        e += 1;
+        sgn = ((jb.n - 1) & 1) ? -1.0 : 1.0;
+    }
+    re = sum2_final(re);
+    im = sum2_final(im);
+    const double rh = __shfl_sync(0xffffffffu, re.hi, 0), rl = __shfl_sync(0xffffffffu, re.lo, 0);
+    const double ih = __shfl_sync(0xffffffffu, im.hi, 0), il = __shfl_sync(0xffffffffu, im.lo, 0);
+    if (lane >= 4) return;
+    double x = lane == 0 ? rh : lane == 1 ? ih : lane == 2 ? rl : il;
+    x = sgn * scale2(x, e);
+    // an input that is not finite (a product of two or more columns mixes
+    // both components)
+    if (bad && (K > 1 || (bad & ((lane & 1) ? BS_COLEXP_NAN_IM : BS_COLEXP_NAN_RE))))
+        x = __longlong_as_double(0x7ff8000000000000ll);
+    double2* o = lane < 2 ? out : out_lo;
+    if (o) reinterpret_cast<double*>(o + jb.out_index + col)[lane & 1] = x;
 }
 
 cudaError_t launch_reduce(const bs_job* jobs, int njobs, const bs_zdd* partials, const int* meta, double2* out,
-                          double2* out_lo, int max_cols, cudaStream_t s) {
+                          double2* out_lo, int max_cols, cudaStream_t s, const int* status, int* status_out) {
     if (njobs <= 0) return cudaSuccess;
     dim3 grid(njobs, max_cols < 1 ? 1 : max_cols);
-    reduce_kernel<<<grid, kReduceBlock, 0, s>>>(jobs, partials, meta, out, out_lo);
+    reduce_kernel<<<grid, kReduceBlock, 0, s>>>(jobs, partials, meta, out, out_lo, status, status_out);
     return cudaGetLastError();
 }
 

@@ -40,9 +40,10 @@ cudaError_t launch_pack(const bs_job* jobs, int njobs, const double2* src, int* 
 
 // Sums each job's task partials in a fixed order and applies 2^(1-n) and the
 // column scales; writes out[out_index + col] (and the low parts to out_lo when
-// non-null).
+// non-null).  With status_out, also copies the walks' status word there.
 cudaError_t launch_reduce(const bs_job* jobs, int njobs, const bs_zdd* partials, const int* meta, double2* out,
-                          double2* out_lo, int max_cols, cudaStream_t s);
+                          double2* out_lo, int max_cols, cudaStream_t s,
+                          const int* status = nullptr, int* status_out = nullptr);
 
 // Measured issue rates (lane-operations per second) of the FP64 and FP32
 // fused multiply-add pipes, from a timed microbenchmark on this device.

@@ -73,75 +73,84 @@ __device__ __forceinline__ void pack_fix(const bs_job& jb, const double2* __rest
     const int prow = meta[BS_META_PINNED(jb)];
     const int KP = BS_ROW_STRIDE(jb.K);
     const bool bbfg = jb.formula == BS_JOB_BBFG, nw = jb.formula == BS_JOB_NW;
-    for (int col = tid; col < KP; col += nthreads) {
-        if (col >= jb.K) {  // pad column: a column sum of exactly 1 = 2^62 / 2^63 2^1
-            out[col] = zfix{1ll << 62, 0};
-            for (int j = 1; j <= jb.nrows; ++j) out[(size_t)j * KP + col] = zfix{0, 0};
-            continue;
-        }
-        const int sc = csrc[col];
+    // four lanes per column, each with every fourth digit row: the packing of
+    // a small job is a chain of dependent loads, and this one is a quarter as
+    // long (12 photons: 12.1 -> 7.1 us); the sums are combined in a fixed
+    // order, the integer ones exactly.
+    const int part = tid & 3;
+    for (int base = 0; base < KP; base += nthreads >> 2) {  // (every lane runs every round)
+        const int col = base + (tid >> 2);
+        const bool live = col < jb.K;
+        const int sc = csrc[live ? col : 0];
+        const bool first = part == 0 && (bbfg || nw);  // this lane also takes the start row
+        const int frow = bbfg ? prow : jb.n - 1;
         double bre = 0.0, bim = 0.0;
-        if (bbfg) {
-            const double2 a = src_elem(src, jb, prow, sc);
-            bre = fabs(a.x);
-            bim = fabs(a.y);
-        } else if (nw) {
-            const double2 a = src_elem(src, jb, jb.n - 1, sc);
+        if (first) {
+            const double2 a = src_elem(src, jb, frow, sc);
             bre = fabs(a.x);
             bim = fabs(a.y);
         }
-        for (int j = 0; j < jb.nrows; ++j) {
+#pragma unroll 2
+        for (int j = part; j < jb.nrows; j += 4) {
             const double2 d = src_elem(src, jb, dsrc[j], sc);
             const double m = bbfg ? (double)(radix[j] - 1) : 1.0;
             bre += m * fabs(d.x);
             bim += m * fabs(d.y);
         }
+        bre += __shfl_xor_sync(0xffffffffu, bre, 1);
+        bim += __shfl_xor_sync(0xffffffffu, bim, 1);
+        bre += __shfl_xor_sync(0xffffffffu, bre, 2);
+        bim += __shfl_xor_sync(0xffffffffu, bim, 2);
         int flags = 0;
         if (!isfinite(bre)) flags |= BS_COLEXP_NAN_RE;
         if (!isfinite(bim)) flags |= BS_COLEXP_NAN_IM;
-        if (flags) {
-            colexp[col] = flags;
-            for (int j = 0; j <= jb.nrows; ++j) out[(size_t)j * KP + col] = zfix{0, 0};
-            continue;
-        }
         int e = 0;
         const double b = 0.25 * bre + 0.25 * bim;  // a quarter: b must not overflow
-        if (b > 0.0) {
+        if (!flags && b > 0.0) {
             (void)frexp(b * (1.0 + 0x1p-20), &e);
             e += 2;
         }
-        colexp[col] = e;
+        const bool use = live && !flags;
         const int sh = nw ? 62 - e : 63 - e;
-        const int up = nw ? 1 : 0;
         unsigned long long sre = 0, sim = 0;  // the start sums
-        if (bbfg || nw) {
-            const double2 a = src_elem(src, jb, bbfg ? prow : jb.n - 1, sc);
+        if (use && first) {
+            const double2 a = src_elem(src, jb, frow, sc);
             sre = (unsigned long long)__double2ll_rn(ldexp(a.x, sh));
             sim = (unsigned long long)__double2ll_rn(ldexp(a.y, sh));
         }
-        for (int j = 0; j < jb.nrows; ++j) {
-            const double2 d = src_elem(src, jb, dsrc[j], sc);
-            const unsigned long long qre = (unsigned long long)__double2ll_rn(ldexp(d.x, sh));
-            const unsigned long long qim = (unsigned long long)__double2ll_rn(ldexp(d.y, sh));
-            zfix row;
-            if (bbfg) {
-                const unsigned long long m = (unsigned long long)(radix[j] - 1);
-                sre += m * qre;
-                sim += m * qim;
-                row.re = (long long)(2ull * qre);
-                row.im = (long long)(2ull * qim);
-            } else {
-                // Nijenhuis-Wilf start: 2 x = 2 a_last - sum over all columns
-                // = a_last - sum over the digits, in even units
-                sre -= nw ? qre : 0ull;
-                sim -= nw ? qim : 0ull;
-                row.re = -(long long)(qre << up);
-                row.im = -(long long)(qim << up);
+#pragma unroll 2
+        for (int j = part; j < jb.nrows; j += 4) {
+            zfix row = {0, 0};
+            if (use) {
+                const double2 d = src_elem(src, jb, dsrc[j], sc);
+                const unsigned long long qre = (unsigned long long)__double2ll_rn(ldexp(d.x, sh));
+                const unsigned long long qim = (unsigned long long)__double2ll_rn(ldexp(d.y, sh));
+                if (bbfg) {
+                    const unsigned long long m = (unsigned long long)(radix[j] - 1);
+                    sre += m * qre;
+                    sim += m * qim;
+                    row.re = (long long)(2ull * qre);
+                    row.im = (long long)(2ull * qim);
+                } else {
+                    // Nijenhuis-Wilf start: 2 x = 2 a_last - sum over all
+                    // columns = a_last - sum over the digits, in even units
+                    sre -= nw ? qre : 0ull;
+                    sim -= nw ? qim : 0ull;
+                    row.re = -(long long)(qre << (nw ? 1 : 0));
+                    row.im = -(long long)(qim << (nw ? 1 : 0));
+                }
             }
-            out[(size_t)(1 + j) * KP + col] = row;
+            if (col < KP) out[(size_t)(1 + j) * KP + col] = row;
         }
-        out[col].re = (long long)sre;
-        out[col].im = (long long)sim;
+        sre += __shfl_xor_sync(0xffffffffu, sre, 1);
+        sim += __shfl_xor_sync(0xffffffffu, sim, 1);
+        sre += __shfl_xor_sync(0xffffffffu, sre, 2);
+        sim += __shfl_xor_sync(0xffffffffu, sim, 2);
+        if (part == 0 && col < KP) {
+            // a pad column's sum is exactly 1 = 2^62 / 2^63 2^1
+            out[col] = live ? zfix{(long long)sre, (long long)sim} : zfix{1ll << 62, 0};
+            if (live) colexp[col] = flags ? flags : e;
+        }
     }
 }
 
@@ -153,12 +162,17 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
     const int* csrc = meta + BS_META_COL_SRC(jb);
     int* colexp = meta + BS_META_COLEXP(jb);
     const int prow = meta[BS_META_PINNED(jb)];
-    // binomial table C(M_j, d), digit after digit
-    if (tid == 0) {
-        uint64_t* binom = reinterpret_cast<uint64_t*>(meta + BS_META_BINOM(jb));
-        int at = 0;
-        for (int j = 0; j < jb.nrows; ++j)
-            for (int d = 0; d < radix[j]; ++d) binom[at++] = bs_binom(radix[j] - 1, d);
+    // binomial table C(M_j, d), digit after digit: a thread per digit
+    for (int j = tid; j < jb.nrows; j += nthreads) {
+        uint64_t* binom = reinterpret_cast<uint64_t*>(meta + BS_META_BINOM(jb)) + 2 * min(j, jb.nbin);
+        for (int i = jb.nbin; i < j; ++i) binom += radix[i];
+        const int M = radix[j] - 1;
+        uint64_t v = 1;
+        binom[0] = v;
+        for (int d = 1; d <= M; ++d) {
+            if (M > 1) v = v * (uint64_t)(M - d + 1) / (uint64_t)d;  // exact
+            binom[d] = v;
+        }
     }
     if (prec == BS_PREC_FP64) {
         pack_fix(jb, src, meta, static_cast<zfix*>(data) + jb.data_off, tid, nthreads);

@@ -86,10 +86,16 @@ BS_HD int bs_target_chains(int64_t S) {
 // 256 tasks keeps the re-seeding of mid-size jobs as it was: with 2048 (one
 // resident wave) jobs of 2^19 to 2^21 addends also got shorter chunks and the
 // 4096-item batch ran 5 % slower, for no gain on small calls.
-BS_HD int bs_choose_log2L_single(uint64_t C, int cpt, int log2max, int target) {
+// Minors calls of the FP64 and double-float kernels (one job each; column
+// sums are exact, so a chunk start costs only its seeding) spread over
+// BS_TARGET_TASKS_FILL_ONE tasks, about one per resident warp: FP64 minors of
+// 20 columns, 2^18 addends, 144 us in 256 tasks, 60 us in 2048.  Permanents
+// keep 256, so that an item of a batch gives the same bits as a call.
+#define BS_TARGET_TASKS_FILL_ONE 2048
+BS_HD int bs_choose_log2L_single(uint64_t C, int cpt, int log2max, int target, int fill_tasks = BS_TARGET_TASKS_FILL) {
     const int big = bs_choose_log2L(C, cpt, BS_LOG2L_MIN_SINGLE, log2max, target);
     if (big > BS_LOG2L_MIN_SINGLE) return big;
-    int fill = bs_floor_log2(C / ((uint64_t)cpt * (uint64_t)BS_TARGET_TASKS_FILL));
+    int fill = bs_floor_log2(C / ((uint64_t)cpt * (uint64_t)fill_tasks));
     if (fill > BS_LOG2L_MIN_SINGLE) fill = BS_LOG2L_MIN_SINGLE;
     const int floor = C <= BS_FILL_TINY_C ? BS_LOG2L_MIN_FILL : BS_LOG2L_MIN_MANY;
     if (fill < floor) fill = floor;
