@@ -335,8 +335,8 @@ constexpr uint32_t kFixRun = 4;
 // Shared memory of one warp of the minors kernel, HX columns per lane, NP =
 // ceil(HX / 2) leaves: the integer sums [col][lane] (rows of 33, so that
 // neighbouring columns of one lane fall into different banks when a run is
-// flushed), the suffix products and then the m_j [leaf][lane], the leaves
-// [leaf][lane] (at the end of a run the units' exponents), the K
+// flushed), the suffix products and the leaves [leaf][lane] (at the
+// end of a run the units' exponents), the K
 // double-double totals, plain-double sums, and a factor per chunk.
 template <int G, int HX>
 struct MinorsSmem {
@@ -402,24 +402,45 @@ __device__ __forceinline__ void suffix_step(const zraw (&c)[HX], int j, zraw& r,
     e += 64 + kLeafExp;
 }
 
-// One step of a prefix chain: m_j = p S_j (p itself for the chain's last
-// leaf), below 2^61, in S_j's place, its exponent in es[j]; p takes leaf j in.
-template <int NP>
-__device__ __forceinline__ void prefix_step(int j, bool last, zlimb& p, int& e, int (&es)[NP],
-                                            longlong2* __restrict__ sm_leaf, const int4* __restrict__ sm_pair) {
+// One step of a prefix chain.  m_j = p S_j (p itself for the chain's last
+// leaf), below 2^61; times the one column of the pair it is added to the
+// other column's sum, whose unit 2^em follows the run's largest addend (that
+// one comes to [2^60, 2^61): m_j is carried 4 times over, so that its shift
+// is to the right); then p takes leaf j in.
+template <int HX>
+__device__ __forceinline__ void prefix_step(const zraw (&c)[HX], int j, bool last, zlimb& p, int& e, int es, int& em,
+                                            longlong2* __restrict__ sm_acc, const longlong2* __restrict__ sm_leaf,
+                                            const int4* __restrict__ sm_pair) {
     zraw m;
     if (last) {
         m = fix_shr(raw_of(p), 1);
-        es[j] = e + 1;
+        es = e + 1;
     } else {
         const longlong2 v = sm_leaf[j * 32];
         m = fix_cmul<0>(p, *reinterpret_cast<const zlimb*>(&v));
-        es[j] += e + 64;
+        es += e + 64;
         const int4 d = sm_pair[j * 32];
         e += 64 + kLeafExp;
         p = fix_normalise(fix_cmul(p, zlimb{d.x, d.y, d.z, d.w}), e);
     }
-    sm_leaf[j * 32] = make_longlong2((long long)m.re, (long long)m.im);
+    const int up = max(em, es - min(fix_norm_shift(m) - 1, 2));
+    const int dl = min(up - em, 63);
+    em = up;
+    m = fix_shr(zraw{m.re << 2, m.im << 2}, min(up - es + 2, 63));
+    const longlong2 a = sm_acc[2 * j * 33];
+    zraw z = fix_shr(zraw{(unsigned long long)a.x, (unsigned long long)a.y}, dl);
+    if (2 * j + 1 < HX) {
+        const zlimb ml = limbs_of(m);
+        z = fix_cmul_add<1, 1>(z, ml, limbs_of(c[2 * j + 1]));
+        sm_acc[2 * j * 33] = make_longlong2((long long)z.re, (long long)z.im);
+        const longlong2 b = sm_acc[(2 * j + 1) * 33];
+        z = fix_cmul_add<1, 1>(fix_shr(zraw{(unsigned long long)b.x, (unsigned long long)b.y}, dl), ml,
+                               limbs_of(c[2 * j]));
+        sm_acc[(2 * j + 1) * 33] = make_longlong2((long long)z.re, (long long)z.im);
+    } else {  // no partner: m_j itself, in the same unit (m / 2)
+        const zraw h = fix_shr(m, 1);
+        sm_acc[2 * j * 33] = make_longlong2((long long)(z.re + h.re), (long long)(z.im + h.im));
+    }
 }
 
 // G lanes share one chunk: lane G p + q owns the HX columns [q HX, q HX + HX)
@@ -428,11 +449,11 @@ __device__ __forceinline__ void prefix_step(int j, bool last, zlimb& p, int& e, 
 //   1. forms its leaves d_j (column pairs), in two chains their exclusive
 //      suffix products S_j, and the product Q of its columns;
 //   2. takes X, the product of the other lanes' Q, by shuffles;
-//   3. runs the prefix products from X over the chains, m_j = prefix_j S_j:
-//      all columns but those of pair j;
-//   4. adds m_j times the one column of the pair to the other column's sum,
-//      in 64-bit integers whose unit, one per pair and lane, follows the
-//      largest addend of the run (the sums move down when it grows).
+//   3. runs the prefix products from X over the chains; m_j = prefix_j S_j
+//      is all columns but those of pair j, and m_j times the one column of
+//      the pair is added to the other column's sum, in 64-bit integers whose
+//      unit, one per pair and lane, follows the largest addend of the run
+//      (the sums move down when it grows).
 // 3 K - 3 complex products per addend, as any prefix / suffix scheme needs.
 // A task covers 16 chunks, with four lanes per chunk in two rounds.
 //
@@ -449,8 +470,9 @@ __device__ __forceinline__ void prefix_step(int j, bool last, zlimb& p, int& e, 
 // double 2.2e-14; runs of 8 addends 2.0e-14, one unit for the whole warp
 // 3.5e-12 (27 columns), without the sums (one addend per run) 2e-15.
 //
-// Time.  29 x 30 minors (2^28 addends): 190 ms in double, 49.7 ms here (1.42e9 ->
-// 5.40e9 addends/s); the FMA-heavy pipe is 67 % busy
+// Time.  29 x 30 minors (2^28 addends): 190 ms in double, 47.8 ms here (1.42e9 ->
+// 5.62e9 addends/s; 49.7 with the m_j of an addend kept before any is added);
+// the FMA-heavy pipe is 68 % busy
 // with integer products (4.35 cycles per warp and product) and every other
 // integer instruction costs about 1.3 cycles beside them, so what bounds it is
 // the instruction count: 112 per column and addend, 33 of them products.
@@ -542,7 +564,11 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
                 pr = shfl_xor_zlimb(pr, 1);
                 e = __shfl_xor_sync(0xffffffffu, e, 1);
             }
-            // 3. m_j, below 2^61
+            // 3. the prefix chains and the sums
+            if ((s & run_mask) == 0u) {
+#pragma unroll
+                for (int j = 0; j < NP; ++j) em[j] = -(1 << 20);
+            }
             {
                 zlimb pa, pb;
                 int fa = e, fb = e;
@@ -555,38 +581,9 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
                 }
 #pragma unroll
                 for (int i = 0; i < NA; ++i) {
-                    prefix_step(i, i + 1 == NA, pa, fa, es, sm_leaf, sm_pair);
-                    if (i < NB) prefix_step(NA + i, i + 1 == NB, pb, fb, es, sm_leaf, sm_pair);
-                }
-            }
-            // 4. the units of the pairs' sums
-            if ((s & run_mask) == 0u) {
-#pragma unroll
-                for (int j = 0; j < NP; ++j) em[j] = -(1 << 20);
-            }
-#pragma unroll
-            for (int j = 0; j < NP; ++j) {
-                // the largest addend so far comes to [2^60, 2^61): m_j is carried
-                // 4 times over, so that its shift is to the right
-                const longlong2 v = sm_leaf[j * 32];
-                const zraw r = {(unsigned long long)v.x, (unsigned long long)v.y};
-                const int up = max(em[j], es[j] - min(fix_norm_shift(r) - 1, 2));
-                const int dl = min(up - em[j], 63);
-                em[j] = up;
-                const zraw m = fix_shr(zraw{r.re << 2, r.im << 2}, min(up - es[j] + 2, 63));
-                const longlong2 a = sm_acc[2 * j * 33];
-                zraw z = fix_shr(zraw{(unsigned long long)a.x, (unsigned long long)a.y}, dl);
-                if (2 * j + 1 < HX) {
-                    const zlimb ml = limbs_of(m);
-                    z = fix_cmul_add<1, 1>(z, ml, limbs_of(c[2 * j + 1]));
-                    sm_acc[2 * j * 33] = make_longlong2((long long)z.re, (long long)z.im);
-                    const longlong2 b = sm_acc[(2 * j + 1) * 33];
-                    z = fix_cmul_add<1, 1>(fix_shr(zraw{(unsigned long long)b.x, (unsigned long long)b.y}, dl), ml,
-                                           limbs_of(c[2 * j]));
-                    sm_acc[(2 * j + 1) * 33] = make_longlong2((long long)z.re, (long long)z.im);
-                } else {  // no partner: m_j itself, in the same unit (m / 2)
-                    const zraw h = fix_shr(m, 1);
-                    sm_acc[2 * j * 33] = make_longlong2((long long)(z.re + h.re), (long long)(z.im + h.im));
+                    prefix_step<HX>(c, i, i + 1 == NA, pa, fa, es[i], em[i], sm_acc, sm_leaf, sm_pair);
+                    if (i < NB)
+                        prefix_step<HX>(c, NA + i, i + 1 == NB, pb, fb, es[NA + i], em[NA + i], sm_acc, sm_leaf, sm_pair);
                 }
             }
             // the end of a run
