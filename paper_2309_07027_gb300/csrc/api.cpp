@@ -262,8 +262,8 @@ int launch_walk(bs_ctx* c, const bs::WalkArgs& a, int prec, int kind) {
     int rc = record_walk_start(c, &e0);
     if (rc) return rc;
     cudaError_t e;
-    if (prec == BS_PREC_DF)
-        e = kind == BS_KIND_PERM ? bs::launch_walk_df_perm(a, c->stream) : bs::launch_walk_df_minors(a, c->stream);
+    if (BS_DF_MINORS(prec, kind))
+        e = bs::launch_walk_df_minors(a, c->stream);
     else if (prec == BS_PREC_FP32)
         e = kind == BS_KIND_PERM ? bs::launch_walk_fp32_perm(a, c->stream) : bs::launch_walk_fp32_minors(a, c->stream);
     else
@@ -334,7 +334,7 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
         r.prec = job_prec(mode, rule != 0);
         r.reseed = r.prec == BS_PREC_FP32 && rule == 2 ? BS_FP32_RESEED_LOG2 : 0;
         r.kind = in.p->kind;
-        r.bucket = r.prec == BS_PREC_DF ? (in.p->K + 7) >> 3 : (in.p->K + 3) >> 2;
+        r.bucket = BS_DF_MINORS(r.prec, r.kind) ? (in.p->K + 7) >> 3 : (in.p->K + 3) >> 2;
         r.cpt = bs_chunks_per_task(r.kind, r.prec, in.p->K);
         r.ncols = r.kind == BS_KIND_PERM ? 1 : in.p->K;
         const bool lone = r.kind == BS_KIND_MINORS && r.prec != BS_PREC_FP32;  // (minors never come in batches)
@@ -408,7 +408,7 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
             meta.push_back(p.pinned_src);
             meta.push_back(0);                                           // pad to 8 bytes
             meta.insert(meta.end(), (size_t)2 * (p.nrows + p.n), 0);     // binomial table (pack kernel)
-            data_off[arena_of(r.prec)] += (int64_t)(1 + p.nrows) * BS_ROW_STRIDE_P(p.K, r.prec);
+            data_off[arena_of(r.prec)] += (int64_t)(1 + p.nrows) * BS_ROW_STRIDE_P(p.K, r.prec, r.kind);
             part_off += (int64_t)r.ntasks * r.ncols;
             tb += r.ntasks;
             max_cols = std::max(max_cols, r.ncols);

@@ -194,9 +194,7 @@ extern "C" int bs_perm_noalloc(const bs_c128* A, int rows, int cols, int ld, con
     w.counter = reinterpret_cast<unsigned long long*>(scr + kCtl);
     w.status = reinterpret_cast<int*>(scr + kCtl + 8);
     w.max_K = p.K;
-    NA_CUDA(prec == BS_PREC_DF     ? bs::launch_walk_df_perm(w, s)
-            : prec == BS_PREC_FP32 ? bs::launch_walk_fp32_perm(w, s)
-                                   : bs::launch_walk_fp64_perm(w, s));
+    NA_CUDA(prec == BS_PREC_FP32 ? bs::launch_walk_fp32_perm(w, s) : bs::launch_walk_fp64_perm(w, s));
     NA_CUDA(bs::launch_reduce(djob, 1, w.partials, dmeta, reinterpret_cast<double2*>(scr + kOut),
                               reinterpret_cast<double2*>(scr + kOut + 16), 1, s));
     double2 res[2];

@@ -1,5 +1,6 @@
-// Double-float walk kernels (walk_df.cuh): permanents and fused Laplace
-// minors with FP64-class accuracy on the FP32 pipe.  One instantiation per
+// Double-float walk kernels (walk_df.cuh): fused Laplace minors with
+// FP64-class accuracy on the FP32 pipe (double-float permanents run in the
+// FP64 kernels, 1.3 times as fast at 30 columns).  One instantiation per
 // 8-column bucket (K in (KB - 8, KB]); persistent grids pull warp tasks from
 // an atomic counter, as the FP64 and FP32 kernels do.
 #include "kernels.h"
@@ -8,26 +9,6 @@
 namespace bs {
 
 constexpr int kDfBlock = 128;
-
-template <int KB>
-__global__ void __launch_bounds__(kDfBlock) walk_df_perm_kernel(WalkArgs a) {
-    const int lane = threadIdx.x & 31;
-    const bs_job* __restrict__ jobs = a.jobs;
-    const unsigned long long total = task_total(a);
-    const int njobs = job_count(a);
-    const unsigned long long deadline = warp_deadline(a.deadline_rel_ns);
-    for (;;) {
-        unsigned long long t = next_task(a.counter, total, a.status, deadline, lane);
-        if (t >= total) break;
-        const bs_job jb = jobs[find_job(jobs, a.job_list, njobs, t)];
-        if (((jb.K + 7) >> 3) != KB / 8 || jb.kind != BS_KIND_PERM) {
-            if (lane == 0) atomicExch(a.status, BS_STATUS_BADJOB);
-            continue;
-        }
-        walk_task_perm_df<KB>(jb, a.data, a.meta + BS_META_RADIX(jb), a.partials,
-                              (uint32_t)(t - jb.task_begin) + jb.task_offset, lane);
-    }
-}
 
 // Resident CTAs per SM the fused-minor kernel is compiled for (register
 // cap 65536 / (128 x value)): 3 at widths 24 and 48 (three pairs per lane,
@@ -87,13 +68,6 @@ static int persistent_grid(Kern k, int block, size_t smem, const WalkArgs& a) {
 }
 
 template <int KB>
-static cudaError_t run_perm(const WalkArgs& a, cudaStream_t s) {
-    int grid = persistent_grid(walk_df_perm_kernel<KB>, kDfBlock, 0, a);
-    walk_df_perm_kernel<KB><<<grid, kDfBlock, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-template <int KB>
 static cudaError_t run_minors(const WalkArgs& a, cudaStream_t s) {
     // per owned column and thread: a float4 fold slot and a float4 staging slot
     const size_t smem = (size_t)kDfBlock * (KB / BS_DF_GROUP_KB(KB)) * 2 * sizeof(float4);
@@ -108,17 +82,6 @@ static cudaError_t run_minors(const WalkArgs& a, cudaStream_t s) {
 #define BS_DF_B48(X) X(1, 8) X(2, 16) X(3, 24) X(4, 32) X(5, 40) X(6, 48)
 
 // a.max_K selects the 8-column bucket: every job of the launch must share it.
-cudaError_t launch_walk_df_perm(const WalkArgs& a, cudaStream_t s) {
-    if (a.total_tasks == 0 && !a.total_dev) return cudaSuccess;
-    switch ((a.max_K + 7) >> 3) {
-#define BS_CASE(b, kb) \
-    case b: return run_perm<kb>(a, s);
-        BS_DF_B48(BS_CASE)
-#undef BS_CASE
-    }
-    return cudaErrorInvalidValue;
-}
-
 cudaError_t launch_walk_df_minors(const WalkArgs& a, cudaStream_t s) {
     if (a.total_tasks == 0 && !a.total_dev) return cudaSuccess;
     switch ((a.max_K + 7) >> 3) {

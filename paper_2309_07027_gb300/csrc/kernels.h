@@ -28,8 +28,7 @@ cudaError_t launch_walk_fp64_perm(const WalkArgs& a, cudaStream_t s);
 cudaError_t launch_walk_fp64_minors(const WalkArgs& a, cudaStream_t s);
 cudaError_t launch_walk_fp32_perm(const WalkArgs& a, cudaStream_t s);
 cudaError_t launch_walk_fp32_minors(const WalkArgs& a, cudaStream_t s);
-// Double-float kernels: 8-column buckets (max_K selects (K + 7) / 8).
-cudaError_t launch_walk_df_perm(const WalkArgs& a, cudaStream_t s);
+// Double-float minors: 8-column buckets (max_K selects (K + 7) / 8).
 cudaError_t launch_walk_df_minors(const WalkArgs& a, cudaStream_t s);
 
 // Builds c0 / 2a (and column scales) of every job from its source matrix.

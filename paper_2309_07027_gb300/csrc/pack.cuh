@@ -3,12 +3,13 @@
 // (every delta = +1) and 2a[j][col] for every digit row, rows of stride KP.
 // Every column is scaled by a power of two whose exponent goes to colexp[col]
 // and is undone exactly by the reduce kernel.
-// FP64 jobs: 64-bit fixed point (pack_fix below, walk_fix.cuh).
+// FP64 jobs and double-float permanents: 64-bit fixed point (pack_fix below,
+// walk_fix.cuh).
 // FP32 jobs: c0 in double-double, rounded; column pairs {re(2p), re(2p+1),
 // im(2p), im(2p+1)} (the packed layout of walk_fp32.cuh), column col scaled
 // by 2^-e (e: smallest integer with sum_rows M_row (|Re a| + |Im a|) <= 2^e);
 // pad columns have zero rows and c0 = 1 (a neutral factor).
-// Double-float (DF) jobs: rows of stride BS_ROW_STRIDE_DF(K) (a multiple of
+// Double-float (DF) minors: rows of stride BS_ROW_STRIDE_DF(K) (a multiple of
 // 8), column col scaled by 2^(2 - e) (colexp = e - 2) so that every column
 // sum has |Re|, |Im| <= 4, and every entry quantised to a high part on the
 // grid 2^-20 and a low part on the grid 2^-44, both exact floats
@@ -156,7 +157,7 @@ __device__ __forceinline__ void pack_fix(const bs_job& jb, const double2* __rest
 
 __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __restrict__ src, int* __restrict__ meta,
                          void* __restrict__ data, int prec, int tid, int nthreads) {
-    const int df = prec == BS_PREC_DF;
+    const int df = BS_DF_MINORS(prec, jb.kind);
     const int* radix = meta + BS_META_RADIX(jb);
     const int* dsrc = meta + BS_META_DIGIT_SRC(jb);
     const int* csrc = meta + BS_META_COL_SRC(jb);
@@ -174,7 +175,7 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
             binom[d] = v;
         }
     }
-    if (prec == BS_PREC_FP64) {
+    if (prec != BS_PREC_FP32 && !df) {
         pack_fix(jb, src, meta, static_cast<zfix*>(data) + jb.data_off, tid, nthreads);
         return;
     }

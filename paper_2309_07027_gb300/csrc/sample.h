@@ -117,15 +117,15 @@ BS_HD int bs_minors_fp32_group(int K) { return BS_MINORS_FP32_GROUP_KB((K + 3) &
 // 32 columns two lanes need 255 registers and run 7-24 % slower than four).
 // A warp task covers 16 chunks either way, in one or two rounds.
 #define BS_MINORS_FP64_GROUP_KB(KB) ((KB) > 32 ? 4 : 2)
-// Lanes per chunk of the double-float kernels (permanent and minors), by
+// Lanes per chunk of the double-float minors, by
 // 8-column bucket width KB: each lane owns KB / (2G) column pairs
 // (8 -> 1 x 4, 16 -> 2 x 4, 24 -> 4 x 3, 32 -> 4 x 4, 40 -> 4 x 5,
 // 48 -> 8 x 3), so a lane's double-float state fits its registers.
 #define BS_DF_GROUP_KB(KB) ((KB) <= 8 ? 1 : (KB) <= 16 ? 2 : (KB) <= 40 ? 4 : 8)
 BS_HD int bs_df_group(int K) { return BS_DF_GROUP_KB((K + 7) & ~7); }
 BS_HD int bs_chunks_per_task(int kind, int prec, int K) {
-    if (prec == BS_PREC_DF) return 32 / bs_df_group(K);
     if (kind != BS_KIND_MINORS) return 32;
+    if (prec == BS_PREC_DF) return 32 / bs_df_group(K);
     return prec == BS_PREC_FP32 ? 32 / bs_minors_fp32_group(K) : 16;  // FP64 minors
 }
 

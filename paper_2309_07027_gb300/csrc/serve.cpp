@@ -211,7 +211,7 @@ size_t request_bytes(const Request& r) {
     auto up = [](size_t b) { return (b + kAlign - 1) / kAlign * kAlign; };
     size_t b = 0;
     b += up((size_t)r.rows * r.cols * 16);                          // source matrix
-    b += up((size_t)(1 + p.nrows) * BS_ROW_STRIDE_P(p.K, r.prec) * 16);  // packed c0 / 2a
+    b += up((size_t)(1 + p.nrows) * BS_ROW_STRIDE_P(p.K, r.prec, r.kind) * 16);  // packed c0 / 2a
     b += up((size_t)BS_META_SIZE(p.nrows, p.K, p.n) * 4);                // metadata
     b += up((size_t)r.ntasks * r.ncols * sizeof(bs_zdd));            // task partials
     return b;
@@ -257,7 +257,7 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
             return o;
         };
         const size_t src_b = take((size_t)r->rows * r->cols * 16);
-        const size_t data_b = take((size_t)(1 + p.nrows) * BS_ROW_STRIDE_P(p.K, r->prec) * 16);
+        const size_t data_b = take((size_t)(1 + p.nrows) * BS_ROW_STRIDE_P(p.K, r->prec, r->kind) * 16);
         const size_t meta_b = take((size_t)BS_META_SIZE(p.nrows, p.K, p.n) * 4);
         const size_t part_b = take((size_t)r->ntasks * r->ncols * sizeof(bs_zdd));
         r->src_off = (int64_t)(src_b / 16);
@@ -334,8 +334,8 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
     // sort into kernel groups, largest slices first
     std::vector<size_t> order(walk.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = i;
-    // kernel bucket of a job: 4-column buckets, 8-column for double-float
-    auto bucket = [](const bs_job& j) { return j.prec == BS_PREC_DF ? (j.K + 7) / 8 : (j.K + 3) / 4; };
+    // kernel bucket of a job: 4-column buckets, 8-column for double-float minors
+    auto bucket = [](const bs_job& j) { return BS_DF_MINORS(j.prec, j.kind) ? (j.K + 7) / 8 : (j.K + 3) / 4; };
     std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) {
         const bs_job &x = walk[a], &y = walk[b];
         if (x.prec != y.prec) return x.prec < y.prec;
@@ -474,12 +474,12 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
             kmax = std::max(kmax, tick[i].K);
         }
         w.total_tasks = tot;
-        w.counter = ctl + gi;  // at most 2 x 2 x 12 + 2 x 6 = 60 groups
+        w.counter = ctl + gi;  // at most 2 x 12 (FP32) + 12 + 6 (DF) = 42 groups
         w.status = reinterpret_cast<int*>(ctl + 64);
         w.max_K = kmax;
         const bs_job& g0 = tick[groups[gi].first];
-        if (g0.prec == BS_PREC_DF)
-            e = g0.kind == BS_KIND_PERM ? bs::launch_walk_df_perm(w, s->stream) : bs::launch_walk_df_minors(w, s->stream);
+        if (BS_DF_MINORS(g0.prec, g0.kind))
+            e = bs::launch_walk_df_minors(w, s->stream);
         else if (g0.prec == BS_PREC_FP32)
             e = g0.kind == BS_KIND_PERM ? bs::launch_walk_fp32_perm(w, s->stream) : bs::launch_walk_fp32_minors(w, s->stream);
         else

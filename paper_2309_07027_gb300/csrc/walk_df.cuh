@@ -81,7 +81,6 @@ struct dfst {
 __device__ __forceinline__ dfc df_one() {
     return dfc{make_float2(1.f, 1.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 }
-__device__ __forceinline__ dfc df_drop(const dfy& y) { return dfc{y.rh, y.rl, y.ih, y.il}; }
 
 // c += sg * A (A: packed high / low parts of one row pair), exact, then the
 // carry of the low part into the high part.
@@ -459,89 +458,6 @@ __device__ void walk_task_minors_df(const bs_job& jb, const void* __restrict__ d
             store_partial(partials + jb.partial_off + (int64_t)local * K + cbase + t, dd_from_dfs(re),
                           dd_from_dfs(im));
     }
-}
-
-// ---------------------------------------------------------------- one task: permanent
-// G lanes share one chunk, each owning NP column pairs; per addend a lane
-// forms the product of its pairs (two packed chains), Q = Q_even Q_odd, and
-// the G lanes multiply their Q in a butterfly; lane q = 0 of each group adds
-// (+-W) prod Q to its Sum2 accumulator, folded into a double-float total
-// every FOLD addends.
-template <int KB>
-__device__ void walk_task_perm_df(const bs_job& jb, const void* __restrict__ data_v, const int* __restrict__ radix,
-                                  bs_zdd* __restrict__ partials, uint32_t local, int lane) {
-    constexpr uint32_t FOLD = 64;
-    constexpr int G = BS_DF_GROUP_KB(KB);
-    constexpr int NP = KB / (2 * G);
-    constexpr int CPT = 32 / G;
-    static_assert(KB % (2 * G) == 0, "bucket must split into G groups of column pairs");
-    const int q = lane & (G - 1);
-    const int p0 = q * NP;
-    const float4* c0 = static_cast<const float4*>(data_v) + jb.data_off;
-    const float4* a2 = c0 + KB;
-    const uint64_t i0_own = ((uint64_t)local * CPT + (uint64_t)(lane / G)) << jb.log2L;
-    const bool has = i0_own < jb.C;
-    const uint64_t i0 = has ? i0_own : 0ull;
-    uint32_t len = 0;
-    if (has) {
-        const uint64_t rem = jb.C - i0;
-        len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
-    }
-    const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
-    bs_gray g;
-    ChunkStepper st;
-    st.init(g, i0, jb.nbin, jb.nrows, radix, reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
-    dfst c[NP];
-    df_seed<NP>(c, g, c0, a2, KB, p0, jb.nbin, jb.nrows);
-    dfs ws = has ? df_weight(g.w, g.parity) : dfs{0.f, 0.f};
-    dfs are = {0.f, 0.f}, aim = {0.f, 0.f};   // Sum2 state
-    dfs tre = {0.f, 0.f}, tim = {0.f, 0.f};   // folded totals
-    for (uint32_t s = 0; s < steps; ++s) {
-        dfc pr = df_norm(c[NP - 1]);
-#pragma unroll
-        for (int p = NP - 2; p >= 0; --p) pr = df_cmul(pr, df_norm_neg(c[p]));
-        dfsc Q = s_cmul(df_half(pr, 0), df_half(pr, 1));
-        if constexpr (G > 1) {
-            Q = s_cmul(Q, shfl_xor_dfsc(Q, 1));
-            if constexpr (G >= 4) Q = s_cmul(Q, shfl_xor_dfsc(Q, 2));
-            if constexpr (G >= 8) Q = s_cmul(Q, shfl_xor_dfsc(Q, 4));
-        }
-        const dfsc a = s_rmul(ws, Q);
-        // Sum2: TwoSum of the high parts, errors and low parts in l
-        const dfs sr = s_two_sum(are.h, a.re.h);
-        are = dfs{sr.h, __fadd_rn(are.l, __fadd_rn(sr.l, a.re.l))};
-        const dfs si = s_two_sum(aim.h, a.im.h);
-        aim = dfs{si.h, __fadd_rn(aim.l, __fadd_rn(si.l, a.im.l))};
-        if (((s + 1u) & (FOLD - 1u)) == 0) {
-            tre = s_add(tre, s_two_sum(are.h, are.l));
-            tim = s_add(tim, s_two_sum(aim.h, aim.l));
-            are = aim = dfs{0.f, 0.f};
-        }
-        if (s + 1u >= steps) break;
-        if (s + 1u >= len) {
-            ws = dfs{0.f, 0.f};
-            continue;
-        }
-        uint32_t neg;
-        int wch;
-        const int row = st.step(g, s, radix, &neg, &wch);
-        ws = wch ? df_weight(g.w, g.parity) : dfs{-ws.h, -ws.l};
-        const float2 sg = p_splat(neg ? -1.0f : 1.0f);
-        const float4* rp = a2 + (size_t)row * KB;
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            float4 h, l;
-            df_load_pair(rp, p0 + p, h, l);
-            df_update(c[p], h, l, sg);
-        }
-    }
-    tre = s_add(tre, s_two_sum(are.h, are.l));
-    tim = s_add(tim, s_two_sum(aim.h, aim.l));
-    // lanes q = 0 hold the chunk totals; combine them over the task
-    if (q != 0) tre = tim = dfs{0.f, 0.f};
-    ddv re = dd_from_dfs(tre), im = dd_from_dfs(tim);
-    warp_reduce_zdd(re, im);
-    if (lane == 0) store_partial(partials + jb.partial_off + local, re, im);
 }
 
 }  // namespace bs
