@@ -313,8 +313,8 @@ struct ChainDesc {
     const int* inputs;      // n expanded input columns
     int* cols;              // n permuted columns
     int* rows;              // n drawn rows
-    int* counts;            // m_det occupation counts (written after step n)
-    bs_job* job;            // the chain's job descriptor
+    int* counts;            // m_det occupation counts (written after step n; pinned host memory)
+    bs_job* job;            // the next step's job descriptor (before step n; pinned host memory)
     int64_t meta_off;       // int units
     int64_t data_byte_off;  // bytes (16-byte aligned)
     int64_t partial_off;    // bs_zdd units
