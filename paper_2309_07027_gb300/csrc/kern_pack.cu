@@ -17,7 +17,7 @@
 
 namespace bs {
 
-__global__ void pack_kernel(const bs_job* __restrict__ jobs, const double2* __restrict__ src, int* __restrict__ meta,
+__global__ void __launch_bounds__(kPackBlock) pack_kernel(const bs_job* __restrict__ jobs, const double2* __restrict__ src, int* __restrict__ meta,
                             void* __restrict__ data, int prec) {
     const bs_job jb = jobs[blockIdx.x];
     pack_job(jb, src, meta, data, prec, threadIdx.x, blockDim.x);
@@ -26,7 +26,7 @@ __global__ void pack_kernel(const bs_job* __restrict__ jobs, const double2* __re
 cudaError_t launch_pack(const bs_job* jobs, int njobs, const double2* src, int* meta, void* data, int prec,
                         cudaStream_t s) {
     if (njobs <= 0) return cudaSuccess;
-    pack_kernel<<<njobs, 64, 0, s>>>(jobs, src, meta, data, prec);
+    pack_kernel<<<njobs, kPackBlock, 0, s>>>(jobs, src, meta, data, prec);
     return cudaGetLastError();
 }
 
@@ -47,12 +47,6 @@ __device__ __forceinline__ ddv sum2_final(ddv a) {
     const double h = __dadd_rn(a.hi, a.lo);
     const double bb = __dsub_rn(h, a.hi);
     return ddv{h, __dadd_rn(__dsub_rn(a.hi, __dsub_rn(h, bb)), __dsub_rn(a.lo, bb))};
-}
-
-// x 2^e: one multiplication where 2^e is a normal double (the same rounding
-// as ldexp, whose general form takes several times as long).
-__device__ __forceinline__ double scale2(double x, int e) {
-    return abs(e) <= 1000 ? x * __hiloint2double((1023 + e) << 20, 0) : ldexp(x, e);
 }
 
 // One CTA per (job, output column).  A CTA's time is its chain of dependent

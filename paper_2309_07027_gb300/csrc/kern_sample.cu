@@ -178,7 +178,7 @@ __device__ int plan_minors_step(const int* __restrict__ rows, const int* __restr
 }
 
 // Plan + pack the step-k minors job of every chain (one CTA per chain).
-__global__ void cc_plan_kernel(const CcArgs* __restrict__ pa, int k) {
+__global__ void __launch_bounds__(kPackBlock) cc_plan_kernel(const CcArgs* __restrict__ pa, int k) {
     const CcArgs& a = *pa;
     __shared__ int urow[BS_MAX_PHOTONS], ucnt[BS_MAX_PHOTONS];
     __shared__ int drad[BS_MAX_PHOTONS], dsrc[BS_MAX_PHOTONS];
@@ -355,7 +355,7 @@ __global__ void chain_init_kernel(const ChainDesc* __restrict__ list, int count)
     }
 }
 
-__global__ void chain_advance_kernel(const ChainDesc* __restrict__ list, void* __restrict__ arena,
+__global__ void __launch_bounds__(kPackBlock) chain_advance_kernel(const ChainDesc* __restrict__ list, void* __restrict__ arena,
                                      const double2* __restrict__ minors_base) {
     extern __shared__ double wts[];
     __shared__ int urow[BS_MAX_PHOTONS], ucnt[BS_MAX_PHOTONS];
@@ -409,7 +409,7 @@ cudaError_t launch_chain_advance(const ChainDesc* d, int count, int max_m_rows, 
             cudaFuncSetAttribute(chain_advance_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    chain_advance_kernel<<<count, 128, smem, st>>>(d, arena, minors_base);
+    chain_advance_kernel<<<count, kPackBlock, smem, st>>>(d, arena, minors_base);
     return cudaGetLastError();
 }
 
@@ -423,7 +423,7 @@ cudaError_t launch_cc_init(const CcArgs& a, const CcArgs* da, cudaStream_t st) {
 }
 
 cudaError_t launch_cc_plan(const CcArgs& a, const CcArgs* da, int k, cudaStream_t st) {
-    cc_plan_kernel<<<a.S, 64, 0, st>>>(da, k);
+    cc_plan_kernel<<<a.S, kPackBlock, 0, st>>>(da, k);
     return cudaGetLastError();
 }
 

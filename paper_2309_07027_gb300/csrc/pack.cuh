@@ -3,9 +3,9 @@
 // (every delta = +1) and 2a[j][col] for every digit row, rows of stride KP.
 // Every column is scaled by a power of two whose exponent goes to colexp[col]
 // and is undone exactly by the reduce kernel.
-// FP64 jobs and double-float permanents: 64-bit fixed point (pack_fix below,
+// FP64 jobs and double-float permanents: 64-bit fixed point (pack_job below,
 // walk_fix.cuh).
-// FP32 jobs: c0 in double-double, rounded; column pairs {re(2p), re(2p+1),
+// FP32 jobs: c0 exact, rounded once to double, then to float; column pairs {re(2p), re(2p+1),
 // im(2p), im(2p+1)} (the packed layout of walk_fp32.cuh), column col scaled
 // by 2^-e (e: smallest integer with sum_rows M_row (|Re a| + |Im a|) <= 2^e);
 // pad columns have zero rows and c0 = 1 (a neutral factor).
@@ -24,6 +24,9 @@
 
 namespace bs {
 
+constexpr int kPackLanes = 8;    // lanes per column
+constexpr int kPackBlock = 256;  // threads per job: 32 columns in one round
+
 __device__ __forceinline__ double2 src_elem(const double2* __restrict__ src, const bs_job& jb, int r, int c) {
     return jb.src_trans ? src[jb.src_off + (int64_t)c * jb.src_ld + r] : src[jb.src_off + (int64_t)r * jb.src_ld + c];
 }
@@ -35,14 +38,71 @@ __device__ __forceinline__ void put_f32(void* data, const bs_job& jb, int KP, in
     q[2] = im;
 }
 
-// The DF split of v (|v| < 16): hi = v rounded to the grid 2^-20, lo = the
-// rest rounded to the grid 2^-44; vlo: a low-order double added to v
-// (double-double input), 0 otherwise.
-__device__ __forceinline__ float2 df_quantise(double v, double vlo) {
-    const double hi = rint(v * 0x1p20) * 0x1p-20;
-    const double rest = (v - hi) + vlo;  // v - hi is exact
-    const double lo = rint(rest * 0x1p44) * 0x1p-44;
-    return make_float2((float)hi, (float)lo);
+// x 2^e: one multiplication where 2^e is a normal double (the same rounding
+// as ldexp, whose general form takes several times as long).
+__device__ __forceinline__ double scale2(double x, int e) {
+    return abs(e) <= 1000 ? x * __hiloint2double((1023 + e) << 20, 0) : ldexp(x, e);
+}
+
+// FP32 and DF start sums are formed in 128-bit integers of unit
+// 2^(e - kWideBits) for a column scaled by 2^-e: exact for entries down to
+// 2^-68 of the column's bound (smaller ones lose what lies below 2^-120 of
+// it), in any order of the rows, and without the double-double additions
+// that an FP64 pipe of one instruction in 64 cycles makes the longest part
+// of the packing.
+constexpr int kWideBits = 120;
+
+// x 2^(kWideBits - e), truncated; x finite, |x| <= 2^(e + 2).
+__device__ __forceinline__ __int128 wide_of(double x, int e) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    int ex = (int)(b >> 52) & 0x7ff;
+    unsigned long long m = b & 0xfffffffffffffull;
+    if (ex)
+        m |= 1ull << 52;
+    else
+        ex = 1;
+    const int s = ex - 1075 - e + kWideBits;
+    const unsigned __int128 v = s >= 0 ? (unsigned __int128)m << min(s, 127) : (unsigned __int128)(s > -64 ? m >> -s : 0ull);
+    return (long long)b < 0 ? -(__int128)v : (__int128)v;
+}
+
+// The wide integer v as a double, rounded to nearest.
+__device__ __forceinline__ double wide_double(__int128 v) {
+    const unsigned __int128 u = v < 0 ? -(unsigned __int128)v : (unsigned __int128)v;
+    if (u == 0) return 0.0;
+    const unsigned long long hi = (unsigned long long)(u >> 64);
+    const int lz = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(unsigned long long)u);
+    const unsigned __int128 n = u << lz;
+    // 64 leading bits and a sticky bit below them: one rounding
+    const unsigned long long top = (unsigned long long)(n >> 64) | ((unsigned long long)n != 0ull ? 1ull : 0ull);
+    const double d = scale2(__ull2double_rn(top), 64 - lz - kWideBits);
+    return v < 0 ? -d : d;
+}
+
+// v / 2^S rounded to the nearest integer, halves to even.
+template <int S>
+__device__ __forceinline__ int wide_round(__int128 v) {
+    const unsigned __int128 r = (unsigned __int128)v & (((unsigned __int128)1 << S) - 1), half = (unsigned __int128)1 << (S - 1);
+    const int q = (int)(v >> S);
+    return q + (int)(r > half || (r == half && (q & 1)));
+}
+
+// The DF split of v 2^-kWideBits (magnitude < 16): hi = v rounded to the grid
+// 2^-20, lo = the rest rounded to the grid 2^-44, both exact floats.
+__device__ __forceinline__ float2 df_split(__int128 v) {
+    const int h = wide_round<kWideBits - 20>(v);
+    const int l = wide_round<kWideBits - 44>(v - ((__int128)h << (kWideBits - 20)));
+    return make_float2(__int2float_rn(h) * 0x1p-20f, __int2float_rn(l) * 0x1p-44f);
+}
+
+__device__ __forceinline__ __int128 wide_add_lanes(__int128 v) {  // over the lanes of a column
+#pragma unroll
+    for (int m = 1; m < kPackLanes; m <<= 1) {
+        const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)v, m);
+        const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(v >> 64), m);
+        v += (__int128)(((unsigned __int128)hi << 64) | lo);
+    }
+    return v;
 }
 
 // Element (row r, column col) of a DF job's packed rows.
@@ -54,110 +114,31 @@ __device__ __forceinline__ void put_df(void* data, const bs_job& jb, int KP, int
     q[6] = im.y;
 }
 
-// Fixed-point rows of an FP64 job (walk_fix.cuh): column col scaled by
+// One job.  A column's entries are read once, by kPackLanes lanes with every
+// eighth digit row each, all loads in flight together: a small job's packing
+// is a chain of dependent loads (metadata, then the source, which may be in
+// host memory) and of FP64 instructions, and both are as short as the lanes
+// make them.  Sums over a column's rows are combined in a fixed order, the
+// integer ones exactly, so the result does not depend on the block size.
+// One FP32 job of 25 rows and 26 columns: 68 us with a thread per column and
+// double-double sums, 11 us so; a sampler step's planning and packing at 26
+// columns 87 -> 17 us; an FP64 job of 20 columns 15 -> 8 us.
+//
+// FP64 jobs and double-float permanents (walk_fix.cuh): column col scaled by
 // 2^(63 - e), e (stored in colexp) the smallest integer with 2^e > b (1 +
 // 2^-20), b = sum over rows of M_row (|Re a| + |Im a|); every entry rounded
-// once to an integer, c0 and 2a formed from those integers modulo 2^64.  Ryser and Nijenhuis-Wilf jobs:
-// product column col is matrix row sc; digit j is matrix column dsrc[j],
-// added with +1 when it enters the subset, so the packed row is -a (the walk
-// subtracts rows of digits whose Delta is 1); start sums 0 (Ryser) or
-// x = a_(sc, n-1) - (sum_j a_(sc, j)) / 2 (Nijenhuis-Wilf, whose entries are
-// rounded to even integers so that the half is exact).  A column with an
-// entry that is not finite gets zeros and BS_COLEXP_NAN_*: the reduce kernel
-// writes NaN wherever such a column enters the product.
-__device__ __forceinline__ void pack_fix(const bs_job& jb, const double2* __restrict__ src, int* __restrict__ meta,
-                                         zfix* __restrict__ out, int tid, int nthreads) {
-    const int* radix = meta + BS_META_RADIX(jb);
-    const int* dsrc = meta + BS_META_DIGIT_SRC(jb);
-    const int* csrc = meta + BS_META_COL_SRC(jb);
-    int* colexp = meta + BS_META_COLEXP(jb);
-    const int prow = meta[BS_META_PINNED(jb)];
-    const int KP = BS_ROW_STRIDE(jb.K);
-    const bool bbfg = jb.formula == BS_JOB_BBFG, nw = jb.formula == BS_JOB_NW;
-    // four lanes per column, each with every fourth digit row: the packing of
-    // a small job is a chain of dependent loads, and this one is a quarter as
-    // long (12 photons: 12.1 -> 7.1 us); the sums are combined in a fixed
-    // order, the integer ones exactly.
-    const int part = tid & 3;
-    for (int base = 0; base < KP; base += nthreads >> 2) {  // (every lane runs every round)
-        const int col = base + (tid >> 2);
-        const bool live = col < jb.K;
-        const int sc = csrc[live ? col : 0];
-        const bool first = part == 0 && (bbfg || nw);  // this lane also takes the start row
-        const int frow = bbfg ? prow : jb.n - 1;
-        double bre = 0.0, bim = 0.0;
-        if (first) {
-            const double2 a = src_elem(src, jb, frow, sc);
-            bre = fabs(a.x);
-            bim = fabs(a.y);
-        }
-#pragma unroll 2
-        for (int j = part; j < jb.nrows; j += 4) {
-            const double2 d = src_elem(src, jb, dsrc[j], sc);
-            const double m = bbfg ? (double)(radix[j] - 1) : 1.0;
-            bre += m * fabs(d.x);
-            bim += m * fabs(d.y);
-        }
-        bre += __shfl_xor_sync(0xffffffffu, bre, 1);
-        bim += __shfl_xor_sync(0xffffffffu, bim, 1);
-        bre += __shfl_xor_sync(0xffffffffu, bre, 2);
-        bim += __shfl_xor_sync(0xffffffffu, bim, 2);
-        int flags = 0;
-        if (!isfinite(bre)) flags |= BS_COLEXP_NAN_RE;
-        if (!isfinite(bim)) flags |= BS_COLEXP_NAN_IM;
-        int e = 0;
-        const double b = 0.25 * bre + 0.25 * bim;  // a quarter: b must not overflow
-        if (!flags && b > 0.0) {
-            (void)frexp(b * (1.0 + 0x1p-20), &e);
-            e += 2;
-        }
-        const bool use = live && !flags;
-        const int sh = nw ? 62 - e : 63 - e;
-        unsigned long long sre = 0, sim = 0;  // the start sums
-        if (use && first) {
-            const double2 a = src_elem(src, jb, frow, sc);
-            sre = (unsigned long long)__double2ll_rn(ldexp(a.x, sh));
-            sim = (unsigned long long)__double2ll_rn(ldexp(a.y, sh));
-        }
-#pragma unroll 2
-        for (int j = part; j < jb.nrows; j += 4) {
-            zfix row = {0, 0};
-            if (use) {
-                const double2 d = src_elem(src, jb, dsrc[j], sc);
-                const unsigned long long qre = (unsigned long long)__double2ll_rn(ldexp(d.x, sh));
-                const unsigned long long qim = (unsigned long long)__double2ll_rn(ldexp(d.y, sh));
-                if (bbfg) {
-                    const unsigned long long m = (unsigned long long)(radix[j] - 1);
-                    sre += m * qre;
-                    sim += m * qim;
-                    row.re = (long long)(2ull * qre);
-                    row.im = (long long)(2ull * qim);
-                } else {
-                    // Nijenhuis-Wilf start: 2 x = 2 a_last - sum over all
-                    // columns = a_last - sum over the digits, in even units
-                    sre -= nw ? qre : 0ull;
-                    sim -= nw ? qim : 0ull;
-                    row.re = -(long long)(qre << (nw ? 1 : 0));
-                    row.im = -(long long)(qim << (nw ? 1 : 0));
-                }
-            }
-            if (col < KP) out[(size_t)(1 + j) * KP + col] = row;
-        }
-        sre += __shfl_xor_sync(0xffffffffu, sre, 1);
-        sim += __shfl_xor_sync(0xffffffffu, sim, 1);
-        sre += __shfl_xor_sync(0xffffffffu, sre, 2);
-        sim += __shfl_xor_sync(0xffffffffu, sim, 2);
-        if (part == 0 && col < KP) {
-            // a pad column's sum is exactly 1 = 2^62 / 2^63 2^1
-            out[col] = live ? zfix{(long long)sre, (long long)sim} : zfix{1ll << 62, 0};
-            if (live) colexp[col] = flags ? flags : e;
-        }
-    }
-}
-
+// once to an integer, c0 and 2a formed from those integers modulo 2^64.
+// Ryser and Nijenhuis-Wilf jobs: product column col is matrix row sc; digit j
+// is matrix column dsrc[j], added with +1 when it enters the subset, so the
+// packed row is -a (the walk subtracts rows of digits whose Delta is 1);
+// start sums 0 (Ryser) or x = a_(sc, n-1) - (sum_j a_(sc, j)) / 2
+// (Nijenhuis-Wilf, whose entries are rounded to even integers so that the
+// half is exact).
+// A column with an entry that is not finite gets zeros and BS_COLEXP_NAN_*:
+// the reduce kernel writes NaN wherever such a column enters the product.
 __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __restrict__ src, int* __restrict__ meta,
-                         void* __restrict__ data, int prec, int tid, int nthreads) {
-    const int df = BS_DF_MINORS(prec, jb.kind);
+                                         void* __restrict__ data, int prec, int tid, int nthreads) {
+    const bool df = BS_DF_MINORS(prec, jb.kind), f32 = prec == BS_PREC_FP32;
     const int* radix = meta + BS_META_RADIX(jb);
     const int* dsrc = meta + BS_META_DIGIT_SRC(jb);
     const int* csrc = meta + BS_META_COL_SRC(jb);
@@ -175,58 +156,114 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
             binom[d] = v;
         }
     }
-    if (prec != BS_PREC_FP32 && !df) {
-        pack_fix(jb, src, meta, static_cast<zfix*>(data) + jb.data_off, tid, nthreads);
-        return;
-    }
     const int KP = df ? BS_ROW_STRIDE_DF(jb.K) : BS_ROW_STRIDE(jb.K);
-    for (int col = tid; col < KP; col += nthreads) {
-        if (col >= jb.K) {  // pad column
-            if (df) {
-                put_df(data, jb, KP, 0, col, make_float2(1.f, 0.f), make_float2(0.f, 0.f));
-                for (int j = 1; j <= jb.nrows; ++j) put_df(data, jb, KP, j, col, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
-            } else {
-                put_f32(data, jb, KP, 0, col, 1.f, 0.f);
-                for (int j = 1; j <= jb.nrows; ++j) put_f32(data, jb, KP, j, col, 0.f, 0.f);
+    const bool bbfg = jb.formula == BS_JOB_BBFG, nw = jb.formula == BS_JOB_NW;
+    constexpr int kRows = (BS_MAX_DIGITS + kPackLanes - 1) / kPackLanes;  // digit rows of a lane
+    const int part = tid % kPackLanes;
+    for (int base = 0; base < KP; base += nthreads / kPackLanes) {  // (every lane runs every round)
+        const int col = base + tid / kPackLanes;
+        const bool live = col < jb.K;
+        const int sc = csrc[live ? col : 0];
+        const bool first = part == 0 && (bbfg || nw);  // this lane also takes the start row
+        double2 a0 = make_double2(0.0, 0.0), a[kRows];
+        int m[kRows];
+        if (first) a0 = src_elem(src, jb, bbfg ? prow : jb.n - 1, sc);
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            const int j = part + kPackLanes * i;
+            a[i] = make_double2(0.0, 0.0);
+            m[i] = 0;
+            if (j < jb.nrows) {
+                a[i] = src_elem(src, jb, dsrc[j], sc);
+                m[i] = bbfg ? radix[j] - 1 : 1;
+            }
+        }
+        double bre = fabs(a0.x), bim = fabs(a0.y);
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            if (kPackLanes * i >= jb.nrows) break;
+            bre += (double)m[i] * fabs(a[i].x);
+            bim += (double)m[i] * fabs(a[i].y);
+        }
+#pragma unroll
+        for (int s = 1; s < kPackLanes; s <<= 1) {
+            bre += __shfl_xor_sync(0xffffffffu, bre, s);
+            bim += __shfl_xor_sync(0xffffffffu, bim, s);
+        }
+        int flags = 0;
+        if (!isfinite(bre)) flags |= BS_COLEXP_NAN_RE;
+        if (!isfinite(bim)) flags |= BS_COLEXP_NAN_IM;
+        int e = 0;
+        const double b = 0.25 * bre + 0.25 * bim;  // a quarter: b must not overflow
+        if (!flags && b > 0.0) {
+            (void)frexp(f32 || df ? b : b * (1.0 + 0x1p-20), &e);
+            e += 2;
+        }
+        if (df) e -= 2;  // column sums up to 4 (walk_df.cuh)
+        if (flags || !live) {
+            a0 = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) a[i] = make_double2(0.0, 0.0);
+        }
+        if (live && part == 0) colexp[col] = flags ? flags : e;
+        if (f32 || df) {
+            __int128 sre = wide_of(a0.x, e), sim = wide_of(a0.y, e);
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                if (kPackLanes * i >= jb.nrows) break;
+                const int j = part + kPackLanes * i;
+                const __int128 qre = wide_of(a[i].x, e), qim = wide_of(a[i].y, e);
+                sre += qre * m[i];
+                sim += qim * m[i];
+                if (j >= jb.nrows || col >= KP) continue;
+                if (df)
+                    put_df(data, jb, KP, 1 + j, col, df_split(2 * qre), df_split(2 * qim));
+                else
+                    put_f32(data, jb, KP, 1 + j, col, (float)scale2(a[i].x, 1 - e), (float)scale2(a[i].y, 1 - e));
+            }
+            sre = wide_add_lanes(sre);
+            sim = wide_add_lanes(sim);
+            if (part == 0 && col < KP) {
+                if (df)
+                    put_df(data, jb, KP, 0, col, live ? df_split(sre) : make_float2(1.f, 0.f), df_split(sim));
+                else
+                    put_f32(data, jb, KP, 0, col, live ? (float)wide_double(sre) : 1.f, (float)wide_double(sim));
             }
             continue;
         }
-        const int sc = csrc[col];
-        int e = 0;
-        double2 a = src_elem(src, jb, prow, sc);
-        double b = fabs(a.x) + fabs(a.y);
-        for (int j = 0; j < jb.nrows; ++j) {
-            double2 d = src_elem(src, jb, dsrc[j], sc);
-            b += (double)(radix[j] - 1) * (fabs(d.x) + fabs(d.y));
-        }
-        if (b > 0.0) (void)frexp(b, &e);  // b = f 2^e, f in [0.5, 1)
-        if (df) e -= 2;                   // DF: column sums up to 4 (walk_df.cuh)
-        colexp[col] = e;
-        // c0 in double-double (each product split exactly with an FMA), rounded
-        ddv sre = {ldexp(a.x, -e), 0.0}, sim = {ldexp(a.y, -e), 0.0};
-        for (int j = 0; j < jb.nrows; ++j) {
-            double2 d = src_elem(src, jb, dsrc[j], sc);
-            double m = (double)(radix[j] - 1);
-            double dre = ldexp(d.x, -e), dim = ldexp(d.y, -e);
-            double pre = m * dre, pim = m * dim;
-            double ere = __fma_rn(m, dre, -pre), eim = __fma_rn(m, dim, -pim);
-            sre = dd_add_d(dd_add_d(sre, pre), ere);
-            sim = dd_add_d(dd_add_d(sim, pim), eim);
-        }
-        if (df) {
-            put_df(data, jb, KP, 0, col, df_quantise(sre.hi, sre.lo), df_quantise(sim.hi, sim.lo));
-            for (int j = 0; j < jb.nrows; ++j) {
-                double2 d = src_elem(src, jb, dsrc[j], sc);
-                put_df(data, jb, KP, 1 + j, col, df_quantise(ldexp(d.x, 1 - e), 0.0),
-                       df_quantise(ldexp(d.y, 1 - e), 0.0));
+        zfix* out = static_cast<zfix*>(data) + jb.data_off;
+        const int sh = nw ? 62 - e : 63 - e;
+        unsigned long long sre = (unsigned long long)__double2ll_rn(scale2(a0.x, sh));  // the start sums
+        unsigned long long sim = (unsigned long long)__double2ll_rn(scale2(a0.y, sh));
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            if (kPackLanes * i >= jb.nrows) break;
+            const int j = part + kPackLanes * i;
+            const unsigned long long qre = (unsigned long long)__double2ll_rn(scale2(a[i].x, sh));
+            const unsigned long long qim = (unsigned long long)__double2ll_rn(scale2(a[i].y, sh));
+            zfix row;
+            if (bbfg) {
+                sre += (unsigned long long)m[i] * qre;
+                sim += (unsigned long long)m[i] * qim;
+                row.re = (long long)(2ull * qre);
+                row.im = (long long)(2ull * qim);
+            } else {
+                // Nijenhuis-Wilf start: 2 x = 2 a_last - sum over all
+                // columns = a_last - sum over the digits, in even units
+                sre -= nw ? qre : 0ull;
+                sim -= nw ? qim : 0ull;
+                row.re = -(long long)(qre << (nw ? 1 : 0));
+                row.im = -(long long)(qim << (nw ? 1 : 0));
             }
-        } else {
-            put_f32(data, jb, KP, 0, col, (float)sre.hi, (float)sim.hi);
-            for (int j = 0; j < jb.nrows; ++j) {
-                double2 d = src_elem(src, jb, dsrc[j], sc);
-                put_f32(data, jb, KP, 1 + j, col, (float)ldexp(d.x, 1 - e), (float)ldexp(d.y, 1 - e));
-            }
+            if (j < jb.nrows && col < KP) out[(size_t)(1 + j) * KP + col] = row;
         }
+#pragma unroll
+        for (int s = 1; s < kPackLanes; s <<= 1) {
+            sre += __shfl_xor_sync(0xffffffffu, sre, s);
+            sim += __shfl_xor_sync(0xffffffffu, sim, s);
+        }
+        // a pad column's sum is exactly 1 = 2^62 / 2^63 2^1
+        if (part == 0 && col < KP) out[col] = live ? zfix{(long long)sre, (long long)sim} : zfix{1ll << 62, 0};
     }
 }
 
