@@ -461,15 +461,16 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
 int enqueue_device(bs_ctx* c, const Prepared& P, const double2* d_src, double2* d_out, double2* d_out_lo,
                    int* d_status_out) {
     int rc;
-    // counters, totals and status; the statistics slots are cleared only by
-    // bs_ctx_reset_stats
-    BS_CUDA(cudaMemsetAsync(c->ctl.p, 0, kCtlCleared * 8, c->stream));
+    // the first pack launch clears counters, totals and status; the statistics
+    // slots are cleared only by bs_ctx_reset_stats
+    unsigned long long* clear = static_cast<unsigned long long*>(c->ctl.p);
     const bs_job* djobs = static_cast<const bs_job*>(c->jobs.p);
     for (int prec = 0; prec < BS_NPREC; ++prec) {
         const size_t lo = P.pbeg[prec], hi = P.pbeg[prec + 1];
         if (hi == lo) continue;
         cudaError_t e = bs::launch_pack(djobs + lo, (int)(hi - lo), d_src, static_cast<int*>(c->meta.p),
-                                        arena_of(prec) ? c->data32.p : c->data64.p, prec, c->stream);
+                                        arena_of(prec) ? c->data32.p : c->data64.p, prec, c->stream, clear, kCtlCleared);
+        clear = nullptr;
         if (e != cudaSuccess) return fail(BS_ECUDA, "pack launch failed: %s", cudaGetErrorString(e));
         c->stats.kernel_launches++;
     }
@@ -517,23 +518,33 @@ int check_status(bs_ctx* c) {
 // Results of the calls that return to the host: the reduce kernel writes
 // `n` values and behind them a copy of the walk status word straight into
 // pinned host memory, so a call ends with one synchronisation and no copy
-// (12 x 12 permanent: 51 -> 42 us).
-int back_buffer(bs_ctx* c, int n, double2** out) {
-    const size_t need = (size_t)n * sizeof(double2) + 16;
+// (12 x 12 permanent: 51 -> 42 us).  Behind them is room for a small source:
+// up to kDirectSrc bytes the pack kernel reads the matrices from there as
+// well, once, without an upload before it (sixteen 8 x 8 permanents, 16 KB:
+// 78 -> 71 us; at 64 KB both ways take the same time).
+constexpr size_t kDirectSrc = 16 << 10;
+int back_buffer(bs_ctx* c, int n, size_t src_bytes, double2** out, bs_c128** src) {
+    if (src_bytes > kDirectSrc) src_bytes = 0;
+    const size_t res_bytes = (size_t)n * sizeof(double2) + 16;
+    const size_t need = res_bytes + src_bytes;
     if (c->h_back_n < need) {
         c->buf_gen++;  // captured graphs hold the old address
+        const size_t want = std::max({need, 2 * c->h_back_n, 2 * kDirectSrc});
         if (c->h_back) cudaFreeHost(c->h_back);
         c->h_back = nullptr;
         c->h_back_n = 0;
-        const size_t want = std::max(need, (size_t)4096);
         BS_CUDA(cudaHostAlloc(&c->h_back, want, cudaHostAllocDefault));
         c->h_back_n = want;
     }
     *out = static_cast<double2*>(c->h_back);
+    *src = src_bytes ? reinterpret_cast<bs_c128*>(static_cast<char*>(c->h_back) + res_bytes) : nullptr;
     return BS_OK;
 }
-int finish_back(bs_ctx* c, const double2* out, int n) {
+// Waits for the call (rc: what enqueuing it returned) and checks its status;
+// after a failed one too, as its kernels may still use the pinned block.
+int finish_back(bs_ctx* c, const double2* out, int n, int rc) {
     cudaError_t e = cudaStreamSynchronize(c->stream);
+    if (rc) return rc;
     if (e != cudaSuccess) return fail(BS_ECUDA, "stream synchronize: %s", cudaGetErrorString(e));
     int st = 0;
     std::memcpy(&st, out + n, sizeof(int));
@@ -681,19 +692,25 @@ int run_single(bs_ctx* c, const bs_c128* A, int rows, int cols, int ld, int kind
     std::lock_guard<std::mutex> lk(c->mu);
     BS_CUDA(cudaSetDevice(c->device));
     const size_t mat_b = (size_t)rows * cols * sizeof(bs_c128);
-    if ((rc = ensure(c, c->src, mat_b))) return rc;
     double2* res = nullptr;
-    if ((rc = back_buffer(c, 2 * nout, &res))) return rc;
-    bs_c128* h = static_cast<bs_c128*>(stage(c, mat_b));
-    if (!h) return fail(BS_ENOMEM, "pinned host staging allocation failed");
-    copy_matrix(h, A, rows, cols, ld);
-    BS_CUDA(cudaMemcpyAsync(c->src.p, h, mat_b, cudaMemcpyHostToDevice, c->stream));
-    BS_CUDA(cudaEventRecord(c->stage_ev[c->stage_cur], c->stream));
+    bs_c128* h = nullptr;
+    if ((rc = back_buffer(c, 2 * nout, mat_b, &res, &h))) return rc;
+    const double2* d_src = reinterpret_cast<const double2*>(h);
+    if (h) {
+        copy_matrix(h, A, rows, cols, ld);
+    } else {
+        if ((rc = ensure(c, c->src, mat_b))) return rc;
+        if (!(h = static_cast<bs_c128*>(stage(c, mat_b)))) return fail(BS_ENOMEM, "pinned host staging allocation failed");
+        copy_matrix(h, A, rows, cols, ld);
+        BS_CUDA(cudaMemcpyAsync(c->src.p, h, mat_b, cudaMemcpyHostToDevice, c->stream));
+        BS_CUDA(cudaEventRecord(c->stage_ev[c->stage_cur], c->stream));
+        d_src = static_cast<const double2*>(c->src.p);
+    }
     std::vector<IntPlan> plans = {p};
     const int64_t off0 = 0;
-    rc = batch_walk(c, plans, plan_key(c, p, rows, cols, mode), &off0, &cols, static_cast<const double2*>(c->src.p),
-                    res, mode, res + nout, reinterpret_cast<int*>(res + 2 * nout), true);
-    if (rc || (rc = finish_back(c, res, 2 * nout))) return rc;
+    rc = batch_walk(c, plans, plan_key(c, p, rows, cols, mode), &off0, &cols, d_src, res, mode, res + nout,
+                    reinterpret_cast<int*>(res + 2 * nout), true);
+    if ((rc = finish_back(c, res, 2 * nout, rc))) return rc;
     std::copy(res, res + nout, hi.begin());
     std::copy(res + nout, res + 2 * nout, lo.begin());
     return BS_OK;
@@ -1208,24 +1225,30 @@ int bs_perm_batch(bs_ctx* c, int count, const bs_c128* A_packed, const int64_t* 
         off[b] = (int64_t)total;
         if (!plans[b].trivial) total += (size_t)rows[b] * cols[b];
     }
-    if ((rc = ensure(c, c->src, total * sizeof(bs_c128)))) return rc;
+    const size_t src_b = total * sizeof(bs_c128);
     double2* res = nullptr;
-    if ((rc = back_buffer(c, count, &res))) return rc;
-    bs_c128* h = static_cast<bs_c128*>(stage(c, total * sizeof(bs_c128)));
-    if (!h) return fail(BS_ENOMEM, "pinned host staging allocation failed");
+    bs_c128* h = nullptr;
+    if ((rc = back_buffer(c, count, src_b, &res, &h))) return rc;
+    const bool direct = h != nullptr;
+    if (!direct) {
+        if ((rc = ensure(c, c->src, src_b))) return rc;
+        if (!(h = static_cast<bs_c128*>(stage(c, src_b)))) return fail(BS_ENOMEM, "pinned host staging allocation failed");
+    }
     for (int b = 0; b < count; ++b)
         if (!plans[b].trivial) copy_matrix(h + off[b], A_packed + a_offset[b], rows[b], cols[b], cols[b]);
-    BS_CUDA(cudaMemcpyAsync(c->src.p, h, total * sizeof(bs_c128), cudaMemcpyHostToDevice, c->stream));
-    BS_CUDA(cudaEventRecord(c->stage_ev[c->stage_cur], c->stream));
+    if (!direct) {
+        BS_CUDA(cudaMemcpyAsync(c->src.p, h, src_b, cudaMemcpyHostToDevice, c->stream));
+        BS_CUDA(cudaEventRecord(c->stage_ev[c->stage_cur], c->stream));
+    }
+    const double2* d_src = direct ? reinterpret_cast<const double2*>(h) : static_cast<const double2*>(c->src.p);
     // the staged sources are contiguous: the key uses their offsets
     const std::vector<int64_t> key =
         batch_key(c, count, off.data(), rows, cols, mult_packed, row_mult_off, col_mult_off, mode);
-    rc = batch_walk(c, plans, key, off.data(), cols, static_cast<const double2*>(c->src.p),
-                    res, mode, nullptr, reinterpret_cast<int*>(res + count));
-    if (rc) return rc;
+    rc = batch_walk(c, plans, key, off.data(), cols, d_src, res, mode, nullptr,
+                    reinterpret_cast<int*>(res + count));
     bool walked = false;
     for (int b = 0; b < count; ++b) walked |= !plans[b].trivial;
-    if (walked && (rc = finish_back(c, res, count))) return rc;
+    if ((walked || rc) && (rc = finish_back(c, res, count, rc))) return rc;
     for (int b = 0; b < count; ++b) {
         if (plans[b].trivial) {
             out[b].re = 1.0;

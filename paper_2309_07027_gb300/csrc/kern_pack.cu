@@ -17,16 +17,20 @@
 
 namespace bs {
 
+// The first CTA also clears `nclear` control words at `clear` (a memset of
+// its own is one more stream operation in a call's chain).
 __global__ void __launch_bounds__(kPackBlock) pack_kernel(const bs_job* __restrict__ jobs, const double2* __restrict__ src, int* __restrict__ meta,
-                            void* __restrict__ data, int prec) {
+                            void* __restrict__ data, int prec, unsigned long long* __restrict__ clear, int nclear) {
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < nclear; i += blockDim.x) clear[i] = 0ull;
     const bs_job jb = jobs[blockIdx.x];
     pack_job(jb, src, meta, data, prec, threadIdx.x, blockDim.x);
 }
 
 cudaError_t launch_pack(const bs_job* jobs, int njobs, const double2* src, int* meta, void* data, int prec,
-                        cudaStream_t s) {
+                        cudaStream_t s, unsigned long long* clear, int nclear) {
     if (njobs <= 0) return cudaSuccess;
-    pack_kernel<<<njobs, kPackBlock, 0, s>>>(jobs, src, meta, data, prec);
+    pack_kernel<<<njobs, kPackBlock, 0, s>>>(jobs, src, meta, data, prec, clear, clear ? nclear : 0);
     return cudaGetLastError();
 }
 

@@ -35,7 +35,8 @@ cudaError_t launch_walk_df_minors(const WalkArgs& a, cudaStream_t s);
 // prec (BS_PREC_*) selects the layout: complex doubles (FP64), packed float
 // pairs (FP32, the float arena) or double-float pairs (DF, 16-byte units).
 cudaError_t launch_pack(const bs_job* jobs, int njobs, const double2* src, int* meta, void* data, int prec,
-                        cudaStream_t s);
+                        cudaStream_t s,
+                        unsigned long long* clear = nullptr, int nclear = 0);
 
 // Sums each job's task partials in a fixed order and applies 2^(1-n) and the
 // column scales; writes out[out_index + col] (and the low parts to out_lo when

@@ -50,3 +50,17 @@ def test_entries_that_are_not_finite(bslib, mode, bad, K):
     assert np.all(np.isnan(got[np.arange(K) != 1])) and np.isfinite(got[1])
     assert got[1] == clean[1]  # a minor never reads its own column
     ctx.close()
+
+
+def test_sources_on_both_sides_of_the_direct_limit(ctx):
+    """Up to 16 KB of matrices are read in place from pinned memory, more are
+    uploaded; either way a batch gives the bits of single calls, also when a
+    captured call repeats after the pinned block has grown."""
+    one = np.ones(8, np.int32)
+    items = [(S.random_complex(8, 8, 900 + i), one, one) for i in range(300)]
+    ref = np.array([ctx.perm(*it) for it in items[:17]])
+    for count in (1, 15, 16, 17, 300, 16, 1):
+        got = ctx.perm_batch(items[:count])
+        assert np.array_equal(got[:17], ref[:count])
+        for _ in range(3):
+            assert ctx.perm(*items[3]) == ref[3]
