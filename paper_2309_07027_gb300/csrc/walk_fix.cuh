@@ -260,8 +260,8 @@ __device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
 // own end, so that the warp stays converged.
 //
 // 30 x 30 permanent (2^29 addends): 165 ms in double (FP64 pipe 94 % busy),
-// 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 30.0
-// ms here; 73 cycles per warp, column and addend, of which the 12 integer
+// 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 28.7
+// ms here; 70 cycles per warp, column and addend, of which the 12 integer
 // products hold the FMA-heavy pipe 52 (72 % busy) and 25 other integer
 // instructions take the rest.  Relative error (23 x 23, Haar): 6.8e-15, in
 // double 2.7e-14.
@@ -330,7 +330,7 @@ __device__ __forceinline__ zraw fix_shr(const zraw& v, int d) {
 }
 
 // Longest integer run of the minors, in addends (a power of two).
-constexpr uint32_t kFixRun = 4;
+constexpr uint32_t kFixRun = 8;
 
 // Shared memory of one warp of the minors kernel, HX columns per lane, NP =
 // ceil(HX / 2) leaves: the integer sums [col][lane] (rows of 33, so that
@@ -431,10 +431,10 @@ __device__ __forceinline__ void prefix_step(const zraw (&c)[HX], int j, bool las
     zraw z = fix_shr(zraw{(unsigned long long)a.x, (unsigned long long)a.y}, dl);
     if (2 * j + 1 < HX) {
         const zlimb ml = limbs_of(m);
-        z = fix_cmul_add<1, 1>(z, ml, limbs_of(c[2 * j + 1]));
+        z = fix_cmul_add<0, 1>(z, ml, limbs_of(c[2 * j + 1]));
         sm_acc[2 * j * 33] = make_longlong2((long long)z.re, (long long)z.im);
         const longlong2 b = sm_acc[(2 * j + 1) * 33];
-        z = fix_cmul_add<1, 1>(fix_shr(zraw{(unsigned long long)b.x, (unsigned long long)b.y}, dl), ml,
+        z = fix_cmul_add<0, 1>(fix_shr(zraw{(unsigned long long)b.x, (unsigned long long)b.y}, dl), ml,
                                limbs_of(c[2 * j]));
         sm_acc[(2 * j + 1) * 33] = make_longlong2((long long)z.re, (long long)z.im);
     } else {  // no partner: m_j itself, in the same unit (m / 2)
@@ -460,22 +460,26 @@ __device__ __forceinline__ void prefix_step(const zraw (&c)[HX], int j, bool las
 // The sums.  A conversion to double and an FMA hold the FP64 pipe for 128
 // cycles; done for every addend that would cost more than the products do
 // (minors at K = 28: 453 cycles per column and addend), so integer sums run
-// over at most 4 addends (|m_j c| < 2^60, so 4 stay below 2^62; never across
-// a change of the binomial weight) and go to plain-double column sums beside
-// the products, sign, weight and unit in one factor; 16 of those runs to the
-// double-double totals.  The unit is what the accuracy hangs on: m_j is
-// brought to [2^60, 2^61) at the run's largest addend, and the sum's rounding
-// is then about 2^-54 of that addend.  Errors against exact minors (24
-// columns, distinct rows, root mean square relative): 1.2e-14, the kernels in
-// double 2.2e-14; runs of 8 addends 2.0e-14, one unit for the whole warp
-// 3.5e-12 (27 columns), without the sums (one addend per run) 2e-15.
+// over at most 8 addends (|m_j c| < 2^60 (1 - 2^-21), so 8 stay below 2^63;
+// never across a change of the binomial weight) and go to plain-double column
+// sums beside the products, sign, weight and unit in one factor; 16 of those
+// runs to the double-double totals.  The unit is what the accuracy hangs on:
+// m_j is brought to [2^60, 2^61) at the run's largest addend (one unit for the
+// whole warp: 3.5e-12 at 27 columns).  Shifts and the products summed round
+// down; with every run of the same sign their half units add up over the
+// walk, so every other run and chunk is summed with the opposite sign.  Errors
+// against exact minors (root mean square relative; kernels in double / runs of
+// 4 of one sign / here): 20 columns 1.0e-14 / 2.9e-15 / 1.3e-15, 24 columns
+// 2.2e-14 / 1.3e-14 / 4.8e-15, 27 columns with collisions 1.0e-13 / 5e-14 /
+// 1.6e-14.  Rounding the products summed as well: 1.1e-15, 4.0e-15, 1.4e-14,
+// 1.4 % slower; truncating the exchanged products too: 1.2e-14 at 24 columns.
 //
-// Time.  29 x 30 minors (2^28 addends): 190 ms in double, 47.8 ms here (1.42e9 ->
-// 5.62e9 addends/s; 49.7 with the m_j of an addend kept before any is added);
-// the FMA-heavy pipe is 68 % busy
-// with integer products (4.35 cycles per warp and product) and every other
-// integer instruction costs about 1.3 cycles beside them, so what bounds it is
-// the instruction count: 112 per column and addend, 33 of them products.
+// Time.  29 x 30 minors (2^28 addends): 190 ms in double, 45.2 ms here (1.42e9 ->
+// 5.94e9 addends/s; 47.8 with runs of 4, 49.7 with the m_j of an addend kept
+// before any is added); 24 columns 0.605 ms (0.670 with runs of 4).  The
+// FMA-heavy pipe is about 70 % busy with integer products (4.35 cycles per
+// warp and product) and every other integer instruction costs about 1.3
+// cycles beside them, so what bounds it is the instruction count.
 template <int G, int KB, int HX>
 __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ data, const int* __restrict__ radix,
                                      bs_zdd* __restrict__ partials, uint32_t local, int lane,
@@ -509,8 +513,8 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
         if (steps == 0u) break;
         // runs end where a repeated-row digit moves (the weight changes there:
         // after every 2^nbin addends)
-        const uint32_t run_mask = jb.nbin >= 2 ? kFixRun - 1u : (1u << jb.nbin) - 1u;
-        static_assert(kFixRun == 4, "2^2 addends per run");
+        const uint32_t run_mask = jb.nbin >= 3 ? kFixRun - 1u : (1u << jb.nbin) - 1u;
+        static_assert(kFixRun == 8, "2^3 addends per run");
         bs_gray g;
         ChunkStepper st;
         st.init(g, i0, jb.nbin, jb.nrows, radix, reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
@@ -523,6 +527,7 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
         const int e_unit = 64 - 63 + (G * HX - K);
         int em[NP];
         uint32_t runs = 0;
+        const uint32_t flip = (uint32_t)(lane / G);  // parity of the chunk
         for (uint32_t s = 0; s < steps; ++s) {
             // 1. leaves, suffix products, Q
             int es[NP];
@@ -546,8 +551,10 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
                     ra = raw_of(qa);
                 }
                 // the addend's sign against the run's first one goes here, and a
-                // lane past its chunk adds zeros from here on
-                const unsigned long long m = 0ull - (unsigned long long)(s & 1u & run_mask);
+                // lane past its chunk adds zeros from here on.  Every other run
+                // (and chunk) is summed with the opposite sign: shifts round down, and the
+                // half unit each of them loses would add up over the runs.
+                const unsigned long long m = 0ull - (unsigned long long)(((s & run_mask) ^ runs ^ flip) & 1u);
                 ra.re = s < len ? (ra.re ^ m) - m : 0ull;
                 ra.im = s < len ? (ra.im ^ m) - m : 0ull;
                 pr = limbs_of(ra);
@@ -587,9 +594,11 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
                 }
             }
             // the end of a run
-            if (((s + 1u) & run_mask) == 0u || s + 1 == steps)
-                minors_flush_fix<G, HX>(sm, scale_pow2(wrun, e_unit), em, lane, K,
-                                        (++runs & (kFixFold - 1u)) == 0u || s + 1 == steps);
+            if (((s + 1u) & run_mask) == 0u || s + 1 == steps) {
+                const double f = scale_pow2(((runs ^ flip) & 1u) ? -wrun : wrun, e_unit);
+                ++runs;
+                minors_flush_fix<G, HX>(sm, f, em, lane, K, (runs & (kFixFold - 1u)) == 0u || s + 1 == steps);
+            }
             if (s + 1 == steps) break;
             uint32_t neg = 0;
             int row = 0;  // a lane past its chunk moves on, adding zeros

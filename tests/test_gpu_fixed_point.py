@@ -108,7 +108,8 @@ def test_entries_that_are_not_finite(ctx, bad, K):
     assert ctx.perm(np.array([[1.5 + 0.5j]]), [1], [1]) == 1.5 + 0.5j
 
 
-@pytest.mark.parametrize("M", [[1] * 9, [2] * 5, [3, 1, 2, 2, 1, 1], [9], [1, 1, 7], [4, 4, 1], [1, 2, 1, 4, 1]])
+@pytest.mark.parametrize("M", [[1] * 9, [2] * 5, [3, 1, 2, 2, 1, 1], [9], [1, 1, 7], [4, 4, 1], [1, 2, 1, 4, 1],
+                               [1, 1, 1, 1, 2, 3], [1, 1, 1, 1, 1, 4]])
 def test_minors_runs_end_where_the_weight_changes(ctx, M):
     """Integer runs of the minors: rows of every kind (no, one, two, three and
     more binary digits before the repeated ones), odd and even widths."""
