@@ -133,16 +133,25 @@ extern "C" int bs_perm_noalloc(const bs_c128* A, int rows, int cols, int ld, con
         prec = plan ? BS_PREC_FP32 : BS_MIXED_FALLBACK_PREC;
         reseed = plan == 2 ? BS_FP32_RESEED_LOG2 : 0;
     }
+    const int target = prec == BS_PREC_FP32 ? BS_TARGET_TASKS_SINGLE_FP32 : BS_TARGET_TASKS_SINGLE;
+    auto tasks_of = [&](int chunks, int& l, uint64_t& per) {
+        l = bs_choose_log2L_single(p.C, chunks, kLog2Max, target);
+        per = (uint64_t)chunks << l;
+        return (p.C + per - 1) / per;
+    };
     const int cpt = bs_chunks_per_task(BS_KIND_PERM, prec, p.K);
-    const int log2L = bs_choose_log2L_single(p.C, cpt, kLog2Max,
-                                             prec == BS_PREC_FP32 ? BS_TARGET_TASKS_SINGLE_FP32 : BS_TARGET_TASKS_SINGLE);
-    const uint64_t per = (uint64_t)cpt << log2L;
-    const uint64_t ntasks = (p.C + per - 1) / per;
-    if (ntasks > kPartSlots)
+    int log2L, lim_l;
+    uint64_t per, lim_per;
+    const uint64_t ntasks = tasks_of(cpt, log2L, per);
+    // the size limit of a double-float call is that of a task of its lane
+    // groups' chunks (never more than cpt), as it always was
+    const uint64_t need = prec == BS_PREC_DF ? tasks_of(32 / bs_df_group(p.K), lim_l, lim_per) : ntasks;
+    if (prec == BS_PREC_DF) per = lim_per;
+    if (need > kPartSlots)
         return bs::fail(BS_EINVAL,
                         "bs_perm_noalloc: %llu addends need %llu task slots; its fixed scratch holds %zu "
                         "(about %.3g addends); use bs_perm",
-                        (unsigned long long)p.C, (unsigned long long)ntasks, kPartSlots,
+                        (unsigned long long)p.C, (unsigned long long)need, kPartSlots,
                         (double)kPartSlots * (double)per);
     // host-side descriptors on the stack
     bs_c128 Ac[BS_MAX_N * BS_MAX_N];
