@@ -53,8 +53,11 @@ typedef struct {
 } bs_c128;
 
 /* Arithmetic of the walk.
- *   BS_FP64:  column sums, products, weights and sums in double precision;
- *             partial sums combined in double-double.
+ *   BS_FP64:  column sums and products in 64-bit fixed point on the integer
+ *             pipes (column sums exact, products of 62-bit operands with
+ *             exponents: errors below those of plain double arithmetic),
+ *             weights and sums in double precision, partial sums combined in
+ *             double-double.
  *   BS_MIXED: column sums and products in single precision (column sums
  *             re-seeded from the matrix every chunk, and every 2^8 steps
  *             inside it for jobs whose error would otherwise drift past the
@@ -68,9 +71,9 @@ typedef struct {
  *             (about 48 significant bits) on the single-precision pipe --
  *             column sums exact in fixed point (no drift), products by
  *             FMA-based exact multiplication, compensated sums, partial sums
- *             in double-double; results within the FP64 tolerance at several
- *             times the FP64 kernels' speed on this part, whose FP64 rate is
- *             1/64 of its FP32 rate. */
+ *             in double-double; minors within the FP64 tolerance at up to 1.7
+ *             times the FP64 kernels' speed.  Permanents run as in BS_FP64,
+ *             whose kernels are the faster ones there. */
 typedef enum { BS_FP64 = 0, BS_MIXED = 1, BS_DF64 = 2 } bs_mode;
 
 typedef struct bs_ctx bs_ctx;
@@ -193,7 +196,7 @@ int bs_laplace_minors(bs_ctx* ctx, const bs_c128* A, int rows, int cols, int ld,
 typedef enum { BS_FORMULA_BBFG = 0, BS_FORMULA_RYSER = 1, BS_FORMULA_NW = 2 } bs_formula;
 
 /* Permanent of the n x n matrix A (row-major, leading dimension ld >= n) by
- * `formula`, walked by the FP64 permanent kernel in double precision with
+ * `formula`, walked by the FP64 permanent kernel (64-bit fixed point) with
  * double-double partial sums: the accuracy and speed comparison of Sec. 3.2
  * (Fig. accuracy) on this GPU.  Only the packing of the start sums and the
  * rows added per step, and the prefactor, differ between formulas.  n = 0

@@ -26,7 +26,7 @@ __all__ = ["BS_FP64", "BS_MIXED", "BS_DF64", "BsError", "Context", "Server", "li
 
 BS_FP64 = 0
 BS_MIXED = 1
-BS_DF64 = 2  # double-float: FP64-class results on the FP32 pipe
+BS_DF64 = 2  # double-float minors: FP64-class results on the FP32 pipe (permanents as BS_FP64)
 # statistics slots by kernel family: FP64, FP32, double-float
 PRECISIONS = ("fp64", "fp32", "df")
 # formulas of bs_perm_formula (bs_formula)

@@ -84,9 +84,8 @@ struct bs_job {
 // the width KB of the bucket kernel that walks the job (inside a kernel the
 // stride is the compile-time KB), so FP32 rows are whole 16-byte column pairs
 // and every bucket column has a slot.  Pad columns are neutral: rows hold
-// zeros, and in FP32 jobs c0 holds 1, so a pad column sum stays exactly 1 and
-// leaves every product unchanged (FP64 jobs keep c0 = 0 there and test
-// columns against K instead).
+// zeros and c0 holds the value 1, so a pad column's sum stays exactly 1 and
+// leaves every product unchanged.
 #define BS_ROW_STRIDE(K) ((((K) + 3) / 4) * 4)
 // Double-float minors: K rounded up to a multiple of 8 (the DF bucket width).
 #define BS_ROW_STRIDE_DF(K) ((((K) + 7) / 8) * 8)
@@ -100,10 +99,10 @@ struct bs_job {
 #define BS_DF_MINORS(prec, kind) ((prec) == BS_PREC_DF && (kind) == BS_KIND_MINORS)
 
 // Precision of a job: the kernel family that walks it.
-//   FP64: double column sums, products and runs (data in complex doubles);
+//   FP64: 64-bit fixed point (walk_fix.cuh; data in pairs of 64-bit integers);
 //   FP32: single-precision packed pairs (data in complex floats);
-//   DF:   double-float (float pairs, exact fixed-point column sums; data in
-//         16-byte units like FP64).
+//   DF:   minors in double-float (float pairs, exact fixed-point column sums;
+//         data in 16-byte units like FP64), permanents as FP64.
 #define BS_PREC_FP64 0
 #define BS_PREC_FP32 1
 #define BS_PREC_DF 2

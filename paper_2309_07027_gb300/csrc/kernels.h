@@ -32,7 +32,7 @@ cudaError_t launch_walk_fp32_minors(const WalkArgs& a, cudaStream_t s);
 cudaError_t launch_walk_df_minors(const WalkArgs& a, cudaStream_t s);
 
 // Builds c0 / 2a (and column scales) of every job from its source matrix.
-// prec (BS_PREC_*) selects the layout: complex doubles (FP64), packed float
+// prec (BS_PREC_*) selects the layout: 64-bit fixed point (FP64), packed float
 // pairs (FP32, the float arena) or double-float pairs (DF, 16-byte units).
 cudaError_t launch_pack(const bs_job* jobs, int njobs, const double2* src, int* meta, void* data, int prec,
                         cudaStream_t s,

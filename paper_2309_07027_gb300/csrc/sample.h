@@ -17,7 +17,7 @@
 // (bs_choose_log2L_single).  The sampler and the server, which always run many jobs
 // together, use BS_TARGET_TASKS_MANY (longer chunks, fewer tasks) with a
 // floor of 2^3: their small jobs (early steps, heavy-collision chains sent to
-// FP64) are latency-bound, and short chunks spread them over more warps.
+// the double-float kernels) are latency-bound, and short chunks spread them over more warps.
 #define BS_TARGET_TASKS_SINGLE 32768
 // FP32 jobs planned one call at a time aim at fewer, longer chunks: the FP32
 // walks are bound by the L1 delivery of rows, and every chunk start re-reads
@@ -37,9 +37,8 @@
 #define BS_LOG2L_MIN_SINGLE 6
 #define BS_LOG2L_MIN_MANY 3
 // Floor for the tiniest jobs planned alone (at most BS_FILL_TINY_C
-// addends): chunks of 2 addends.  Such a job's walk time is one warp's FP64
-// instruction stream (one instruction per 64 cycles per scheduler on this
-// part), and more, shorter chunks spread it over more warps; a chunk start
+// addends): chunks of 2 addends.  Such a job's walk time is one warp's
+// instruction stream, and more, shorter chunks spread it over more warps; a chunk start
 // decodes its index and seeds the column sums (about the work of one or two
 // addends), so shorter chunks would only add work.  Larger small jobs keep
 // the 2^3 floor: batches of them are throughput-bound, and there the extra
@@ -81,8 +80,8 @@ BS_HD int bs_target_chains(int64_t S) {
 // BS_TARGET_TASKS_FILL tasks at that floor gets shorter chunks (down to 2^3,
 // or 2^BS_LOG2L_MIN_FILL for the tiniest) until it does: such a job is
 // latency-bound, and
-// its walk time is one lane's chunk, not the total work (a 576-addend FP64
-// job in one warp of 9 chunks of 64 runs at one scheduler's FP64 rate).
+// its walk time is one lane's chunk, not the total work (a 576-addend job in
+// one warp of 9 chunks of 64 runs at one scheduler's rate).
 // 256 tasks keeps the re-seeding of mid-size jobs as it was: with 2048 (one
 // resident wave) jobs of 2^19 to 2^21 addends also got shorter chunks and the
 // 4096-item batch ran 5 % slower, for no gain on small calls.
@@ -109,16 +108,15 @@ BS_HD int bs_choose_log2L_single(uint64_t C, int cpt, int log2max, int target, i
 // twice as long) and measured faster wherever their registers allow 2-3
 // CTAs per SM: widths 32 and 40 by 6-12 %; at 24 four lanes at 5 CTAs per SM
 // are faster, and at 48 two lanes would spill.  A warp task of that kernel
-// covers 32 / G chunks, one of the FP64 fused-minor kernel 16 (lane pairs);
-// the permanent kernels give each lane its own chunk (32 per task).
+// covers 32 / G chunks, one of the FP64 fused-minor kernel 16; a task of a
+// permanent kernel covers 32.
 #define BS_MINORS_FP32_GROUP_KB(KB) (((KB) == 24 || (KB) == 48) ? 4 : 2)
 BS_HD int bs_minors_fp32_group(int K) { return BS_MINORS_FP32_GROUP_KB((K + 3) & ~3); }
 // Lanes per chunk of the FP64 fused minors, by 4-column bucket width (above
 // 32 columns two lanes need 255 registers and run 7-24 % slower than four).
 // A warp task covers 16 chunks either way, in one or two rounds.
 #define BS_MINORS_FP64_GROUP_KB(KB) ((KB) > 32 ? 4 : 2)
-// Lanes per chunk of the double-float minors, by
-// 8-column bucket width KB: each lane owns KB / (2G) column pairs
+// Lanes per chunk of the double-float minors, by 8-column bucket width KB: each lane owns KB / (2G) column pairs
 // (8 -> 1 x 4, 16 -> 2 x 4, 24 -> 4 x 3, 32 -> 4 x 4, 40 -> 4 x 5,
 // 48 -> 8 x 3), so a lane's double-float state fits its registers.
 #define BS_DF_GROUP_KB(KB) ((KB) <= 8 ? 1 : (KB) <= 16 ? 2 : (KB) <= 40 ? 4 : 8)
@@ -165,8 +163,9 @@ BS_HD int64_t bs_flops_per_addend(int K, int kind) {
 // (block structure) cancel far more than it predicts and belong in FP64.
 #define BS_MIXED_LOG2_TOL_DEFAULT (-19.93f)  // log2(1e-6)
 // Kernels of the MIXED jobs that fail the FP32 rule: the double-float
-// kernels (errors about 2^-46 relative, far inside the MIXED tolerance, at
-// about 5x the FP64 kernels' speed on this part).
+// minors (errors about 2^-46 relative, far inside the MIXED tolerance; 1.2
+// times as fast as the FP64 minors at 30 columns) and, for permanents, the
+// FP64 kernels.
 #define BS_MIXED_FALLBACK_PREC BS_PREC_DF
 #define BS_MIXED_QMAX (BS_MAX_PHOTONS * BS_MAX_PHOTONS)  // Q <= sum M_k^2 <= n^2
 #define BS_MIXED_RESIDUAL (-21.02)

@@ -1,6 +1,6 @@
-// Double-float ("DF") Gray-walk tasks: FP64-class accuracy on the FP32 pipe.
+// Double-float ("DF") fused minors: FP64-class accuracy on the FP32 pipe.
 //
-// FP64 runs at 1/64 of the FP32 rate on this part, so the DF kernels carry
+// FP64 runs at 1/64 of the FP32 rate on this part, so these kernels carry
 // every quantity as an unevaluated pair of floats (about 48 significant bits)
 // and do all arithmetic with single-precision FMAs, packed two columns per
 // instruction (fma / add / sub / mul .rn.f32x2: even column in the low half,
