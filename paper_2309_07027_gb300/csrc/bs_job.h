@@ -95,7 +95,7 @@ struct bs_job {
 // than products on the FP32 pipe were (calls: 12 x 12 98 -> 55 us, 20 x 20
 // 160 -> 105, 24 x 24 645 -> 480, 26 x 26 2.63 -> 1.80 ms, 30 x 30 34.8 -> 28.9
 // ms).  Only double-float minors have kernels of their own: at 30 columns they
-// take 38.7 ms where the fixed point takes 47.7.
+// take 38.7 ms where the fixed point takes 45.2.
 #define BS_DF_MINORS(prec, kind) ((prec) == BS_PREC_DF && (kind) == BS_KIND_MINORS)
 
 // Precision of a job: the kernel family that walks it.
