@@ -132,10 +132,18 @@ __device__ __forceinline__ zlimb fix_normalise(const zraw& v, int& e) {
 
 // 2^e w for w a nonzero double of magnitude below 2^64, by the exponent
 // field; e clamped so that the result stays normal (a product 2^-900 below
-// the column bounds adds nothing to a sum of them).
+// the column bounds adds nothing to a sum of them), and zero for e below
+// -8000 (the exponent of a product that is zero).
 __device__ __forceinline__ double scale_pow2(double w, int e) {
+    if (e < -8000) return 0.0;
     if (e < -900) e = -900;
     return __hiloint2double(__double2hiint(w) + (e << 20), __double2loint(w));
+}
+
+// v 2^e as a double (e: a constant that keeps the result normal).
+__device__ __forceinline__ double scale_int(long long v, int e) {
+    const double x = (double)v;
+    return v == 0 ? 0.0 : __hiloint2double(__double2hiint(x) + (e << 20), __double2loint(x));
 }
 
 // Column sums of the decoded state, c0 - sum_j Delta_j 2a_j, for N columns
@@ -223,15 +231,42 @@ __device__ __forceinline__ zraw fix_leaf(const zraw (&c)[N], int j) {
 // running product, normalised after every leaf.  A typical column sum is
 // 2^59.5 (its bound 2^63 is a sum of moduli, it is a root of squares), a pair
 // 2^55, and a pair times a normalised operand 2^52.5, so a pair costs about
-// 2^-54 in relative rounding, where two products of doubles cost 2^-53.
+// 2^-54 in relative rounding, where two products of doubles cost 2^-53.  Sums
+// that cancel lose more: smax is the largest of the normalising shifts, so the
+// relative error is a few 2^(smax - 61), and slast the last one (29 or 30:
+// the product is zero, or has lost everything; smax shows it as well).
 template <int N>
-__device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e) {
+__device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e, int& smax, int& slast) {
     e = kLeafExp;
-    zlimb p = fix_normalise(fix_leaf(c, 0), e);
+    zraw r = fix_leaf(c, 0);
+    slast = fix_norm_shift(r);
+    smax = slast;
+    e -= slast;
+    zlimb p = fix_shift(r, slast);
 #pragma unroll
     for (int j = 1; 2 * j < N; ++j) {
-        e += 64 + kLeafExp;
-        p = fix_normalise(fix_cmul(p, limbs_of(fix_leaf(c, j))), e);
+        r = fix_cmul(p, limbs_of(fix_leaf(c, j)));
+        slast = fix_norm_shift(r);
+        smax = max(smax, slast);
+        e += 64 + kLeafExp - slast;
+        p = fix_shift(r, slast);
+    }
+    return p;
+}
+
+// Product of n column sums in double, in units of kDblUnit bits below each
+// column's bound (so that 48 columns at their bounds stay in range, as do
+// products 2^-1800 below them): every factor is the exact sum rounded once, so
+// the product is as accurate as a product of doubles, however much the sums
+// cancelled.  6 FP64 instructions per column: for the addends that need it.
+constexpr int kDblUnit = 18;
+template <int N>
+__device__ __forceinline__ cx<double> fix_product_dbl(const zraw (&c)[N]) {
+    cx<double> p;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const cx<double> x = {scale_int((long long)c[j].re, kDblUnit - 63), scale_int((long long)c[j].im, kDblUnit - 63)};
+        p = j ? cmul(p, x) : x;
     }
     return p;
 }
@@ -259,8 +294,20 @@ __device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
 // lane 0.  Every lane walks the warp's longest chunk, with weight 0 after its
 // own end, so that the warp stays converged.
 //
+// Cancelling column sums.  An addend is formed again in double from the exact
+// sums (fix_product_dbl) when a normalising shift exceeds s0 = 12 + log2 K (its
+// relative error is then above 2^(s0 - 61)) and that error is more than
+// 2^(s0 - 65) of the lane's largest addend so far, or when a product is lost
+// altogether.  So the error of an addend stays below K 2^-49 of itself or K
+// 2^-53 of the largest one, per pair of columns, for any matrix (two blocks
+// [[B, B], [B + 1, -B]], B = 3^25: 2.8e-7, or all of it with the blocks' columns
+// in different pairs, without this).  Haar matrices need it for one addend of
+// a warp in 300 at 30 columns: 28.6 -> 29.1 ms, 23 columns 214 -> 218 us; the
+// same at s0 - 1: 29.5 ms, with the addends' mean in place of the largest 30.5,
+// with the double product in a function of its own 4 % more.
+//
 // 30 x 30 permanent (2^29 addends): 165 ms in double (FP64 pipe 94 % busy),
-// 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 28.7
+// 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 29.1
 // ms here; 70 cycles per warp, column and addend, of which the 12 integer
 // products hold the FMA-heavy pipe 52 (72 % busy) and 25 other integer
 // instructions take the rest.  Relative error (23 x 23, Haar): 6.8e-15, in
@@ -294,13 +341,40 @@ __device__ void walk_task_perm_fix(const bs_job& jb, const zfix* __restrict__ da
     fix_seed<HX, KP>(c, g, c0, jb.nbin, jb.nrows);
     double ws = signed_weight<double>(g.w, g.parity);
     double acc = 0.0;
+    int emax = -(1 << 28);  // largest exponent of an addend so far
+    const int s0 = 12 + (31 - __clz(jb.K));
     for (uint32_t s = 0; s < steps; ++s) {
-        int e;
-        const zlimb p = fix_product<HX>(c, e);
+        int e, smax, slast;
+        const zlimb p = fix_product<HX>(c, e, smax, slast);
+        if (slast >= 29) e -= 1 << 14;  // zero (or lost): no weight
         const zlimb q = shfl_xor_zlimb(p, 1);
         e += __shfl_xor_sync(0xffffffffu, e, 1) + e_pair;
         const long long v = fix_cmul_part(p, q, half);
-        const double f = s < len ? scale_pow2(ws, e) : 0.0;
+        double f = s < len ? scale_pow2(ws, e) : 0.0;
+        e += __double2hiint(ws) >> 20 & 0x7ff;  // (for comparison, with the weight's exponent)
+        emax = max(emax, e);
+        if (__any_sync(0xffffffffu, smax > s0)) {
+            bool redo = s < len && smax > s0 && (smax >= 28 || e - emax + smax > s0 - 4);
+            if (__any_sync(0xffffffffu, redo)) {
+                bool zero = false;
+#pragma unroll
+                for (int t = 0; t < HX; ++t) zero |= (c[t].re | c[t].im) == 0ull;
+                redo |= __shfl_xor_sync(0xffffffffu, (int)redo, 1) != 0;
+                zero |= __shfl_xor_sync(0xffffffffu, (int)zero, 1) != 0;
+                redo = redo && !zero;
+                cx<double> x = {0.0, 0.0};
+                if (redo) x = fix_product_dbl(c);
+                cx<double> y;
+                y.re = __shfl_xor_sync(0xffffffffu, x.re, 1);
+                y.im = __shfl_xor_sync(0xffffffffu, x.im, 1);
+                if (redo) {
+                    f = 0.0;
+                    // 2 HX columns in units of 2^kDblUnit below their bounds
+                    const double w = scale_pow2(ws, (jb.K & 1) - 2 * HX * kDblUnit);
+                    acc = bfma(w, half ? bfma(x.re, y.im, x.im * y.re) : bfma(x.re, y.re, -(x.im * y.im)), acc);
+                }
+            }
+        }
         acc = bfma(f, (double)v, acc);
         if (((s + 1u) & (FOLD - 1u)) == 0u) {
             sum = dd_add_d(sum, acc);
