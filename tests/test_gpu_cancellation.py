@@ -90,3 +90,42 @@ def test_permanents_of_noise_and_zeros(ctx, K):
     for a in (signs, roots, signs * (1 + 2.0 ** -40 * g.standard_normal((R, K)))):
         got = ctx.perm(a, M, N)
         assert abs(got - sum(oracle.perm_mult(a, M, N))) <= tol(K) * oracle.perm_mult_abs(a, M, N)
+
+
+# Minors: products of normalised sums err by 2^-55 (K + 1 of them enter an
+# addend), an addend's place in its run's integer sum by 3 units of 2^-54 of the
+# run's largest addend of that column (8 in a run), the sums of runs in double
+# by 2^-53 in at most 256 additions before they are folded.
+TOL_MINORS = (48 + 1) * 2.0 ** -55 + 8 * 3 * 2.0 ** -54 + 256 * 2.0 ** -53 + 2.0 ** -50
+
+
+@pytest.mark.parametrize("nb,B,seed", [(1, 3.0 ** 25, 1), (2, 789.0, 2), (2, 3.0 ** 20, 3), (3, 3.0 ** 25, 4), (4, 789.0, 5),
+                                       (4, 3.0 ** 25, 6), (5, 3.0 ** 31, 7), (6, 808037.0, 8)])
+def test_minors_of_cancelling_blocks(ctx, nb, B, seed):
+    K = 2 * nb + 1
+    g = np.random.Generator(np.random.PCG64(seed))
+    a = np.concatenate([blocks(nb, B), g.standard_normal((K - 1, 1))], axis=1)
+    ones, cols = np.ones(K - 1, np.int32), np.ones(K, np.int32)
+    exact = [float(perm_exact(np.delete(a, l, 1))) for l in range(K)]
+    for order in orders(K, seed):
+        got = ctx.laplace_minors(a[:, order], ones, cols)
+        for i, l in enumerate(order):
+            bound = oracle.perm_mult_abs(np.delete(a, l, 1), ones, ones)
+            assert got[i].imag == 0.0 and abs(got[i].real - exact[l]) <= TOL_MINORS * bound, (order, i)
+
+
+@pytest.mark.parametrize("K", [9, 14, 27, 34])
+def test_minors_of_noise_and_zeros(ctx, K):
+    R = min(K - 1, 6)
+    M = np.full(R, (K - 1) // R, np.int32)
+    M[: K - 1 - int(M.sum())] += 1
+    N = np.ones(K, np.int32)
+    g = np.random.Generator(np.random.PCG64(K))
+    signs = g.choice([-1.0, 1.0], size=(R, K))
+    roots = np.exp(2j * np.pi * np.outer(np.arange(R), np.arange(K)) / 12)
+    for a in (signs, roots, signs * (1 + 2.0 ** -40 * g.standard_normal((R, K)))):
+        got = ctx.laplace_minors(a, M, N)
+        for l in (0, K // 2, K - 1):
+            keep = [j for j in range(K) if j != l]
+            ref = sum(oracle.perm_mult(a[:, keep], M, N[keep]))
+            assert abs(got[l] - ref) <= TOL_MINORS * oracle.perm_mult_abs(a[:, keep], M, N[keep]), l
