@@ -64,19 +64,25 @@ struct bs_job {
 //   col_src[K]          source column of each product column
 //   colexp[K]           power-of-two column scale chosen by the pack kernel
 //   pinned_src          source row of the pinned (delta = +1) row
-//   (one int of padding to an 8-byte boundary)
+//   split               1: a column has parts of its own scale (pack kernel)
 //   binom[]             uint64 table written by the pack kernel: for each
 //                       digit j in order, C(M_j, d) for d = 0..M_j
 //                       (nrows + n - 1 entries in all)
-// colexp values of an FP64 column with a component that is not finite (its
+// colexp values: the exponent e of the column's scale, how far the bound of its
+// imaginary part lies below that of its real part (d > 0) or above it (d < 0;
+// both scaled alike: 0), and marks of a component that is not finite (its
 // sum of moduli reaches 2^1022 or is NaN): no finite scale, results NaN.
-#define BS_COLEXP_NAN_RE (1 << 20)
-#define BS_COLEXP_NAN_IM (1 << 21)
+#define BS_COLEXP(e, d) (((e) + 2048) | (((d) + 1024) << 12))
+#define BS_COLEXP_E(x) (((x) & 4095) - 2048)
+#define BS_COLEXP_D(x) ((((x) >> 12) & 2047) - 1024)
+#define BS_COLEXP_NAN_RE (1 << 24)
+#define BS_COLEXP_NAN_IM (1 << 25)
 #define BS_META_RADIX(jb) ((jb).meta_off)
 #define BS_META_DIGIT_SRC(jb) ((jb).meta_off + (jb).nrows)
 #define BS_META_COL_SRC(jb) ((jb).meta_off + 2 * (jb).nrows)
 #define BS_META_COLEXP(jb) ((jb).meta_off + 2 * (jb).nrows + (jb).K)
 #define BS_META_PINNED(jb) ((jb).meta_off + 2 * (jb).nrows + 2 * (jb).K)
+#define BS_META_SPLIT(jb) (BS_META_PINNED(jb) + 1)
 #define BS_META_BINOM(jb) ((jb).meta_off + 2 * (jb).nrows + 2 * (jb).K + 2)
 #define BS_META_SIZE(nrows, K, n) (2 * (nrows) + 2 * (K) + 2 + 2 * ((nrows) + (n)))
 

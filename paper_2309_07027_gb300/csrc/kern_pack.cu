@@ -93,10 +93,8 @@ __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __re
         for (int c = lane; c < K; c += 32) {
             if (minors && c == col) continue;
             const int x = colexp[c];
-            if (x >= BS_COLEXP_NAN_RE)
-                bad |= x;
-            else
-                e += x;
+            bad |= x & (BS_COLEXP_NAN_RE | BS_COLEXP_NAN_IM);
+            e += BS_COLEXP_E(x);
         }
         e = __reduce_add_sync(0xffffffffu, e);
         bad = (int)__reduce_or_sync(0xffffffffu, (unsigned)bad);

@@ -42,6 +42,11 @@ __global__ void __launch_bounds__(kPermBlock, KB <= 32 ? 8 : 6) walk_fp64_perm_k
         ddv re = {0.0, 0.0}, im = {0.0, 0.0};
         if (!ok) {
             if (threadIdx.x == 0) atomicExch(a.status, BS_STATUS_BADJOB);
+        } else if (radix[BS_META_SPLIT(jb) - jb.meta_off] != 0) {
+            if (((jb.K + 1) >> 1) == KB / 2)
+                walk_task_perm_dbl<KB, KB / 2>(jb, data, radix, local, warp, lane, re, im);
+            else
+                walk_task_perm_dbl<KB, KB / 2 - 1>(jb, data, radix, local, warp, lane, re, im);
         } else if (((jb.K + 1) >> 1) == KB / 2) {  // the instance whose lanes own exactly ceil(K / 2) columns
             walk_task_perm_fix<KB, KB / 2>(jb, data, radix, local, warp, lane, re, im);
         } else {

@@ -127,7 +127,11 @@ __device__ __forceinline__ void put_df(void* data, const bs_job& jb, int KP, int
 // FP64 jobs and double-float permanents (walk_fix.cuh): column col scaled by
 // 2^(63 - e), e (stored in colexp) the smallest integer with 2^e > b (1 +
 // 2^-20), b = sum over rows of M_row (|Re a| + |Im a|); every entry rounded
-// once to an integer, c0 and 2a formed from those integers modulo 2^64.
+// once to an integer, c0 and 2a formed from those integers modulo 2^64.  Where
+// one part's bound is less than 1/8 of the other's, each part is scaled by its
+// own (colexp holds the larger and how far the other lies below it) and the
+// job is marked: its addends are formed in double (walk_fix.cuh), which keeps
+// the accuracy of the smaller part.
 // Ryser and Nijenhuis-Wilf jobs: product column col is matrix row sc; digit j
 // is matrix column dsrc[j], added with +1 when it enters the subset, so the
 // packed row is -a (the walk subtracts rows of digits whose Delta is 1);
@@ -160,6 +164,7 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
     const bool bbfg = jb.formula == BS_JOB_BBFG, nw = jb.formula == BS_JOB_NW;
     constexpr int kRows = (BS_MAX_DIGITS + kPackLanes - 1) / kPackLanes;  // digit rows of a lane
     const int part = tid % kPackLanes;
+    int split = 0;
     for (int base = 0; base < KP; base += nthreads / kPackLanes) {  // (every lane runs every round)
         const int col = base + tid / kPackLanes;
         const bool live = col < jb.K;
@@ -205,7 +210,16 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
 #pragma unroll
             for (int i = 0; i < kRows; ++i) a[i] = make_double2(0.0, 0.0);
         }
-        if (live && part == 0) colexp[col] = flags ? flags : e;
+        int ere = e, eim = e;
+        if (!f32 && !df && !flags && bre > 0.0 && bim > 0.0 && (bre < 0.125 * bim || bim < 0.125 * bre)) {
+            (void)frexp(0.25 * bre * (1.0 + 0x1p-20), &ere);
+            (void)frexp(0.25 * bim * (1.0 + 0x1p-20), &eim);
+            ere = max(ere, eim - 900) + 2;
+            eim = max(eim + 2, ere - 900);
+            e = max(ere, eim);
+            split |= live;
+        }
+        if (live && part == 0) colexp[col] = flags | BS_COLEXP(e, ere - eim);
         if (f32 || df) {
             __int128 sre = wide_of(a0.x, e), sim = wide_of(a0.y, e);
 #pragma unroll
@@ -232,15 +246,15 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
             continue;
         }
         zfix* out = static_cast<zfix*>(data) + jb.data_off;
-        const int sh = nw ? 62 - e : 63 - e;
-        unsigned long long sre = (unsigned long long)__double2ll_rn(scale2(a0.x, sh));  // the start sums
-        unsigned long long sim = (unsigned long long)__double2ll_rn(scale2(a0.y, sh));
+        const int shre = (nw ? 62 : 63) - ere, shim = (nw ? 62 : 63) - eim;
+        unsigned long long sre = (unsigned long long)__double2ll_rn(scale2(a0.x, shre));  // the start sums
+        unsigned long long sim = (unsigned long long)__double2ll_rn(scale2(a0.y, shim));
 #pragma unroll
         for (int i = 0; i < kRows; ++i) {
             if (kPackLanes * i >= jb.nrows) break;
             const int j = part + kPackLanes * i;
-            const unsigned long long qre = (unsigned long long)__double2ll_rn(scale2(a[i].x, sh));
-            const unsigned long long qim = (unsigned long long)__double2ll_rn(scale2(a[i].y, sh));
+            const unsigned long long qre = (unsigned long long)__double2ll_rn(scale2(a[i].x, shre));
+            const unsigned long long qim = (unsigned long long)__double2ll_rn(scale2(a[i].y, shim));
             zfix row;
             if (bbfg) {
                 sre += (unsigned long long)m[i] * qre;
@@ -265,6 +279,9 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
         // a pad column's sum is exactly 1 = 2^62 / 2^63 2^1
         if (part == 0 && col < KP) out[col] = live ? zfix{(long long)sre, (long long)sim} : zfix{1ll << 62, 0};
     }
+    if (f32 || df) return;
+    split = __syncthreads_or(split);
+    if (tid == 0) meta[BS_META_SPLIT(jb)] = split ? 1 : 0;
 }
 
 }  // namespace bs

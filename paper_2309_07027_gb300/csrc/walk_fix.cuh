@@ -271,6 +271,19 @@ __device__ __forceinline__ cx<double> fix_product_dbl(const zraw (&c)[N]) {
     return p;
 }
 
+// A column sum in those units, with parts of their own scales; x: the column's
+// colexp.
+__device__ __forceinline__ cx<double> split_column(const zraw& c, int x) {
+    const int d = BS_COLEXP_D(x);
+    return cx<double>{scale_int((long long)c.re, kDblUnit - 63 + min(d, 0)),
+                      scale_int((long long)c.im, kDblUnit - 63 - max(d, 0))};
+}
+// colexp of column t of a lane's columns, which begin with column `first` (a
+// pad column: parts of one scale).
+__device__ __forceinline__ int lane_colexp(const bs_job& jb, const int* __restrict__ radix, int first, int t) {
+    return first + t < jb.K ? radix[BS_META_COLEXP(jb) - jb.meta_off + first + t] : BS_COLEXP(0, 0);
+}
+
 __device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
     zlimb o;
     o.rh = __shfl_xor_sync(0xffffffffu, v.rh, mask);
@@ -392,6 +405,62 @@ __device__ void walk_task_perm_fix(const bs_job& jb, const zfix* __restrict__ da
     }
     sum = dd_add_d(sum, acc);
     // over the 16 lanes of each part, then the imaginary part to lane 0
+#pragma unroll
+    for (int off = 16; off > 1; off >>= 1) sum = dd_add_sum2(sum, shfl_down_dd(sum, off));
+    im = shfl_down_dd(sum, 1);
+}
+
+// The same task with every addend in double from the exact sums: jobs with
+// columns of very unequal parts, whose smaller parts the products above would
+// round at the larger ones' scale (a 5 x 5 matrix with imaginary parts of 1e-9:
+// 1.6e-10 of Im, here 1e-15).  Up to 6 FP64 instructions per column and addend,
+// the pipe's time for a product of doubles.
+template <int KB, int HX>
+__device__ __noinline__ void walk_task_perm_dbl(const bs_job& jb, const zfix* __restrict__ data,
+                                                const int* __restrict__ radix, uint32_t local, int half_task, int lane,
+                                                ddv& sum, ddv& im) {
+    const int half = lane & 1;
+    const zfix* c0 = data + jb.data_off + half * HX;
+    sum = im = ddv{0.0, 0.0};
+    const uint64_t i0_own = ((uint64_t)local * 32u + (uint64_t)(16 * half_task + (lane >> 1))) << jb.log2L;
+    const uint64_t i0 = i0_own < jb.C ? i0_own : 0ull;
+    const uint64_t rem = i0_own < jb.C ? jb.C - i0_own : 0ull;
+    const uint32_t len = (uint32_t)(rem < (1ull << jb.log2L) ? rem : (1ull << jb.log2L));
+    const uint32_t steps = __reduce_max_sync(0xffffffffu, len);
+    if (steps == 0u) return;
+    bs_gray g;
+    ChunkStepper st;
+    st.init(g, i0, jb.nbin, jb.nrows, radix, reinterpret_cast<const uint64_t*>(radix + (BS_META_BINOM(jb) - jb.meta_off)));
+    zraw c[HX];
+    fix_seed<HX, KB>(c, g, c0, jb.nbin, jb.nrows);
+    double ws = signed_weight<double>(g.w, g.parity), acc = 0.0;
+    for (uint32_t s = 0; s < steps; ++s) {
+        cx<double> x;
+#pragma unroll
+        for (int t = 0; t < HX; ++t) {
+            const cx<double> v = split_column(c[t], lane_colexp(jb, radix, half * HX, t));
+            x = t ? cmul(x, v) : v;
+        }
+        cx<double> y;
+        y.re = __shfl_xor_sync(0xffffffffu, x.re, 1);
+        y.im = __shfl_xor_sync(0xffffffffu, x.im, 1);
+        const double w = s < len ? scale_pow2(ws, (jb.K & 1) - 2 * HX * kDblUnit) : 0.0;
+        acc = bfma(w, half ? bfma(x.re, y.im, x.im * y.re) : bfma(x.re, y.re, -(x.im * y.im)), acc);
+        if (((s + 1u) & 63u) == 0u) {
+            sum = dd_add_d(sum, acc);
+            acc = 0.0;
+        }
+        if (s + 1 == steps) break;
+        uint32_t neg = 0;
+        int row = 0;
+        if (s + 1 < len) {
+            int wch;
+            row = st.step(g, s, radix, &neg, &wch);
+            ws = wch ? signed_weight<double>(g.w, g.parity) : flip_sign(ws);
+        }
+        fix_update<HX>(c, c0 + (size_t)(1 + row) * KB, neg);
+    }
+    sum = dd_add_d(sum, acc);
 #pragma unroll
     for (int off = 16; off > 1; off >>= 1) sum = dd_add_sum2(sum, shfl_down_dd(sum, off));
     im = shfl_down_dd(sum, 1);
@@ -612,10 +681,9 @@ __device__ __forceinline__ double2* dbl_slot(longlong2* sm_leaf, int4* sm_pair, 
     return t < NP ? reinterpret_cast<double2*>(sm_leaf + t * 32) : reinterpret_cast<double2*>(sm_pair + (t - NP) * 32);
 }
 template <int G, int HX>
-__device__ __forceinline__ void minors_addend_dbl(const zraw (&c)[HX], double w, longlong2* sm_leaf, int4* sm_pair) {
-    auto column = [&](int t) {
-        return cx<double>{scale_int((long long)c[t].re, kDblUnit - 63), scale_int((long long)c[t].im, kDblUnit - 63)};
-    };
+__device__ __forceinline__ void minors_addend_dbl(const zraw (&c)[HX], const bs_job& jb, const int* __restrict__ radix,
+                                                  int first, double w, longlong2* sm_leaf, int4* sm_pair) {
+    auto column = [&](int t) { return split_column(c[t], lane_colexp(jb, radix, first, t)); };
     auto swap = [](const cx<double>& v, int mask) {
         return cx<double>{__shfl_xor_sync(0xffffffffu, v.re, mask), __shfl_xor_sync(0xffffffffu, v.im, mask)};
     };
@@ -661,7 +729,8 @@ __device__ __forceinline__ void minors_flush_dbl(MinorsSmem<G, HX>& sm, int lane
 }
 
 // The whole task with the addends of minors_addend_dbl, summed per lane in
-// double in runs of 64.
+// double in runs of 64: tasks whose integer sums came too close to their
+// units, and jobs with columns of very unequal parts.
 template <int G, int KB, int HX>
 __device__ __noinline__ void walk_task_minors_dbl(const bs_job& jb, const zfix* __restrict__ data,
                                                   const int* __restrict__ radix, uint32_t local, int lane,
@@ -687,7 +756,7 @@ __device__ __noinline__ void walk_task_minors_dbl(const bs_job& jb, const zfix* 
         double ws = signed_weight<double>(g.w, g.parity);
         for (uint32_t s = 0; s < steps; ++s) {
             const double w = s < len ? scale_pow2(ws, (G * HX - K) - (G * HX - 1) * kDblUnit) : 0.0;
-            minors_addend_dbl<G, HX>(c, w, sm.leaf + lane, sm.pair + lane);
+            minors_addend_dbl<G, HX>(c, jb, radix, q * HX, w, sm.leaf + lane, sm.pair + lane);
 #pragma unroll
             for (int t = 0; t < HX; ++t) {
                 const double2 v = *dbl_slot<HX>(sm.leaf + lane, sm.pair + lane, t);
@@ -783,7 +852,8 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
         sm.est[t] = make_float2(0.f, __int_as_float(-(1 << 24)));
     }
     const int s0 = 13 + (31 - __clz(K));
-    for (int round = 0; round < G / 2; ++round) {
+    bool dbl = radix[BS_META_SPLIT(jb) - jb.meta_off] != 0;  // (columns of very unequal parts)
+    for (int round = 0; round < G / 2 && !dbl; ++round) {
         const uint64_t i0_own = ((uint64_t)local * 16u + (uint64_t)(round * (32 / G) + lane / G)) << jb.log2L;
         const bool has = i0_own < jb.C;
         const uint64_t i0 = has ? i0_own : 0ull;
@@ -892,9 +962,8 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
             fix_update<HX>(c, a2 + (size_t)row * KP, neg);
         }
     }
-    bool bad = false;
-    for (int t = lane; t < K; t += 32) bad |= sm.est[t].x < 0.f;
-    if (__any_sync(0xffffffffu, bad)) walk_task_minors_dbl<G, KB, HX>(jb, data, radix, local, lane, sm);
+    for (int t = lane; t < K; t += 32) dbl |= sm.est[t].x < 0.f;
+    if (__any_sync(0xffffffffu, dbl)) walk_task_minors_dbl<G, KB, HX>(jb, data, radix, local, lane, sm);
     for (int t = lane; t < K; t += 32) {
         const double4 v = sm.tot[t];
         store_partial(partials + jb.partial_off + (int64_t)local * K + t, ddv{v.x, v.y}, ddv{v.z, v.w});
