@@ -226,6 +226,18 @@ __device__ __forceinline__ zraw fix_leaf(const zraw (&c)[N], int j) {
     return zraw{(unsigned long long)((long long)c[2 * j].re >> 1), (unsigned long long)((long long)c[2 * j].im >> 1)};
 }
 
+// A column sum (below 2^63) normalised, and its shift (-1..60).
+__device__ __forceinline__ zlimb norm_column(const zraw& v, int& k) {
+    zraw n = v;
+    k = fix_norm_shift(v);
+    if (k < 0) n = zraw{(unsigned long long)((long long)v.re >> 1), (unsigned long long)((long long)v.im >> 1)};
+    if (k > 0) n = zraw{v.re << k, v.im << k};
+    if (k < 29) return limbs_of(n);
+    const int k2 = fix_norm_shift(n);
+    k += k2;
+    return fix_shift(n, k2);
+}
+
 // Product of a lane's N column sums as a normalised operand, and its exponent
 // against the column bounds: leaves (independent of one another), then their
 // running product, normalised after every leaf.  A typical column sum is
@@ -233,44 +245,41 @@ __device__ __forceinline__ zraw fix_leaf(const zraw (&c)[N], int j) {
 // 2^55, and a pair times a normalised operand 2^52.5, so a pair costs about
 // 2^-54 in relative rounding, where two products of doubles cost 2^-53.  Sums
 // that cancel lose more: smax is the largest of the normalising shifts, so the
-// relative error is a few 2^(smax - 61), and slast the last one (29 or 30:
-// the product is zero, or has lost everything; smax shows it as well).
-template <int N>
-__device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e, int& smax, int& slast) {
-    e = kLeafExp;
-    zraw r = fix_leaf(c, 0);
-    slast = fix_norm_shift(r);
-    smax = slast;
-    e -= slast;
-    zlimb p = fix_shift(r, slast);
+// relative error is a few 2^(smax - 61).  NORM: leaves of normalised column
+// sums, 2^-56 at most for any sums.  A product that is zero (or lost: smax
+// shows it) has a last shift of 29 or 30 and gets no weight.
+template <int NORM, int N>
+__device__ __forceinline__ zlimb fix_product(const zraw (&c)[N], int& e, int& smax) {
+    zlimb p;
+    int s = 0;
+    smax = 0;
+    e = -64;
 #pragma unroll
-    for (int j = 1; 2 * j < N; ++j) {
-        r = fix_cmul(p, limbs_of(fix_leaf(c, j)));
-        slast = fix_norm_shift(r);
-        smax = max(smax, slast);
-        e += 64 + kLeafExp - slast;
-        p = fix_shift(r, slast);
+    for (int j = 0; 2 * j < N; ++j) {
+        zraw leaf;
+        e += 64 + kLeafExp;
+        if (NORM) {
+            int ka, kb = 1;
+            const zlimb a = norm_column(c[2 * j], ka);
+            leaf = 2 * j + 1 < N ? fix_cmul<0>(a, norm_column(c[2 * j + 1], kb)) : raw_of(a);
+            e -= ka + kb;
+        } else {
+            leaf = fix_leaf(c, j);
+        }
+        const zraw r = j ? fix_cmul(p, limbs_of(leaf)) : leaf;
+        s = fix_norm_shift(r);
+        smax = max(smax, s);
+        e -= s;
+        p = fix_shift(r, s);
     }
+    if (s >= 29) e -= 1 << 14;
     return p;
 }
 
-// Product of n column sums in double, in units of kDblUnit bits below each
-// column's bound (so that 48 columns at their bounds stay in range, as do
-// products 2^-1800 below them): every factor is the exact sum rounded once, so
-// the product is as accurate as a product of doubles, however much the sums
-// cancelled.  6 FP64 instructions per column: for the addends that need it.
+// Exact column sums in double, in units of kDblUnit bits below each column's
+// bound: 48 columns at their bounds stay in range, as do products 2^-1800 below
+// them.
 constexpr int kDblUnit = 18;
-template <int N>
-__device__ __forceinline__ cx<double> fix_product_dbl(const zraw (&c)[N]) {
-    cx<double> p;
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        const cx<double> x = {scale_int((long long)c[j].re, kDblUnit - 63), scale_int((long long)c[j].im, kDblUnit - 63)};
-        p = j ? cmul(p, x) : x;
-    }
-    return p;
-}
-
 // A column sum in those units, with parts of their own scales; x: the column's
 // colexp.
 __device__ __forceinline__ cx<double> split_column(const zraw& c, int x) {
@@ -307,17 +316,18 @@ __device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
 // lane 0.  Every lane walks the warp's longest chunk, with weight 0 after its
 // own end, so that the warp stays converged.
 //
-// Cancelling column sums.  An addend is formed again in double from the exact
-// sums (fix_product_dbl) when a normalising shift exceeds s0 = 12 + log2 K (its
+// Cancelling column sums.  An addend is formed again from normalised sums
+// (fix_product<1>) when a normalising shift exceeds s0 = 12 + log2 K (its
 // relative error is then above 2^(s0 - 61)) and that error is more than
-// 2^(s0 - 65) of the lane's largest addend so far, or when a product is lost
-// altogether.  So the error of an addend stays below K 2^-49 of itself or K
-// 2^-53 of the largest one, per pair of columns, for any matrix (two blocks
-// [[B, B], [B + 1, -B]], B = 3^25: 2.8e-7, or all of it with the blocks' columns
-// in different pairs, without this).  Haar matrices need it for one addend of
-// a warp in 300 at 30 columns: 28.6 -> 29.1 ms, 23 columns 214 -> 218 us; the
-// same at s0 - 1: 29.5 ms, with the addends' mean in place of the largest 30.5,
-// with the double product in a function of its own 4 % more.
+// 2^(s0 - 65) of the lane's largest addend so far, or when a product that is
+// not zero is lost altogether.  So the error of an addend stays below K 2^-49 of
+// itself or K 2^-53 of the largest one, per pair of columns, for any matrix (two
+// blocks [[B, B], [B + 1, -B]], B = 3^25: 2.8e-7, or all of it with the blocks'
+// columns in different pairs, without this).  Haar matrices need it for one
+// addend of a warp in 300 at 30 columns: 28.6 -> 29.1 ms, 23 columns 214 -> 221
+// us (at s0 - 1 29.4 ms and 223 us; formed in double instead, 6 FP64
+// instructions per column, the same for Haar matrices, but 1.9 ms instead of
+// 0.9 for 24 columns of roots of unity, whose sums cancel more often).
 //
 // 30 x 30 permanent (2^29 addends): 165 ms in double (FP64 pipe 94 % busy),
 // 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 29.1
@@ -357,34 +367,24 @@ __device__ void walk_task_perm_fix(const bs_job& jb, const zfix* __restrict__ da
     int emax = -(1 << 28);  // largest exponent of an addend so far
     const int s0 = 12 + (31 - __clz(jb.K));
     for (uint32_t s = 0; s < steps; ++s) {
-        int e, smax, slast;
-        const zlimb p = fix_product<HX>(c, e, smax, slast);
-        if (slast >= 29) e -= 1 << 14;  // zero (or lost): no weight
-        const zlimb q = shfl_xor_zlimb(p, 1);
+        int e, smax;
+        zlimb p = fix_product<0, HX>(c, e, smax);
+        long long v = fix_cmul_part(p, shfl_xor_zlimb(p, 1), half);
         e += __shfl_xor_sync(0xffffffffu, e, 1) + e_pair;
-        const long long v = fix_cmul_part(p, q, half);
         double f = s < len ? scale_pow2(ws, e) : 0.0;
         e += __double2hiint(ws) >> 20 & 0x7ff;  // (for comparison, with the weight's exponent)
         emax = max(emax, e);
         if (__any_sync(0xffffffffu, smax > s0)) {
             bool redo = s < len && smax > s0 && (smax >= 28 || e - emax + smax > s0 - 4);
             if (__any_sync(0xffffffffu, redo)) {
-                bool zero = false;
 #pragma unroll
-                for (int t = 0; t < HX; ++t) zero |= (c[t].re | c[t].im) == 0ull;
-                redo |= __shfl_xor_sync(0xffffffffu, (int)redo, 1) != 0;
-                zero |= __shfl_xor_sync(0xffffffffu, (int)zero, 1) != 0;
-                redo = redo && !zero;
-                cx<double> x = {0.0, 0.0};
-                if (redo) x = fix_product_dbl(c);
-                cx<double> y;
-                y.re = __shfl_xor_sync(0xffffffffu, x.re, 1);
-                y.im = __shfl_xor_sync(0xffffffffu, x.im, 1);
-                if (redo) {
-                    f = 0.0;
-                    // 2 HX columns in units of 2^kDblUnit below their bounds
-                    const double w = scale_pow2(ws, (jb.K & 1) - 2 * HX * kDblUnit);
-                    acc = bfma(w, half ? bfma(x.re, y.im, x.im * y.re) : bfma(x.re, y.re, -(x.im * y.im)), acc);
+                for (int t = 0; t < HX; ++t) redo = redo && (c[t].re | c[t].im) != 0ull;
+                if (__any_sync(0xffffffffu, redo)) {
+                    p = fix_product<1, HX>(c, e, smax);
+                    v = fix_cmul_part(p, shfl_xor_zlimb(p, 1), half);
+                    e += __shfl_xor_sync(0xffffffffu, e, 1) + e_pair;
+                    f = s < len ? scale_pow2(ws, e) : 0.0;
+                    emax = max(emax, e + (__double2hiint(ws) >> 20 & 0x7ff));
                 }
             }
         }
@@ -561,18 +561,6 @@ __device__ __forceinline__ zlimb fix_normalise(const zraw& v, int& e, int& smax)
     return fix_shift(v, s);
 }
 
-// A column sum (below 2^63) normalised, and its shift (-1..60).
-__device__ __forceinline__ zlimb norm_column(const zraw& v, int& k) {
-    zraw n = v;
-    k = fix_norm_shift(v);
-    if (k < 0) n = zraw{(unsigned long long)((long long)v.re >> 1), (unsigned long long)((long long)v.im >> 1)};
-    if (k > 0) n = zraw{v.re << k, v.im << k};
-    if (k < 29) return limbs_of(n);
-    const int k2 = fix_norm_shift(n);
-    k += k2;
-    return fix_shift(n, k2);
-}
-
 // Leaf j of the minors.  NORM: of normalised column sums, and their shifts in
 // byte j of ls (plus kLeafBias); else fix_leaf.  Its exponent is leaf_exp.
 constexpr int kLeafBias = 2;
@@ -683,15 +671,17 @@ __device__ __forceinline__ double2* dbl_slot(longlong2* sm_leaf, int4* sm_pair, 
 template <int G, int HX>
 __device__ __forceinline__ void minors_addend_dbl(const zraw (&c)[HX], const bs_job& jb, const int* __restrict__ radix,
                                                   int first, double w, longlong2* sm_leaf, int4* sm_pair) {
-    auto column = [&](int t) { return split_column(c[t], lane_colexp(jb, radix, first, t)); };
+    cx<double> x[HX];
+#pragma unroll
+    for (int t = 0; t < HX; ++t) x[t] = split_column(c[t], lane_colexp(jb, radix, first, t));
     auto swap = [](const cx<double>& v, int mask) {
         return cx<double>{__shfl_xor_sync(0xffffffffu, v.re, mask), __shfl_xor_sync(0xffffffffu, v.im, mask)};
     };
-    cx<double> r = column(HX - 1);
+    cx<double> r = x[HX - 1];
 #pragma unroll
     for (int t = HX - 2; t >= 0; --t) {
         *dbl_slot<HX>(sm_leaf, sm_pair, t) = make_double2(r.re, r.im);
-        r = cmul(r, column(t));
+        r = cmul(r, x[t]);
     }
     cx<double> p = swap(r, 1);
     if constexpr (G == 4) p = cmul(p, swap(cmul(r, p), 2));
@@ -702,7 +692,7 @@ __device__ __forceinline__ void minors_addend_dbl(const zraw (&c)[HX], const bs_
         double2* slot = dbl_slot<HX>(sm_leaf, sm_pair, t);
         const cx<double> v = t + 1 < HX ? cmul(p, cx<double>{slot->x, slot->y}) : p;
         *slot = make_double2(v.re, v.im);
-        if (t + 1 < HX) p = cmul(p, column(t));
+        if (t + 1 < HX) p = cmul(p, x[t]);
     }
 }
 
@@ -890,7 +880,19 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
 #pragma unroll
             for (int j = 0; j < (NP + 3) / 4; ++j) ls[j] = 0x01010101u * kLeafBias;
             suffix_chains<0, HX>(c, ls, qa, qb, ea, eb, smax, es, sm_leaf, sm_pair);
-            if (__any_sync(0xffffffffu, smax > s0)) suffix_chains<1, HX>(c, ls, qa, qb, ea, eb, smax, es, sm_leaf, sm_pair);
+            if (__any_sync(0xffffffffu, smax > s0)) {
+                // (a sum that is zero is exact, and with the others above 2^55
+                // every other pair is accurate)
+                bool zero = false, small = false;
+#pragma unroll
+                for (int t = 0; t < HX; ++t) {
+                    const bool z = (c[t].re | c[t].im) == 0ull;
+                    zero |= z;
+                    small |= !z && (abs((int)(c[t].re >> 32)) | abs((int)(c[t].im >> 32))) < 1 << 23;
+                }
+                if (__any_sync(0xffffffffu, smax > s0 && (small || !zero)))
+                    suffix_chains<1, HX>(c, ls, qa, qb, ea, eb, smax, es, sm_leaf, sm_pair);
+            }
             {
                 zraw ra;
                 e = ea;
