@@ -70,8 +70,7 @@ struct bs_job {
 //                       (nrows + n - 1 entries in all)
 // colexp values: the exponent e of the column's scale, how far the bound of its
 // imaginary part lies below that of its real part (d > 0) or above it (d < 0;
-// both scaled alike: 0), and marks of a component that is not finite (its
-// sum of moduli reaches 2^1022 or is NaN): no finite scale, results NaN.
+// both scaled alike: 0), and marks of a part with an entry that is not finite.
 #define BS_COLEXP(e, d) (((e) + 2048) | (((d) + 1024) << 12))
 #define BS_COLEXP_E(x) (((x) & 4095) - 2048)
 #define BS_COLEXP_D(x) ((((x) >> 12) & 2047) - 1024)

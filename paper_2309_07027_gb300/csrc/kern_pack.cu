@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __re
     x = sgn * scale2(x, e);
     // an input that is not finite (a product of two or more columns mixes
     // both components)
-    if (bad && (K > 1 || (bad & ((lane & 1) ? BS_COLEXP_NAN_IM : BS_COLEXP_NAN_RE))))
+    if (bad && (K - (minors ? 1 : 0) > 1 || (bad & ((lane & 1) ? BS_COLEXP_NAN_IM : BS_COLEXP_NAN_RE))))
         x = __longlong_as_double(0x7ff8000000000000ll);
     double2* o = lane < 2 ? out : out_lo;
     if (o) reinterpret_cast<double*>(o + jb.out_index + col)[lane & 1] = x;

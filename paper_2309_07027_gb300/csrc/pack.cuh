@@ -138,8 +138,9 @@ __device__ __forceinline__ void put_df(void* data, const bs_job& jb, int KP, int
 // start sums 0 (Ryser) or x = a_(sc, n-1) - (sum_j a_(sc, j)) / 2
 // (Nijenhuis-Wilf, whose entries are rounded to even integers so that the
 // half is exact).
-// A column with an entry that is not finite gets zeros and BS_COLEXP_NAN_*:
-// the reduce kernel writes NaN wherever such a column enters the product.
+// A column with an entry that is not finite gets zeros in that part and
+// BS_COLEXP_NAN_*: the reduce kernel writes NaN wherever such a column enters
+// a product.
 __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __restrict__ src, int* __restrict__ meta,
                                          void* __restrict__ data, int prec, int tid, int nthreads) {
     const bool df = BS_DF_MINORS(prec, jb.kind), f32 = prec == BS_PREC_FP32;
@@ -195,27 +196,52 @@ __device__ __forceinline__ void pack_job(const bs_job& jb, const double2* __rest
             bre += __shfl_xor_sync(0xffffffffu, bre, s);
             bim += __shfl_xor_sync(0xffffffffu, bim, s);
         }
+        // columns near the ends of the exponent range: the bounds once more, of
+        // entries scaled by 2^up (finite entries may overflow in their sum, and
+        // bounds of subnormal ones lose their bits below)
+        int up = 0;
+        const bool end = !(bre + bim < 0x1p1000) || (bre + bim < 0x1p-900 && bre + bim > 0.0);
+        if (__any_sync(0xffffffffu, end)) {
+            if (end) up = bre + bim < 1.0 ? 200 : -12;
+            bre = fabs(scale2(a0.x, up));
+            bim = fabs(scale2(a0.y, up));
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                bre += (double)m[i] * fabs(scale2(a[i].x, up));
+                bim += (double)m[i] * fabs(scale2(a[i].y, up));
+            }
+#pragma unroll
+            for (int s = 1; s < kPackLanes; s <<= 1) {
+                bre += __shfl_xor_sync(0xffffffffu, bre, s);
+                bim += __shfl_xor_sync(0xffffffffu, bim, s);
+            }
+        }
         int flags = 0;
         if (!isfinite(bre)) flags |= BS_COLEXP_NAN_RE;
         if (!isfinite(bim)) flags |= BS_COLEXP_NAN_IM;
+        if ((flags & BS_COLEXP_NAN_RE) || !live) {
+            bre = a0.x = 0.0;
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) a[i].x = 0.0;
+        }
+        if ((flags & BS_COLEXP_NAN_IM) || !live) {
+            bim = a0.y = 0.0;
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) a[i].y = 0.0;
+        }
         int e = 0;
-        const double b = 0.25 * bre + 0.25 * bim;  // a quarter: b must not overflow
-        if (!flags && b > 0.0) {
+        const double b = bre + bim;
+        if (b > 0.0) {
             (void)frexp(f32 || df ? b : b * (1.0 + 0x1p-20), &e);
-            e += 2;
+            e -= up;
         }
         if (df) e -= 2;  // column sums up to 4 (walk_df.cuh)
-        if (flags || !live) {
-            a0 = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int i = 0; i < kRows; ++i) a[i] = make_double2(0.0, 0.0);
-        }
         int ere = e, eim = e;
         if (!f32 && !df && !flags && bre > 0.0 && bim > 0.0 && (bre < 0.125 * bim || bim < 0.125 * bre)) {
-            (void)frexp(0.25 * bre * (1.0 + 0x1p-20), &ere);
-            (void)frexp(0.25 * bim * (1.0 + 0x1p-20), &eim);
-            ere = max(ere, eim - 900) + 2;
-            eim = max(eim + 2, ere - 900);
+            (void)frexp(bre * (1.0 + 0x1p-20), &ere);
+            (void)frexp(bim * (1.0 + 0x1p-20), &eim);
+            ere = max(ere, eim - 900) - up;
+            eim = max(eim - up, ere - 900);
             e = max(ere, eim);
             split |= live;
         }
