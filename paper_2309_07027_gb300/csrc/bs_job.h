@@ -103,6 +103,12 @@ struct bs_job {
 // take 38.7 ms where the fixed point takes 45.2.
 #define BS_DF_MINORS(prec, kind) ((prec) == BS_PREC_DF && (kind) == BS_KIND_MINORS)
 
+// Task partials of the fixed-point kernels are in units of 2^-BS_FIX_BIAS of the
+// product of the column bounds, so that addends far below it keep their
+// digits; the reduce kernel takes the factor out.
+#define BS_FIX_BIAS 512
+#define BS_FIXED(prec, kind) ((prec) == BS_PREC_FP64 || ((prec) == BS_PREC_DF && (kind) == BS_KIND_PERM))
+
 // Precision of a job: the kernel family that walks it.
 //   FP64: 64-bit fixed point (walk_fix.cuh; data in pairs of 64-bit integers);
 //   FP32: single-precision packed pairs (data in complex floats);

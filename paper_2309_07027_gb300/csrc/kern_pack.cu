@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __re
         e += 1;
         sgn = ((jb.n - 1) & 1) ? -1.0 : 1.0;
     }
+    if (BS_FIXED(jb.prec, jb.kind)) e -= BS_FIX_BIAS;
     re = sum2_final(re);
     im = sum2_final(im);
     const double rh = __shfl_sync(0xffffffffu, re.hi, 0), rl = __shfl_sync(0xffffffffu, re.lo, 0);

@@ -130,14 +130,11 @@ __device__ __forceinline__ zlimb fix_normalise(const zraw& v, int& e) {
     return fix_shift(v, s);
 }
 
-// 2^e w for w a nonzero double of magnitude below 2^64, by the exponent
-// field; e clamped so that the result stays normal (a product 2^-900 below
-// the column bounds adds nothing to a sum of them), and zero for e below
-// -8000 (the exponent of a product that is zero).
+// 2^(e + BS_FIX_BIAS) w for w a nonzero double of magnitude 1 to 2^64, by the
+// exponent field; zero where that is below 2^-1000 (an addend 2^-1450 below the
+// column bounds, or the exponent of a product that is zero).
 __device__ __forceinline__ double scale_pow2(double w, int e) {
-    if (e < -8000) return 0.0;
-    if (e < -900) e = -900;
-    return __hiloint2double(__double2hiint(w) + (e << 20), __double2loint(w));
+    return e < -1000 - BS_FIX_BIAS ? 0.0 : __hiloint2double(__double2hiint(w) + ((e + BS_FIX_BIAS) << 20), __double2loint(w));
 }
 
 // v 2^e as a double (e: a constant that keeps the result normal).
@@ -521,11 +518,11 @@ __device__ __forceinline__ float2 minors_look(float2 est, const longlong2* __res
 // 2^exp, to the column's plain-double sum, and clears the sums; with fold, the
 // plain-double sum goes to the column's double-double total.
 template <int G, int HX>
-__device__ __forceinline__ void minors_flush_fix(MinorsSmem<G, HX>& sm, double f, const int (&em)[(HX + 1) / 2],
+__device__ __forceinline__ void minors_flush_fix(MinorsSmem<G, HX>& sm, double f, int e_unit, const int (&em)[(HX + 1) / 2],
                                                  int lane, int K, bool fold, bool look) {
     if ((lane & (G - 1)) == 0) sm.fac[lane / G] = f;
 #pragma unroll
-    for (int j = 0; j < (HX + 1) / 2; ++j) sm.pair[j * 32 + lane].x = em[j];
+    for (int j = 0; j < (HX + 1) / 2; ++j) sm.pair[j * 32 + lane].x = em[j] + e_unit;
     __syncwarp();
 #pragma unroll 1
     for (int t = lane; t < K; t += 32) {
@@ -947,10 +944,10 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
             }
             // the end of a run
             if (((s + 1u) & run_mask) == 0u || s + 1 == steps) {
-                const double f = scale_pow2(((runs ^ flip) & 1u) ? -wrun : wrun, e_unit);
+                const double f = ((runs ^ flip) & 1u) ? -wrun : wrun;
                 const bool look = runs * 0x9e3779b9u < 1u << 29;
                 ++runs;
-                minors_flush_fix<G, HX>(sm, f, em, lane, K, (runs & (kFixFold - 1u)) == 0u || s + 1 == steps, look);
+                minors_flush_fix<G, HX>(sm, f, e_unit, em, lane, K, (runs & (kFixFold - 1u)) == 0u || s + 1 == steps, look);
             }
             if (s + 1 == steps) break;
             uint32_t neg = 0;

@@ -48,3 +48,17 @@ def test_one_part_that_is_not_finite(ctx):
         assert math.isnan(v.imag) and v.real == -2.0
         m = ctx.laplace_minors(np.array([[complex(bad, 3.0), 5.0]]), [1], one(2))
         assert m[0] == 5.0 and math.isnan(m[1].real) and m[1].imag == 3.0
+
+
+def test_addends_far_below_the_column_bounds(ctx):
+    """Sixteen blocks [[B, B], [B + 1, -B]], B = 2^52: every nonzero addend is
+    2^-848 of the product of the column bounds, and the permanent is B^16.
+    Tolerance: K^2 2^-47 of the modulus sum, which is the permanent."""
+    B, nb = 2.0 ** 52, 16
+    K = 2 * nb
+    a = np.kron(np.eye(nb), np.array([[B, B], [B + 1, -B]]))
+    got = ctx.perm(a, one(K), one(K))
+    assert got.imag == 0.0 and abs(got.real / B ** nb - 1.0) <= K * K * 2.0 ** -47
+    r = np.concatenate([a[:28, :28], np.ones((28, 1))], axis=1)
+    m = ctx.laplace_minors(r, one(28), one(29))
+    assert m[28].imag == 0.0 and abs(m[28].real / B ** 14 - 1.0) <= K * K * 2.0 ** -47
