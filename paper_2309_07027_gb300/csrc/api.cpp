@@ -298,7 +298,7 @@ bool valid_mode(bs_mode mode) { return mode == BS_FP64 || mode == BS_MIXED || mo
 struct Prepared {
     struct Group {
         size_t first, last;
-        int prec, kind, kmax;
+        int prec, kind, kmax, groups;
         unsigned long long tasks;
     };
     std::vector<Group> groups;
@@ -314,7 +314,7 @@ struct Prepared {
 int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
     struct Row {
         JobIn in;
-        int prec, kind, bucket, log2L, cpt, ncols, reseed;
+        int prec, kind, bucket, log2L, cpt, ncols, reseed, walk, fold;
         uint32_t ntasks;
     };
     std::vector<Row> rows;
@@ -337,14 +337,13 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
         r.bucket = BS_DF_MINORS(r.prec, r.kind) ? (in.p->K + 7) >> 3 : (in.p->K + 3) >> 2;
         r.cpt = bs_chunks_per_task(r.kind, r.prec, in.p->K);
         r.ncols = r.kind == BS_KIND_PERM ? 1 : in.p->K;
-        const bool lone = r.kind == BS_KIND_MINORS && r.prec != BS_PREC_FP32;  // (minors never come in batches)
-        for (int fill : {lone ? BS_TARGET_TASKS_FILL_ONE : BS_TARGET_TASKS_FILL, BS_TARGET_TASKS_FILL}) {
-            r.log2L = bs_choose_log2L_single(in.p->C, r.cpt, c->log2max[r.prec],
-                                             r.prec == BS_PREC_FP32 ? BS_TARGET_TASKS_SINGLE_FP32 : BS_TARGET_TASKS_SINGLE,
-                                             fill);
-            const uint64_t per = (uint64_t)r.cpt << r.log2L;
-            r.ntasks = (uint32_t)((in.p->C + per - 1) / per);
-            // (the longer chunks again where a budget would not hold the partials)
+        const bs_cut cut = bs_cut_single(in.p->C, r.kind, r.prec, r.cpt, c->log2max[r.prec]);
+        r.log2L = cut.log2L;
+        for (int tight : {0, 1}) {
+            r.walk = tight ? cut.group : 0;
+            r.fold = cut.group - r.walk;
+            r.ntasks = bs_cut_tasks(in.p->C, r.cpt, cut, tight);
+            // (a slot per group where a budget would not hold one per task)
             if (!c->budget || c->used - c->partials.n + (size_t)r.ntasks * r.ncols * sizeof(bs_zdd) + (1u << 20) <= c->budget)
                 break;
         }
@@ -390,6 +389,8 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
             jb.nbin = p.nbin;
             jb.kind = r.kind;
             jb.log2L = r.log2L;
+            jb.walk_log2 = r.walk;
+            jb.fold_log2 = r.fold;
             jb.out_index = r.in.out_index;
             jb.n = p.n;
             jb.prec = r.prec;
@@ -446,8 +447,10 @@ int plan_upload(bs_ctx* c, std::vector<JobIn>& ins, bs_mode mode, Prepared& P) {
         G.prec = rows[g.first].prec;
         G.kind = rows[g.first].kind;
         G.kmax = 0;
+        G.groups = 0;
         G.tasks = 0;
         for (size_t i = g.first; i < g.second; ++i) {
+            G.groups |= rows[i].walk > 0;
             G.tasks += rows[i].ntasks;
             G.kmax = std::max(G.kmax, rows[i].in.p->K);
         }
@@ -489,6 +492,7 @@ int enqueue_device(bs_ctx* c, const Prepared& P, const double2* d_src, double2* 
         w.status = reinterpret_cast<int*>(ctl + kCtlStatus);
         w.deadline_rel_ns = c->deadline_s > 0 ? (unsigned long long)(c->deadline_s * 1e9) : 0ull;
         w.max_K = g.kmax;
+        w.groups = g.groups;
         if ((rc = launch_walk(c, w, g.prec, g.kind))) return rc;
     }
     {
@@ -781,6 +785,7 @@ int enqueue_sampler_batch(bs_ctx* c, const bs::CcArgs& a, const bs::CcArgs* da, 
                 w.status = reinterpret_cast<int*>(ctl + kCtlStatus);
                 w.deadline_rel_ns = c->deadline_s > 0 ? (unsigned long long)(c->deadline_s * 1e9) : 0ull;
                 w.max_K = k;
+                w.groups = a.tight;
                 if ((rc = launch_walk(c, w, prec, BS_KIND_MINORS))) return rc;
                 c->stats.kernel_launches--;  // the caller counts every kernel
                 ++*kernels;
@@ -821,8 +826,8 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
         return BS_OK;
     }
     // worst-case tasks of one chain at the last step (C <= 2^(n-2)), over
-    // the kernels a chain may be given (bs_choose_log2L gives at most
-    // 2 x target tasks unless the chunk length is capped, and then at most
+    // the kernels a chain may be given (bs_cut_many gives at most 2 x target
+    // slots unless the chunk length is capped, and then at most
     // C / (cpt 2^log2max) + 1; cpt >= 16 for FP64 minors, 8 for FP32, 4 for DF)
     // a step-k job has <= k - 1 digit rows, K = k <= n columns, n' = k - 1;
     // a chain's data slot fits the widest row stride (DF: multiples of 8)
@@ -848,10 +853,9 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
         size_t free_b = c->budget > c->used ? c->budget - c->used : 0;
         cap_bytes = std::min(cap_bytes, free_b / 2 + c->cc_partials.n);
     }
-    // few chains: more tasks per job, where their partials fit in one pass
-    int target = bs_target_chains(n_samples);
-    if (chain_bytes(stride_for(target)) * (size_t)n_samples > cap_bytes) target = BS_TARGET_TASKS_MANY;
-    const uint64_t tasks_stride = stride_for(target);
+    // a slot per task, where they fit in one pass, or one per group
+    const int tight = chain_bytes(stride_for(BS_TARGET_TASKS_FINE)) * (size_t)n_samples > cap_bytes;
+    const uint64_t tasks_stride = stride_for(tight ? BS_TARGET_TASKS_MANY : BS_TARGET_TASKS_FINE);
     const size_t per_chain = chain_bytes(tasks_stride);
     int S_max = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_samples, cap_bytes / per_chain));
     int rc;
@@ -910,7 +914,7 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
         a.log2max64 = c->log2max[BS_PREC_FP64];
         a.log2max32 = c->log2max[BS_PREC_FP32];
         a.log2maxdf = c->log2max[BS_PREC_DF];
-        a.target = target;
+        a.tight = tight;
         a.mixed_log2_tol = c->mixed_log2_tol;
         a.mixed_fallback = kMixedFallback;
         // the kernels read the arguments from device memory (pageable copy:
@@ -933,7 +937,7 @@ int sample_dev(bs_ctx* c, const double2* dU, int m_rows, int m_cols, int ld, con
         const uint64_t dl = c->deadline_s > 0 ? (uint64_t)(c->deadline_s * 1e9) : 0;
         std::vector<uint64_t> key = {(uint64_t)a.S, (uint64_t)n, (uint64_t)m_rows, (uint64_t)m_det, (uint64_t)ld,
                                      (uint64_t)a.mode, (uint64_t)a.log2max64, (uint64_t)a.log2max32,
-                                     (uint64_t)a.log2maxdf,
+                                     (uint64_t)a.log2maxdf, (uint64_t)a.tight,
                                      (uint64_t)(uintptr_t)dU, (uint64_t)(uintptr_t)c->cc_cols.p,
                                      (uint64_t)(uintptr_t)c->cc_rows.p, (uint64_t)(uintptr_t)c->cc_jobs.p,
                                      (uint64_t)(uintptr_t)c->cc_meta.p, (uint64_t)(uintptr_t)c->cc_data.p,
@@ -1585,11 +1589,9 @@ int bs_debug_plan(int rows, int cols, const int* row_mult, const int* col_mult, 
     // chunking of this job planned alone in FP64 mode (default maximum 2^12)
     const int kd = kind == 1 ? BS_KIND_MINORS : BS_KIND_PERM;
     const int cpt = bs_chunks_per_task(kd, 0, p.K);
-    const int l = p.trivial ? 0 : bs_choose_log2L_single(p.C, cpt, bs_default_log2max(BS_PREC_FP64), BS_TARGET_TASKS_SINGLE,
-                                                         kd == BS_KIND_MINORS ? BS_TARGET_TASKS_FILL_ONE : BS_TARGET_TASKS_FILL);
-    const uint64_t per = (uint64_t)cpt << l;
-    info[6] = l;
-    info[7] = p.trivial ? 0 : (int64_t)((p.C + per - 1) / per);
+    const bs_cut cut = p.trivial ? bs_cut{0, 0} : bs_cut_single(p.C, kd, BS_PREC_FP64, cpt, bs_default_log2max(BS_PREC_FP64));
+    info[6] = cut.log2L;
+    info[7] = p.trivial ? 0 : (int64_t)bs_cut_tasks(p.C, cpt, cut, 0);
     return BS_OK;
 }
 

@@ -47,9 +47,13 @@ struct bs_job {
     int32_t src_ld;        // source leading dimension (complex elements)
     int32_t src_trans;     // 1: formula row r / column c read source (c, r)
     int32_t formula;       // BS_JOB_BBFG (0), BS_JOB_RYSER or BS_JOB_NW (plain permanents, FP64)
+    int32_t walk_log2;     // a warp task walks 2^walk_log2 consecutive tasks of the cut, summed in one slot
+    int32_t fold_log2;     // the reduce kernel adds 2^fold_log2 consecutive slots first (bs_cut)
     int32_t reseed_log2;   // FP32 jobs: > 0 re-seeds the column sums from the matrix every 2^reseed_log2
                            // steps inside a chunk as well (0: at chunk starts only)
 };
+
+#define BS_MAX_GROUP 8  // most tasks of a group (2^walk_log2, 2^fold_log2)
 
 // Formula of a job (see bs_perm_formula).  Ryser and Nijenhuis-Wilf jobs
 // walk the columns of the matrix as binary digits with the rows as product

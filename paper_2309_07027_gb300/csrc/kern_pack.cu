@@ -36,15 +36,6 @@ cudaError_t launch_pack(const bs_job* jobs, int njobs, const double2* src, int* 
 
 constexpr int kReduceBlock = 256;
 
-// One Sum2 step: (s, c) + (hi, lo) -> (s', c + e + lo) with s' + e = s + hi
-// exactly (TwoSum, Knuth).
-__device__ __forceinline__ ddv sum2_add(ddv a, double hi, double lo) {
-    const double s = __dadd_rn(a.hi, hi);
-    const double bb = __dsub_rn(s, a.hi);
-    const double e = __dadd_rn(__dsub_rn(a.hi, __dsub_rn(s, bb)), __dsub_rn(hi, bb));
-    return ddv{s, __dadd_rn(a.lo, __dadd_rn(e, lo))};
-}
-
 // (s, c) -> normalised double-double (TwoSum of s and c: c may exceed s when
 // the sum cancels).
 __device__ __forceinline__ ddv sum2_final(ddv a) {
@@ -77,13 +68,16 @@ __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __re
     const int ncols = minors ? K : 1;
     const int col = blockIdx.y;
     if (col >= ncols) return;
-    const uint32_t ntasks = jb.ntasks;
+    const uint32_t ntasks = jb.ntasks, ngroups = (ntasks + (1u << jb.fold_log2) - 1u) >> jb.fold_log2;
     const int lane = threadIdx.x & 31;
-    if (ntasks <= 32u && threadIdx.x >= 32) return;
+    if (ngroups <= 32u && threadIdx.x >= 32) return;
     const bs_zdd* p = partials + jb.partial_off + col;
     ddv re = {0.0, 0.0}, im = {0.0, 0.0};  // (s, c)
-    for (uint32_t t = threadIdx.x; t < ntasks; t += kReduceBlock) {
-        const bs_zdd v = p[(int64_t)t * ncols];
+    for (uint32_t t = threadIdx.x; t < ngroups; t += kReduceBlock) {
+        bs_zdd v = p[(int64_t)(t << jb.fold_log2) * ncols];
+        // a group's slots first, as a warp that walks a whole group sums them
+        const uint32_t end = min((t + 1) << jb.fold_log2, ntasks);
+        for (uint32_t i = (t << jb.fold_log2) + 1; i < end; ++i) v = sum2_add(v, p[(int64_t)i * ncols]);
         re = sum2_add(re, v.re_hi, v.re_lo);
         im = sum2_add(im, v.im_hi, v.im_lo);
     }
@@ -99,12 +93,12 @@ __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __re
         e = __reduce_add_sync(0xffffffffu, e);
         bad = (int)__reduce_or_sync(0xffffffffu, (unsigned)bad);
     }
-    if (ntasks > 32u) {
+    if (ngroups > 32u) {
         sre[threadIdx.x] = re;
         sim[threadIdx.x] = im;
         __syncthreads();
         int w = kReduceBlock / 2;
-        while (w >= (int)ntasks) w >>= 1;  // the upper half holds zeros
+        while (w >= (int)ngroups) w >>= 1;  // the upper half holds zeros
         for (; w >= 32; w >>= 1) {
             if ((int)threadIdx.x < w) {
                 const ddv r2 = sre[threadIdx.x + w], i2 = sim[threadIdx.x + w];
@@ -116,7 +110,7 @@ __global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const bs_job* __re
         if (threadIdx.x >= 32) return;
     }
     for (int off = 16; off > 0; off >>= 1) {
-        if (off >= (int)ntasks) continue;
+        if (off >= (int)ngroups) continue;
         const ddv r2 = shfl_down_dd(re, off), i2 = shfl_down_dd(im, off);
         re = sum2_add(re, r2.hi, r2.lo);
         im = sum2_add(im, i2.hi, i2.lo);

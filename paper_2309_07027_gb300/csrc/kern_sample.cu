@@ -170,9 +170,11 @@ __device__ int plan_minors_step(const int* __restrict__ rows, const int* __restr
     for (int c = 0; c < k; ++c) meta[2 * nrows + c] = cols[c];
     meta[2 * nrows + 2 * k] = urow[p];
     jb.C = C;
-    jb.log2L = bs_choose_log2L(C, cpt, BS_LOG2L_MIN_MANY, rule.log2max[prec],
-                              prec == BS_PREC_FP32 ? BS_TARGET_TASKS_MANY : rule.target);
-    jb.ntasks = (uint32_t)((C + ((uint64_t)cpt << jb.log2L) - 1) / ((uint64_t)cpt << jb.log2L));
+    const bs_cut cut = bs_cut_many(C, prec, cpt, rule.log2max[prec]);
+    jb.log2L = cut.log2L;
+    jb.walk_log2 = rule.tight ? cut.group : 0;
+    jb.fold_log2 = cut.group - jb.walk_log2;
+    jb.ntasks = bs_cut_tasks(C, cpt, cut, rule.tight);
     jb.task_begin = 0;
     return prec;
 }
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(kPackBlock) cc_plan_kernel(const CcArgs* __res
         jb.src_off = 0;
         jb.src_ld = a.ld;
         const StepRule rule = {a.mode, a.mixed_log2_tol, a.mixed_fallback, {a.log2max64, a.log2max32, a.log2maxdf},
-                               a.target};
+                               a.tight};
         const int prec = plan_minors_step(a.rows + (size_t)s * a.n, a.cols + (size_t)s * a.n, k, rule, jb,
                                           a.meta + jb.meta_off, urow, ucnt, drad, dsrc, q_work);
         // the chain's data slot holds data_stride complex doubles; an FP32

@@ -25,7 +25,8 @@ struct DfMinorsMinBlocks {
 #endif
 };
 
-template <int KB>
+// GROUPS: tasks may be groups (walk_log2).
+template <int KB, bool GROUPS>
 __global__ void __launch_bounds__(kDfBlock, DfMinorsMinBlocks<KB>::value) walk_df_minors_kernel(WalkArgs a) {
     extern __shared__ float4 smem_df[];
     const int lane = threadIdx.x & 31;
@@ -45,8 +46,13 @@ __global__ void __launch_bounds__(kDfBlock, DfMinorsMinBlocks<KB>::value) walk_d
             if (lane == 0) atomicExch(a.status, BS_STATUS_BADJOB);
             continue;
         }
-        walk_task_minors_df<KB>(jb, a.data, a.meta + BS_META_RADIX(jb), a.partials,
-                                (uint32_t)(t - jb.task_begin) + jb.task_offset, lane, sm, stage, stride);
+        const uint32_t local = (uint32_t)(t - jb.task_begin) + jb.task_offset;
+        bs_zdd* slot = a.partials + jb.partial_off + (int64_t)local * jb.K;
+        for (uint32_t i = 0; GROUPS ? i >> jb.walk_log2 == 0 : i < 1; ++i) {
+            const uint32_t task = GROUPS ? (local << jb.walk_log2) + i : local;
+            if (GROUPS && !task_exists(jb, task, 32 / BS_DF_GROUP_KB(KB))) break;
+            walk_task_minors_df<KB>(jb, a.data, a.meta + BS_META_RADIX(jb), slot, i > 0, task, lane, sm, stage, stride);
+        }
     }
 }
 
@@ -69,13 +75,13 @@ static int persistent_grid(Kern k, int block, size_t smem, const WalkArgs& a) {
 
 template <int KB>
 static cudaError_t run_minors(const WalkArgs& a, cudaStream_t s) {
+    const auto kernel = a.groups ? walk_df_minors_kernel<KB, true> : walk_df_minors_kernel<KB, false>;
     // per owned column and thread: a float4 fold slot and a float4 staging slot
     const size_t smem = (size_t)kDfBlock * (KB / BS_DF_GROUP_KB(KB)) * 2 * sizeof(float4);
-    cudaError_t e =
-        cudaFuncSetAttribute(walk_df_minors_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int grid = persistent_grid(walk_df_minors_kernel<KB>, kDfBlock, smem, a);
-    walk_df_minors_kernel<KB><<<grid, kDfBlock, smem, s>>>(a);
+    int grid = persistent_grid(kernel, kDfBlock, smem, a);
+    kernel<<<grid, kDfBlock, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -17,7 +17,9 @@ constexpr int kMinorsBlock = 64;
 // slower at widths 26 to 30.  Two warps per task instead of one with twice
 // the chunks: a task's latency halves, which is the time of a job with fewer
 // tasks than resident warps (20 x 20: 109 -> 58 us).
-template <int KB>
+// GROUPS: tasks may be groups (walk_log2); instances of their own, as the loop
+// over a group costs 2 to 4 % in registers.
+template <int KB, bool GROUPS>
 __global__ void __launch_bounds__(kPermBlock, KB <= 32 ? 8 : 6) walk_fp64_perm_kernel(WalkArgs a) {
     __shared__ unsigned long long s_task;
     __shared__ ddv s_half[2];
@@ -39,26 +41,31 @@ __global__ void __launch_bounds__(kPermBlock, KB <= 32 ? 8 : 6) walk_fp64_perm_k
         const bool ok = ((jb.K + 3) >> 2) == KB / 4 && jb.kind == BS_KIND_PERM;
         const uint32_t local = (uint32_t)(t - jb.task_begin) + jb.task_offset;
         const int* radix = a.meta + BS_META_RADIX(jb);
-        ddv re = {0.0, 0.0}, im = {0.0, 0.0};
-        if (!ok) {
-            if (threadIdx.x == 0) atomicExch(a.status, BS_STATUS_BADJOB);
-        } else if (radix[BS_META_SPLIT(jb) - jb.meta_off] != 0) {
-            if (((jb.K + 1) >> 1) == KB / 2)
-                walk_task_perm_dbl<KB, KB / 2>(jb, data, radix, local, warp, lane, re, im);
-            else
-                walk_task_perm_dbl<KB, KB / 2 - 1>(jb, data, radix, local, warp, lane, re, im);
-        } else if (((jb.K + 1) >> 1) == KB / 2) {  // the instance whose lanes own exactly ceil(K / 2) columns
-            walk_task_perm_fix<KB, KB / 2>(jb, data, radix, local, warp, lane, re, im);
-        } else {
-            walk_task_perm_fix<KB, KB / 2 - 1>(jb, data, radix, local, warp, lane, re, im);
+        if (!ok && threadIdx.x == 0) atomicExch(a.status, BS_STATUS_BADJOB);
+        for (uint32_t i = 0; GROUPS ? i >> jb.walk_log2 == 0 : i < 1; ++i) {
+            const uint32_t task = GROUPS ? (local << jb.walk_log2) + i : local;
+            if (!ok || (GROUPS && !task_exists(jb, task, 32))) break;
+            ddv re = {0.0, 0.0}, im = {0.0, 0.0};
+            if (radix[BS_META_SPLIT(jb) - jb.meta_off] != 0) {
+                if (((jb.K + 1) >> 1) == KB / 2)
+                    walk_task_perm_dbl<KB, KB / 2>(jb, data, radix, task, warp, lane, re, im);
+                else
+                    walk_task_perm_dbl<KB, KB / 2 - 1>(jb, data, radix, task, warp, lane, re, im);
+            } else if (((jb.K + 1) >> 1) == KB / 2) {  // the instance whose lanes own exactly ceil(K / 2) columns
+                walk_task_perm_fix<KB, KB / 2>(jb, data, radix, task, warp, lane, re, im);
+            } else {
+                walk_task_perm_fix<KB, KB / 2 - 1>(jb, data, radix, task, warp, lane, re, im);
+            }
+            if (threadIdx.x == 32) {
+                s_half[0] = re;
+                s_half[1] = im;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0)
+                store_partial(a.partials + jb.partial_off + local, dd_add_sum2(re, s_half[0]), dd_add_sum2(im, s_half[1]), i > 0);
+            if (GROUPS) __syncthreads();  // (s_half is written again)
         }
-        if (threadIdx.x == 32) {
-            s_half[0] = re;
-            s_half[1] = im;
-        }
-        __syncthreads();
-        if (ok && threadIdx.x == 0)
-            store_partial(a.partials + jb.partial_off + local, dd_add_sum2(re, s_half[0]), dd_add_sum2(im, s_half[1]));
+        if (GROUPS || !ok) __syncthreads();  // (s_task as well)
     }
 }
 
@@ -70,7 +77,7 @@ struct MinorsMinBlocks {
     static constexpr int value = KB <= 4 ? 14 : KB <= 8 ? 10 : KB <= 12 ? 8 : 6;
 };
 
-template <int KB>
+template <int KB, bool GROUPS>
 __global__ void __launch_bounds__(kMinorsBlock, MinorsMinBlocks<KB>::value) walk_fp64_minors_kernel(WalkArgs a) {
     constexpr int G = BS_MINORS_FP64_GROUP_KB(KB);
     constexpr int HM = KB / G;  // most columns a lane owns
@@ -92,13 +99,18 @@ __global__ void __launch_bounds__(kMinorsBlock, MinorsMinBlocks<KB>::value) walk
         }
         const uint32_t local = (uint32_t)(t - jb.task_begin) + jb.task_offset;
         const int* radix = a.meta + BS_META_RADIX(jb);
-        // the instance whose lanes own exactly ceil(K / G) columns
-        if (G == 4 || ((jb.K + 1) >> 1) == HM)
-            walk_task_minors_fix<G, KB, HM>(jb, data, radix, a.partials, local, lane,
-                                            *reinterpret_cast<MinorsSmem<G, HM>*>(smem));
-        else
-            walk_task_minors_fix<G, KB, HM - 1>(jb, data, radix, a.partials, local, lane,
-                                                *reinterpret_cast<MinorsSmem<G, HM - 1>*>(smem));
+        bs_zdd* slot = a.partials + jb.partial_off + (int64_t)local * jb.K;
+        for (uint32_t i = 0; GROUPS ? i >> jb.walk_log2 == 0 : i < 1; ++i) {
+            const uint32_t task = GROUPS ? (local << jb.walk_log2) + i : local;
+            if (GROUPS && !task_exists(jb, task, 16)) break;
+            // the instance whose lanes own exactly ceil(K / G) columns
+            if (G == 4 || ((jb.K + 1) >> 1) == HM)
+                walk_task_minors_fix<G, KB, HM>(jb, data, radix, slot, i > 0, task, lane,
+                                                *reinterpret_cast<MinorsSmem<G, HM>*>(smem));
+            else
+                walk_task_minors_fix<G, KB, HM - 1>(jb, data, radix, slot, i > 0, task, lane,
+                                                    *reinterpret_cast<MinorsSmem<G, HM - 1>*>(smem));
+        }
     }
 }
 
@@ -121,8 +133,9 @@ static int persistent_grid(Kern k, int block, size_t smem, int threads_per_task,
 
 template <int KB>
 static cudaError_t run_perm(const WalkArgs& a, cudaStream_t s) {
-    int grid = persistent_grid(walk_fp64_perm_kernel<KB>, kPermBlock, 0, kPermBlock, a);
-    walk_fp64_perm_kernel<KB><<<grid, kPermBlock, 0, s>>>(a);
+    const auto kernel = a.groups ? walk_fp64_perm_kernel<KB, true> : walk_fp64_perm_kernel<KB, false>;
+    int grid = persistent_grid(kernel, kPermBlock, 0, kPermBlock, a);
+    kernel<<<grid, kPermBlock, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -130,11 +143,11 @@ template <int KB>
 static cudaError_t run_minors(const WalkArgs& a, cudaStream_t s) {
     constexpr int G = BS_MINORS_FP64_GROUP_KB(KB);
     const size_t smem = (kMinorsBlock / 32) * sizeof(MinorsSmem<G, KB / G>);
-    cudaError_t e =
-        cudaFuncSetAttribute(walk_fp64_minors_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = a.groups ? walk_fp64_minors_kernel<KB, true> : walk_fp64_minors_kernel<KB, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int grid = persistent_grid(walk_fp64_minors_kernel<KB>, kMinorsBlock, smem, 32, a);
-    walk_fp64_minors_kernel<KB><<<grid, kMinorsBlock, smem, s>>>(a);
+    int grid = persistent_grid(kernel, kMinorsBlock, smem, 32, a);
+    kernel<<<grid, kMinorsBlock, smem, s>>>(a);
     return cudaGetLastError();
 }
 

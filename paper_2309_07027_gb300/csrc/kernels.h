@@ -20,6 +20,7 @@ struct WalkArgsBase {
     int* status;                           // device status word
     unsigned long long deadline_rel_ns;    // per-warp deadline after its start, 0 = none
     int max_K;                             // bucket: every job has (K+3)/4 == (max_K+3)/4
+    int groups;                            // 1: jobs may have walk_log2 > 0 (FP64 and double-float)
     int grid_cap;                          // upper bound on CTAs (0 = fill the GPU)
 };
 typedef WalkArgsBase WalkArgs;

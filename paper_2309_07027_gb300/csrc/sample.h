@@ -24,16 +24,18 @@
 // about half the rows (4096-item batch: 3.6 % faster than with 32768).
 #define BS_TARGET_TASKS_SINGLE_FP32 8192
 #define BS_TARGET_TASKS_MANY 64
-// FP64 and double-float jobs of a sampler call with few chains aim at more
-// tasks, so that the call fills the GPU (about 8192 tasks in all, several per
-// resident warp): 40 chains at 64 tasks each are 1.4 tasks per resident warp,
-// and a call of one chain leaves 9 of 10 schedulers idle.  Served jobs, which
-// know nothing of their company, aim at 512.  Neither form drifts inside a
-// chunk (exact column sums), so shorter chunks cost only their seeding.  FP32
-// jobs keep 64: their chunk length is part of the MIXED rule.
-#define BS_TARGET_TASKS_ALL 8192
-#define BS_TARGET_TASKS_MAX 1024
-#define BS_TARGET_TASKS_SERVED 512
+// FP64 and double-float jobs of the sampler and the server aim at more tasks:
+// 64 per job are 1.4 per resident warp for 40 chains, and a crowded tick's
+// steps are as long as their largest tasks.  Neither form drifts inside a chunk
+// (exact column sums), so shorter chunks cost only their seeding, down to 2^4
+// addends (FP64) and 2^5 (double-float).  Against 64 for all: 48 served chains
+// 26 -> 14 ms, 40 samples of 30 photons 350 -> 334 ms, 25 double-float samples
+// of 26 photons 29 -> 21 ms.  The lower ends trade many chains against few:
+// 300 (8) samples of 20 photons 8.5 (1.45) ms, with 2^3 9.1 (1.39), with 2^6
+// 8.4 (1.63); in double-float 8.25 (1.42), 9.0 (1.37) with 2^4, 8.1 (1.62)
+// with 2^7.  FP32 jobs keep 64: their chunk length is part of the MIXED rule.
+#define BS_TARGET_TASKS_FINE 512
+#define BS_LOG2L_MIN_FINE(prec) ((prec) == BS_PREC_FP64 ? 4 : 5)
 #define BS_LOG2L_MIN_SINGLE 6
 #define BS_LOG2L_MIN_MANY 3
 // Floor for the tiniest jobs planned alone (at most BS_FILL_TINY_C
@@ -69,12 +71,6 @@ BS_HD int bs_choose_log2L(uint64_t C, int cpt, int log2min, int log2max, int tar
     if (l > log2max) l = log2max;
     return l;
 }
-// Task target of an FP64 or double-float job in a sampler call of S chains.
-BS_HD int bs_target_chains(int64_t S) {
-    int t = BS_TARGET_TASKS_MANY;
-    while (t < BS_TARGET_TASKS_MAX && (int64_t)t * S < BS_TARGET_TASKS_ALL) t *= 2;
-    return t;
-}
 // The rule for jobs planned one call at a time: bs_choose_log2L with the
 // single-call target and floor 2^6, except that a job too small to give
 // BS_TARGET_TASKS_FILL tasks at that floor gets shorter chunks (down to 2^3,
@@ -99,6 +95,41 @@ BS_HD int bs_choose_log2L_single(uint64_t C, int cpt, int log2max, int target, i
     const int floor = C <= BS_FILL_TINY_C ? BS_LOG2L_MIN_FILL : BS_LOG2L_MIN_MANY;
     if (fill < floor) fill = floor;
     return fill > log2max ? log2max : fill;
+}
+
+// The cut of a job into tasks of chunks of 2^log2L addends, and the order in
+// which its partials are summed: 2^group consecutive tasks first, then those
+// sums.  Both depend on the job alone.  Where memory is short, one warp walks a
+// group and sums it by itself (walk_log2 = group, a slot per group); otherwise
+// the reduce kernel does (fold_log2 = group, a slot per task).  The additions are the same, and so
+// are the bits of the result, whatever the budget, the number of chains and
+// the company.
+struct bs_cut {
+    int log2L, group;
+};
+static_assert(BS_TARGET_TASKS_FINE / BS_TARGET_TASKS_MANY <= BS_MAX_GROUP &&
+                  BS_TARGET_TASKS_FILL_ONE / BS_TARGET_TASKS_FILL <= BS_MAX_GROUP,
+              "the finer targets bound the groups");
+// Jobs of the sampler and the server.
+BS_HD bs_cut bs_cut_many(uint64_t C, int prec, int cpt, int log2max) {
+    const int lc = bs_choose_log2L(C, cpt, BS_LOG2L_MIN_MANY, log2max, BS_TARGET_TASKS_MANY);
+    if (prec == BS_PREC_FP32) return bs_cut{lc, 0};
+    int lf = bs_choose_log2L(C, cpt, BS_LOG2L_MIN_FINE(prec), log2max, BS_TARGET_TASKS_FINE);
+    if (lf > lc) lf = lc;
+    return bs_cut{lf, lc - lf};
+}
+// Jobs planned one call at a time.
+BS_HD bs_cut bs_cut_single(uint64_t C, int kind, int prec, int cpt, int log2max) {
+    const int target = prec == BS_PREC_FP32 ? BS_TARGET_TASKS_SINGLE_FP32 : BS_TARGET_TASKS_SINGLE;
+    const int lc = bs_choose_log2L_single(C, cpt, log2max, target);
+    if (prec == BS_PREC_FP32 || kind != BS_KIND_MINORS) return bs_cut{lc, 0};
+    const int lf = bs_choose_log2L_single(C, cpt, log2max, target, BS_TARGET_TASKS_FILL_ONE);
+    return bs_cut{lf, lc - lf};
+}
+// Walk tasks (and slots) of the cut; tight: a warp per group.
+BS_HD uint32_t bs_cut_tasks(uint64_t C, int cpt, bs_cut cut, int tight) {
+    const uint64_t per = (uint64_t)cpt << (cut.log2L + (tight ? cut.group : 0));
+    return (uint32_t)((C + per - 1) / per);
 }
 
 // Lanes that walk one chunk together in the FP32 fused-minor kernel (each
@@ -270,7 +301,7 @@ struct StepRule {
     float mixed_log2_tol;
     int mixed_fallback;
     int log2max[BS_NPREC];
-    int target;  // task target of FP64 and double-float jobs
+    int tight;  // a warp per group of tasks (bs_cut)
 };
 
 struct CcArgs {
@@ -300,7 +331,7 @@ struct CcArgs {
     float mixed_log2_tol;         // the rule's threshold, log2 of the MIXED tolerance
     int mixed_fallback;           // MIXED: precision of the jobs that fail the rule
     int log2max64, log2max32, log2maxdf;
-    int target;                   // task target of FP64 and double-float jobs
+    int tight;                    // a warp per group of tasks (bs_cut)
 };
 
 // One served Clifford & Clifford chain (one sample) resident in a server's

@@ -126,7 +126,8 @@ struct Request {
     std::vector<int> counts;           // result: m_det occupation counts
     bs_job job_host{};                 // the pending step's job, as planned on the device
     uint64_t tasks_stride = 0;         // task partial slots per step
-    int target = BS_TARGET_TASKS_MANY; // task target of its FP64 and double-float steps
+    int tight = 0;                     // a warp and a slot per group of tasks (bs_cut)
+    int walk = 0, fold = 0;            // the job's walk_log2 and fold_log2
     // byte offsets of the chain's regions inside its arena block
     size_t c_u = 0, c_in = 0, c_cols = 0, c_rows = 0, c_meta = 0, c_data = 0, c_part = 0;
 };
@@ -215,8 +216,8 @@ size_t request_bytes(const Request& r) {
 }
 
 // Whether requests of this size could fill every slot at once: only then does
-// a request take the larger task target, so that no budget holds fewer
-// requests than it would with the smaller one.
+// a request take a slot per task, so that no budget holds fewer requests than
+// it would with one per group.
 bool fits_slot(const bs_server* s, size_t bytes) { return bytes <= s->budget / (size_t)s->max_active; }
 
 void finish(bs_server* s, Request* r, int status) {
@@ -284,6 +285,8 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
         jb.nbin = p.nbin;
         jb.kind = r->kind;
         jb.log2L = r->log2L;
+        jb.walk_log2 = r->walk;
+        jb.fold_log2 = r->fold;
         jb.n = p.n;
         jb.prec = r->prec;
         jb.reseed_log2 = r->reseed;
@@ -316,6 +319,8 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
             jb.nbin = p.nbin;
             jb.kind = r->kind;
             jb.log2L = r->log2L;
+            jb.walk_log2 = r->walk;
+            jb.fold_log2 = r->fold;
             jb.n = p.n;
             jb.prec = r->prec;
             jb.reseed_log2 = r->reseed;
@@ -323,16 +328,14 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
             jb.meta_off = r->meta_off;
             jb.partial_off = r->part_off;
         }
-        // A step cut into more tasks than BS_TARGET_TASKS_MANY has shorter ones,
-        // and as many more of them make up its share of a crowded tick (jobs at
-        // the cap of the chunk length, which have more than twice their target,
-        // keep the plain one): otherwise a middling step takes four ticks, each
-        // as long as the slices of the largest jobs (64 requests of 16 to 34
-        // photons arriving at 1000 / s, samples / s: FP64 56 -> 73, MIXED 361 -> 410,
-        // double-float 91 -> 104, where the coarse steps gave 103).
+        // A step whose tasks come in groups has shorter ones, and as many more of
+        // them make up its share of a crowded tick: otherwise a middling step
+        // takes four ticks, each as long as the slices of the largest jobs (64
+        // requests of 16 to 34 photons arriving at 1000 / s, samples / s: FP64 56
+        // -> 73, MIXED 361 -> 410, double-float 91 -> 104).
         // Few requests keep short ticks, so a cancellation is prompt.
-        const bool fine = walking > 4 && r->chain && jb.prec != BS_PREC_FP32 && r->ntasks <= 2u * (uint32_t)r->target;
-        jb.ntasks = std::min(fine ? share * (uint32_t)(r->target / BS_TARGET_TASKS_MANY) : share, r->ntasks - r->done);
+        const int more = walking > 4 && r->chain ? jb.fold_log2 : 0;
+        jb.ntasks = std::min(share << more, r->ntasks - r->done);
         jb.task_offset = r->done;
         walk.push_back(jb);
         walk_req.push_back(r);
@@ -422,7 +425,7 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
         d.rule.mixed_log2_tol = BS_MIXED_LOG2_TOL_DEFAULT;
         d.rule.mixed_fallback = BS_MIXED_FALLBACK_PREC;
         for (int q = 0; q < BS_NPREC; ++q) d.rule.log2max[q] = bs_default_log2max(q);
-        d.rule.target = r->target;
+        d.rule.tight = r->tight;
         descs.push_back(d);
         max_m_rows = std::max(max_m_rows, r->m_rows);
         back_bytes += back_of(r);
@@ -493,6 +496,7 @@ int run_tick(bs_server* s, std::vector<Request*>& admit, std::vector<Request*>& 
         for (size_t i = groups[gi].first; i < groups[gi].second; ++i) {
             tot += tick[i].ntasks;
             kmax = std::max(kmax, tick[i].K);
+            w.groups |= tick[i].walk_log2 > 0;
         }
         w.total_tasks = tot;
         w.counter = ctl + gi;  // at most 2 x 12 (FP32) + 12 + 6 (DF) = 42 groups
@@ -747,10 +751,12 @@ int64_t bs_server_submit(bs_server* s, int kind, const bs_c128* A, int rows, int
     }
     r->cpt = bs_chunks_per_task(r->kind, r->prec, r->plan.K);
     r->ncols = r->kind == BS_KIND_PERM ? 1 : r->plan.K;
-    for (int target : {r->prec == BS_PREC_FP32 ? BS_TARGET_TASKS_MANY : BS_TARGET_TASKS_SERVED, BS_TARGET_TASKS_MANY}) {
-        r->log2L = bs_choose_log2L(r->plan.C, r->cpt, BS_LOG2L_MIN_MANY, bs_default_log2max(r->prec), target);
-        const uint64_t per = (uint64_t)r->cpt << r->log2L;
-        r->ntasks = (uint32_t)((r->plan.C + per - 1) / per);
+    const bs_cut cut = bs_cut_many(r->plan.C, r->prec, r->cpt, bs_default_log2max(r->prec));
+    r->log2L = cut.log2L;
+    for (int tight : {0, 1}) {
+        r->walk = tight ? cut.group : 0;
+        r->fold = cut.group - r->walk;
+        r->ntasks = bs_cut_tasks(r->plan.C, r->cpt, cut, tight);
         r->bytes = request_bytes(*r);
         if (fits_slot(s, r->bytes)) break;
     }
@@ -849,14 +855,14 @@ int64_t bs_server_submit_sample(bs_server* s, const bs_c128* U, int m_rows, int 
         const int precs_mixed[2] = {BS_PREC_FP32, BS_MIXED_FALLBACK_PREC};
         const int prec_one = s->mode == BS_DF64 ? BS_PREC_DF : BS_PREC_FP64;
         const int np = s->mode == BS_MIXED ? 2 : 1;
-        for (int target : {BS_TARGET_TASKS_SERVED, BS_TARGET_TASKS_MANY}) {
-            uint64_t ts = 2 * (uint64_t)target + 1;
+        for (int tight : {0, 1}) {
+            uint64_t ts = 2 * (uint64_t)(tight ? BS_TARGET_TASKS_MANY : BS_TARGET_TASKS_FINE) + 1;
             for (int i = 0; i < np; ++i) {
                 const int q = s->mode == BS_MIXED ? precs_mixed[i] : prec_one;
                 const uint64_t cpt_min = q == BS_PREC_FP64 ? 16 : q == BS_PREC_FP32 ? 8 : 4;
                 ts = std::max<uint64_t>(ts, cmax / (cpt_min << bs_default_log2max(q)) + 2);
             }
-            r->target = target;
+            r->tight = tight;
             r->tasks_stride = ts;
             r->bytes = chain_layout(*r);
             if (fits_slot(s, r->bytes)) break;

@@ -25,8 +25,10 @@
 // walk_df.cuh (double-float jobs).  In each, a lane sums its addends for a
 // short run and folds the run into a compensated sum, and the lanes of a task
 // are combined in a fixed order.  Tasks write one partial per output; the
-// reduce kernel sums them in a fixed order, so results do not depend on which
-// warp ran which task or on what else was in the launch.
+// reduce kernel sums them in a fixed order.  The cut into tasks and that order
+// are functions of the job (bs_cut in sample.h), so results do not depend on
+// which warp ran which task, on what else was in the launch or on the memory
+// at hand.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -230,6 +232,26 @@ __device__ __forceinline__ T signed_weight(uint64_t w, int parity) {
     return parity ? -x : x;
 }
 
+// One Sum2 step: (s, c) + (hi, lo) -> (s', c + e + lo) with s' + e = s + hi
+// exactly (TwoSum, Knuth).
+__device__ __forceinline__ ddv sum2_add(ddv a, double hi, double lo) {
+    const double s = __dadd_rn(a.hi, hi);
+    const double bb = __dsub_rn(s, a.hi);
+    const double e = __dadd_rn(__dsub_rn(a.hi, __dsub_rn(s, bb)), __dsub_rn(hi, bb));
+    return ddv{s, __dadd_rn(a.lo, __dadd_rn(e, lo))};
+}
+
+__device__ __forceinline__ bs_zdd sum2_add(const bs_zdd& a, const bs_zdd& b) {
+    const ddv re = sum2_add(ddv{a.re_hi, a.re_lo}, b.re_hi, b.re_lo), im = sum2_add(ddv{a.im_hi, a.im_lo}, b.im_hi, b.im_lo);
+    return bs_zdd{re.hi, re.lo, im.hi, im.lo};
+}
+
+// A task's partial into its slot; `more`: it joins those of its group before it.
+__device__ __forceinline__ void store_partial(bs_zdd* p, ddv re, ddv im, bool more) {
+    const bs_zdd v = {re.hi, re.lo, im.hi, im.lo};
+    *p = more ? sum2_add(*p, v) : v;
+}
+
 __device__ __forceinline__ void store_partial(bs_zdd* p, ddv re, ddv im) {
     bs_zdd o;
     o.re_hi = re.hi;
@@ -278,6 +300,11 @@ __device__ __forceinline__ unsigned long long next_task(unsigned long long* coun
         }
     }
     return __shfl_sync(0xffffffffu, t, 0);
+}
+
+// Whether the cut's task `local` of chunks_per_task chunks has any addends.
+__device__ __forceinline__ bool task_exists(const bs_job& jb, uint32_t local, uint32_t chunks_per_task) {
+    return (uint64_t)local * chunks_per_task << jb.log2L < jb.C;
 }
 
 // Per-warp absolute deadline from a relative one (0 = none).

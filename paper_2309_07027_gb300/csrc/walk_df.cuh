@@ -351,8 +351,8 @@ __device__ __forceinline__ void df_fold(float4* __restrict__ sm, float4* __restr
 // warp.
 template <int KB>
 __device__ void walk_task_minors_df(const bs_job& jb, const void* __restrict__ data_v,
-                                    const int* __restrict__ radix, bs_zdd* __restrict__ partials, uint32_t local,
-                                    int lane, float4* __restrict__ sm, float4* __restrict__ stage, int stride) {
+                                    const int* __restrict__ radix, bs_zdd* __restrict__ slot, bool more,
+                                    uint32_t local, int lane, float4* __restrict__ sm, float4* __restrict__ stage, int stride) {
     constexpr uint32_t FOLD = 64;
     constexpr int G = BS_DF_GROUP_KB(KB);
     constexpr int NP = KB / (2 * G);
@@ -455,8 +455,7 @@ __device__ void walk_task_minors_df(const bs_job& jb, const void* __restrict__ d
             im = s_add(im, shfl_down_dfs(im, off));
         }
         if (lane < G && t < KH)
-            store_partial(partials + jb.partial_off + (int64_t)local * K + cbase + t, dd_from_dfs(re),
-                          dd_from_dfs(im));
+            store_partial(slot + cbase + t, dd_from_dfs(re), dd_from_dfs(im), more);
     }
 }
 

@@ -819,7 +819,7 @@ __device__ __noinline__ void walk_task_minors_dbl(const bs_job& jb, const zfix* 
 // cycles beside them, so what bounds it is the instruction count.
 template <int G, int KB, int HX>
 __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ data, const int* __restrict__ radix,
-                                     bs_zdd* __restrict__ partials, uint32_t local, int lane,
+                                     bs_zdd* __restrict__ slot, bool more, uint32_t local, int lane,
                                      MinorsSmem<G, HX>& sm) {
     constexpr int KP = KB;            // = BS_ROW_STRIDE(K) for every K of the bucket
     constexpr int NP = (HX + 1) / 2;  // leaves, in two chains of NA and NB
@@ -965,7 +965,7 @@ __device__ void walk_task_minors_fix(const bs_job& jb, const zfix* __restrict__ 
     if (__any_sync(0xffffffffu, dbl)) walk_task_minors_dbl<G, KB, HX>(jb, data, radix, local, lane, sm);
     for (int t = lane; t < K; t += 32) {
         const double4 v = sm.tot[t];
-        store_partial(partials + jb.partial_off + (int64_t)local * K + t, ddv{v.x, v.y}, ddv{v.z, v.w});
+        store_partial(slot + t, ddv{v.x, v.y}, ddv{v.z, v.w}, more);
     }
     __syncwarp();  // the next task's initialisation overwrites the totals
 }
