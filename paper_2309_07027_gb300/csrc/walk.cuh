@@ -141,18 +141,6 @@ __device__ __forceinline__ ddv shfl_down_dd(ddv v, int off) {
     return r;
 }
 
-// Fixed-order warp reduction of a double-double complex value; lane 0 ends
-// with the sum.
-__device__ __forceinline__ void warp_reduce_zdd(ddv& re, ddv& im) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        ddv ore = shfl_down_dd(re, off);
-        ddv oim = shfl_down_dd(im, off);
-        re = dd_add_sum2(re, ore);
-        im = dd_add_sum2(im, oim);
-    }
-}
-
 __device__ __forceinline__ double flip_sign(double x) {
     return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
 }
