@@ -53,7 +53,7 @@ struct bs_job {
                            // steps inside a chunk as well (0: at chunk starts only)
 };
 
-#define BS_MAX_GROUP 8  // most tasks of a group (2^walk_log2, 2^fold_log2)
+#define BS_MAX_GROUP 16  // most tasks of a group (2^walk_log2, 2^fold_log2)
 
 // Formula of a job (see bs_perm_formula).  Ryser and Nijenhuis-Wilf jobs
 // walk the columns of the matrix as binary digits with the rows as product
@@ -104,7 +104,7 @@ struct bs_job {
 // than products on the FP32 pipe were (calls: 12 x 12 98 -> 55 us, 20 x 20
 // 160 -> 105, 24 x 24 645 -> 480, 26 x 26 2.63 -> 1.80 ms, 30 x 30 34.8 -> 28.9
 // ms).  Only double-float minors have kernels of their own: at 30 columns they
-// take 38.7 ms where the fixed point takes 45.2.
+// take 38.7 ms where the fixed point takes 49.0.
 #define BS_DF_MINORS(prec, kind) ((prec) == BS_PREC_DF && (kind) == BS_KIND_MINORS)
 
 // Task partials of the fixed-point kernels are in units of 2^-BS_FIX_BIAS of the

@@ -25,16 +25,18 @@
 #define BS_TARGET_TASKS_SINGLE_FP32 8192
 #define BS_TARGET_TASKS_MANY 64
 // FP64 and double-float jobs of the sampler and the server aim at more tasks:
-// 64 per job are 1.4 per resident warp for 40 chains, and a crowded tick's
-// steps are as long as their largest tasks.  Neither form drifts inside a chunk
-// (exact column sums), so shorter chunks cost only their seeding, down to 2^4
-// addends (FP64) and 2^5 (double-float).  Against 64 for all: 48 served chains
-// 26 -> 14 ms, 40 samples of 30 photons 350 -> 334 ms, 25 double-float samples
-// of 26 photons 29 -> 21 ms.  The lower ends trade many chains against few:
-// 300 (8) samples of 20 photons 8.5 (1.45) ms, with 2^3 9.1 (1.39), with 2^6
-// 8.4 (1.63); in double-float 8.25 (1.42), 9.0 (1.37) with 2^4, 8.1 (1.62)
-// with 2^7.  FP32 jobs keep 64: their chunk length is part of the MIXED rule.
-#define BS_TARGET_TASKS_FINE 512
+// 64 per job are 1.4 per resident warp for 40 chains and leave most of the GPU
+// idle for one, and a crowded tick's steps are as long as their largest tasks.
+// Neither form drifts inside a chunk (exact column sums), so shorter chunks
+// cost only their seeding, down to 2^4 addends (FP64) and 2^5 (double-float).
+// Against 64 for all: 48 served chains 26 -> 14 ms, 40 samples of 30 photons
+// 350 -> 330 ms, 25 double-float samples of 26 photons 29 -> 20 ms.  The figures
+// trade many chains against few: one sample of 30 (24) photons 6.7 (1.7) ms,
+// 100 of 24 photons 26.8 ms; at 512 tasks 11.2 (1.7) and 25.9, at 2048 5.9 (1.7)
+// and 28.0; 300 (8) samples of 20 photons 8.5 (1.46) ms, with a lower end of 2^3
+// 9.2 (1.41), of 2^6 8.4 (1.63).  FP32 jobs keep 64: their chunk length is part
+// of the MIXED rule.
+#define BS_TARGET_TASKS_FINE 1024
 #define BS_LOG2L_MIN_FINE(prec) ((prec) == BS_PREC_FP64 ? 4 : 5)
 #define BS_LOG2L_MIN_SINGLE 6
 #define BS_LOG2L_MIN_MANY 3
