@@ -8,9 +8,8 @@ hot-path stage on the GPU: per-chain planning, Gray decode / re-seed, the
 incremental column-sum walk, the per-addend products, the fused Laplace
 minors, compensated accumulation and the weighted draw.  The headline runs
 the FP64 form (``--mode fp64``: exact 63-bit column sums and 62-bit products on
-the integer pipes, whose errors are below plain double arithmetic's, weights
-in double precision, double-double partial sums); the MIXED form is reported
-beside it.
+the integer pipes, weights in double precision, double-double partial sums);
+the MIXED form is reported beside it.
 
   value     samples/s with U resident on the device (bs_sample_dev), CUDA
             events around every step, L2 flushed (256 MiB write) between steps
@@ -328,8 +327,8 @@ def aggregate_rate(world, units_per_rank, seconds):
 DTYPES = {"fp64": "f64", "mixed": "f32", "df": "f32x2"}
 DTYPE_DETAIL = {
     "fp64": ("f64 in and out; exact 63-bit fixed-point column sums and products of normalised 62-bit mantissas on "
-             "the integer pipes (errors against the exact value below those of f64 products, "
-             "tests/test_gpu_fixed_point.py), f64 weights and runs, double-double task partials (Sum2 reduce)"),
+             "the integer pipes (on Haar-random matrices errors below those of f64 products; elsewhere as "
+             "include/bs.h states: tests/test_gpu_cancellation.py, tests/test_gpu_unequal_parts.py), f64 weights and runs, double-double task partials (Sum2 reduce)"),
     "mixed": ("f32 column sums and products where the MIXED rule predicts an error below 1e-6 prod ||a_j|| "
               "(column sums re-seeded every 2^8 steps where only their drift would exceed it; the rule is "
               "oracle-checked in tests/test_gpu_widths.py), double-float otherwise; float-float runs folded into "
@@ -349,9 +348,11 @@ DTYPE_DETAIL = {
 # there is none, or where the kernel changed since the capture.
 TRAFFIC_K30 = [None, None, None]
 # The bounding pipe's busy fraction under ncu (pct of peak sustained active):
-# the FMA-heavy pipe (integer products) on a 27 x 28 minors launch for the FP64
-# kernel, the FMA pipe on the k = 30 launch for the others.
-PIPE_K30 = [{"pipe": "fmaheavy", "active": 0.67}, {"pipe": "fma", "active": 0.709}, {"pipe": "fma", "active": 0.788}]
+# the FMA-heavy pipe (integer products) for the FP64 kernel, the FMA pipe for
+# the others, and the launch it was taken on (profiles/).
+PIPE_ACTIVE = [{"pipe": "fmaheavy", "active": 0.690, "launch": "one call of 27 x 28 minors"},
+               {"pipe": "fma", "active": 0.709, "launch": "the k = 30 launch"},
+               {"pipe": "fma", "active": 0.788, "launch": "the k = 30 launch"}]
 # Flops of the algorithmic counts per 32 x 32 -> 64 bit product of the FP64
 # kernels: minors 22 K - 22 flops and 3 K - 3 complex products of 12, permanents
 # 8 K - 2 flops and K - 1 complex products.
@@ -473,7 +474,7 @@ def run_mine(args):
             "frac": achieved / peak if peak else None, "traffic": traffic,
             "traffic_launch": (f"the k = 30 launch of {S_} chains (ncu dram__bytes_read.sum + dram__bytes_write.sum)"
                                if traffic is not None else None),
-            "ncu_pipe_active_k30": PIPE_K30[p],
+            "ncu_pipe_active": PIPE_ACTIVE[p],
             "kernel": ("walk_fp64_minors_kernel", "walk_fp32_minors_kernel", "walk_df_minors_kernel")[p],
             "peak_source": ("measured on this GPU by bs_measure_wide_rate: 32 x 32 -> 64 bit integer products, "
                             "22 algorithmic flops per 36 of them" if p == 0 else
@@ -560,9 +561,14 @@ def run_mine(args):
         ops = 12 * 29 if kind == "perm" else 36 * 29
         fp64_k30[kind] = {"addends_per_s": rate,
                           "vs_fp64_fma_peak": flops / secs / (2.0 * fp64_rate),
-                          # of the peak of the pipe the FP64 jobs run on, a product counted as 2 flops
-                          "frac_of_fp64_peak": flops / secs / (2.0 * wide_rate),
                           "wide_products_per_addend": ops,
+                          # of the measured rate of wide products: the products counted, and the credited
+                          # flops at FLOPS_PER_WIDE of them
+                          "frac_of_wide_pipe": rate * ops / wide_rate,
+                          "frac_of_wide_peak": flops / secs / (FLOPS_PER_WIDE[kind] * wide_rate),
+                          # earlier lines' names, of the integer pipe since the FP64 jobs run on it (two flops
+                          # per product, and the products): not comparable with lines from double walks
+                          "frac_of_fp64_peak": flops / secs / (2.0 * wide_rate),
                           "frac_of_fp64_pipe": rate * ops / wide_rate}
         vd, secs_d, adds_d, flops_d = res[2]
         norms = np.sqrt((np.abs(a) ** 2).sum(axis=0))

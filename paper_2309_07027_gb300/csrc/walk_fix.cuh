@@ -26,6 +26,12 @@
 //     stays below 2^63 in magnitude (four terms of at most 2^61, or two of
 //     2^61 and two that add up to less than 2^62), every high sum below 2^62.
 //     Only high limbs are negated (a low limb of -2^31 has no negative).
+//   * What this loses by itself, and what is done about it: a pair of column
+//     sums is multiplied before it is normalised, so sums that cancel lose
+//     their bits against the bounds (fix_product<1> and suffix_chains<1>
+//     normalise the sums first, where it matters); both parts of a column
+//     share one scale (columns whose parts' bounds differ by more than 8 get a
+//     scale per part, and their jobs' addends are formed in double).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -328,9 +334,9 @@ __device__ __forceinline__ zlimb shfl_xor_zlimb(const zlimb& v, int mask) {
 //
 // 30 x 30 permanent (2^29 addends): 165 ms in double (FP64 pipe 94 % busy),
 // 36.2 ms with one lane per chunk (255 registers, 2 warps per scheduler), 29.1
-// ms here; 70 cycles per warp, column and addend, of which the 12 integer
-// products hold the FMA-heavy pipe 52 (72 % busy) and 25 other integer
-// instructions take the rest.  Relative error (23 x 23, Haar): 6.8e-15, in
+// ms here; 72 cycles per warp, column and addend, of which the 12 integer
+// products hold the FMA-heavy pipe 52 (78 % busy with what else runs there) and
+// 26 other integer instructions take the rest.  Relative error (23 x 23, Haar): 6.8e-15, in
 // double 2.7e-14.
 template <int KB, int HX>
 __device__ void walk_task_perm_fix(const bs_job& jb, const zfix* __restrict__ data, const int* __restrict__ radix,
@@ -810,10 +816,10 @@ __device__ __noinline__ void walk_task_minors_dbl(const bs_job& jb, const zfix* 
 // addends in double instead of suffix_chains<1>: 52.4 ms, and 10 us of latency
 // for one in a small call; the look at every run in double: 2.6 ms more.
 //
-// Time.  29 x 30 minors (2^28 addends): 190 ms in double, 48.5 ms here (1.42e9 ->
-// 5.53e9 addends/s; 45.2 without the provisions for cancelling sums, and 47.8
+// Time.  29 x 30 minors (2^28 addends): 190 ms in double, 49.0 ms here (1.42e9 ->
+// 5.48e9 addends/s; 45.2 without the provisions for cancelling sums, and 47.8
 // with runs of 4, 49.7 with the m_j of an addend kept before any is added);
-// 24 columns 0.637 ms (0.603 without, 0.670 with runs of 4).  The
+// 24 columns 0.640 ms (0.603 without, 0.670 with runs of 4).  The
 // FMA-heavy pipe is about 70 % busy with integer products (4.35 cycles per
 // warp and product) and every other integer instruction costs about 1.3
 // cycles beside them, so what bounds it is the instruction count.
